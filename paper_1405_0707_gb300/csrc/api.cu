@@ -90,7 +90,7 @@ inline bool fused_qr(const expm_plan* P, int p) {
 // the second CGS pass's correction W -= V[:, 0:cgs_cols] h, with h followed by the Gram
 // matrix of W before it (k_qr_mixed_rows<3>).
 expm_status qr_block(expm_plan* P, int p, double* out, int64_t ldo, bool withH, int hrow, int hcol,
-                     double* normsq, bool gram_done, int cgs_cols = 0) {
+                     double* normsq, bool gram_done, int cgs_cols = 0, const int* skip = nullptr) {
     cudaStream_t s = P->stream;
     const int64_t n = P->n, ld = P->ld;
     const double shift = 11.0 * ((double)n * p + (double)p * (p + 1)) * std::ldexp(1.0, -53);
@@ -122,16 +122,16 @@ expm_status qr_block(expm_plan* P, int p, double* out, int64_t ldo, bool withH, 
     const int* extra = flags + 2;
     // pass 1: unshifted Cholesky, shifted when W is ill-conditioned (sets the third-pass flag)
     LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, P->nblk, p, shift, sm(P, kOffR), sm(P, kOffRi),
-                                      sm(P, kOffRt), 0, Hq, P->ldH, hrow, hcol, normsq, flags, s));
-    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), P->W, ld, P->part, P->nblk, 1, extra, 0, s));
+                                      sm(P, kOffRt), 0, Hq, P->ldH, hrow, hcol, normsq, flags, s, skip));
+    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), P->W, ld, P->part, P->nblk, 1, extra, 0, s, skip));
     // pass 2: the last one for a well-conditioned block (writes the final block directly)
     LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, P->nblk, p, 0.0, sm(P, kOffR), sm(P, kOffRi),
-                                      sm(P, kOffRt), 1, Hq, P->ldH, hrow, hcol, nullptr, flags, s));
-    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), out, ldo, P->part, P->nblk, 1, extra, 1, s));
+                                      sm(P, kOffRt), 1, Hq, P->ldH, hrow, hcol, nullptr, flags, s, skip));
+    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), out, ldo, P->part, P->nblk, 1, extra, 1, s, skip));
     // pass 3: only when pass 1 needed the shift (no-op otherwise)
     LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, P->nblk, p, 0.0, sm(P, kOffR), sm(P, kOffRi),
-                                      sm(P, kOffRt), 2, Hq, P->ldH, hrow, hcol, nullptr, flags, s));
-    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), out, ldo, nullptr, P->nblk, 0, extra, 2, s));
+                                      sm(P, kOffRt), 2, Hq, P->ldH, hrow, hcol, nullptr, flags, s, skip));
+    LAUNCH(EXPM_STAGE_QR, launch_trsm(P->W, ld, p, n, sm(P, kOffRi), out, ldo, nullptr, P->nblk, 0, extra, 2, s, skip));
     return EXPM_OK;
 }
 
@@ -336,6 +336,55 @@ expm_status prec_apply_internal(expm_plan* P, double t, const double* V, int64_t
     return EXPM_OK;
 }
 
+// The mixed path's Gram-Schmidt and Cholesky-QR of block step j (W = Op V_j in P->W): projection,
+// update (h rounded to the digits it is applied with, the Gram matrix of the result), projection,
+// reduction and factor, the row pass; then the passes that take over when the block is too
+// ill-conditioned for the single factor (they return at once otherwise).
+expm_status ortho_mma(expm_plan* P, int j, int p) {
+    cudaStream_t s = P->stream;
+    const int64_t n = P->n, ld = P->ld;
+    const int cols = (j + 1) * p, hrow = (j + 1) * p, hcol = j * p;
+    double* h = sm(P, kOffH);
+    int* flags = flags_of(P->stat);
+    double* out = P->V + (int64_t)cols * ld;
+    float* out32 = P->V32 + (int64_t)cols * ld;
+    const int maxb = std::max(P->nblk, P->nblk_cgs);
+    int nb = 0, nbG = 0;
+    LAUNCH(EXPM_STAGE_CGS, launch_proj_mma(P->V32, ld, cols, P->W, ld, p, n, P->part, maxb, P->sms, &nb, s));
+    LAUNCH(EXPM_STAGE_REDUCE, launch_reduce_h(P->part, nb, cols, p, h, P->H, P->ldH, 0, hcol, 0, s));
+    LAUNCH(EXPM_STAGE_CGS, launch_upd_mma(P->V, ld, cols, P->W, ld, p, n, h, P->colexp, P->partG, P->H, P->ldH, hcol,
+                                          flags, P->nblkG, P->sms, &nbG, s));
+    LAUNCH(EXPM_STAGE_CGS, launch_proj_mma(P->V32, ld, cols, P->W, ld, p, n, P->part, maxb, P->sms, &nb, s));
+    LAUNCH(EXPM_STAGE_REDUCE, launch_reduce_factor(P->part, nb, P->partG, nbG, cols, p, h, P->H, P->ldH, hrow, hcol,
+                                                   sm(P, kOffR), sm(P, kOffRt), P->fac, P->ctr + 1, flags,
+                                                   P->qr_single ? 1 : 0, s));
+    LAUNCH(EXPM_STAGE_QR, launch_qr_apply(P->W, ld, p, n, P->V32, ld, cols, h, P->fac, out, out32, ld, P->colexp + cols,
+                                          flags, P->sms_rows, s));
+    if (p <= kRowsMaxP) {
+        double* G = sm(P, kOffG);
+        LAUNCH(EXPM_STAGE_QR, launch_qr_mixed_rows(P->W, ld, p, n, P->nblk, G, P->part, P->ctr, 0, sm(P, kOffR),
+                                                   sm(P, kOffRi), nullptr, sm(P, kOffRt), P->H, P->ldH, hrow, hcol,
+                                                   nullptr, flags, P->W, ld, s, P->V, ld, cols, h, nullptr, ld, nullptr,
+                                                   nullptr, 1));
+        LAUNCH(EXPM_STAGE_QR, launch_qr_mixed_rows(P->W, ld, p, n, P->nblk, G, P->part, P->ctr, 1, sm(P, kOffR),
+                                                   sm(P, kOffRi), sm(P, kOffRt), sm(P, kOffRt2), P->H, P->ldH, hrow,
+                                                   hcol, nullptr, flags, out, ld, s, nullptr, 0, 0, nullptr, nullptr, 0,
+                                                   out32, P->colexp + cols));
+        LAUNCH(EXPM_STAGE_QR, launch_qr_mixed_rows(P->W, ld, p, n, P->nblk, G, P->part, P->ctr, 2, sm(P, kOffR),
+                                                   sm(P, kOffRi), sm(P, kOffRt2), sm(P, kOffRt3), P->H, P->ldH, hrow,
+                                                   hcol, nullptr, flags, out, ld, s, nullptr, 0, 0, nullptr, nullptr, 0,
+                                                   out32, P->colexp + cols));
+        return EXPM_OK;
+    }
+    const int* done = flags + 3;
+    LAUNCH(EXPM_STAGE_QR, launch_update_proj(P->V, ld, cols, P->W, ld, p, n, h, P->part, P->nblk, 1, s, 0, 1, nullptr,
+                                             nullptr, done));
+    expm_status st = qr_block(P, p, out, ld, true, hrow, hcol, nullptr, true, 0, done);
+    if (st != EXPM_OK) return st;
+    LAUNCH(EXPM_STAGE_QR, launch_pack_block(out, out32, ld, n, p, P->colexp + cols, done, s));
+    return EXPM_OK;
+}
+
 // Block step j (0-based): V_j -> W = Op V_j -> V_{j+1}, H column block j.
 // Op = (tA)^{-1} (Algorithm 2) or tA (Algorithm 1).
 expm_status block_step(expm_plan* P, double t, int j, int p, int alg) {
@@ -351,6 +400,7 @@ expm_status block_step(expm_plan* P, double t, int j, int p, int alg) {
         if (st != EXPM_OK) return st;
     }
     const int cols = (j + 1) * p;
+    if (P->mma) return ortho_mma(P, j, p);
     const int f32 = P->opts.precision == EXPM_PREC_MIXED ? 1 : 0;
     const int nbc = P->nblk_cgs;
     // first pass: FP64, or in the mixed path FP32 projection and double-float update (the
@@ -444,6 +494,7 @@ expm_status restart_prologue(expm_plan* P, int p, int kk, int prologue) {
     double* Vnext = P->V + (int64_t)mp * ld;
     if (prologue == 1) {
         LAUNCH(EXPM_STAGE_UPDATE, launch_copy(Vnext, ld, P->V, ld, n, p, s));
+        if (P->mma) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
         return EXPM_OK;
     }
     CK(cudaMemcpyAsync(P->Pkd, P->hPk, sizeof(double) * (size_t)mp * kk, cudaMemcpyHostToDevice, s));
@@ -455,6 +506,7 @@ expm_status restart_prologue(expm_plan* P, int p, int kk, int prologue) {
     }
     LAUNCH(EXPM_STAGE_UPDATE, launch_copy(Vnext, ld, P->V + (int64_t)kk * ld, ld, n, p, s));
     LAUNCH(EXPM_STAGE_UPDATE, launch_copy(P->Vk, ld, P->V, ld, n, kk, s));
+    if (P->mma) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, kk + p, P->colexp, nullptr, s));
     CK(cudaMemsetAsync(P->H, 0, sizeof(double) * (size_t)P->ldH * P->opts.m * P->p_max, s));
     CK(cudaMemcpy2DAsync(P->H, sizeof(double) * P->ldH, P->hHnew, sizeof(double) * P->ldH,
                          sizeof(double) * (size_t)(kk + p), kk, cudaMemcpyHostToDevice, s));
@@ -492,7 +544,10 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
     // mixed path: the product V Wc in double-float on the FP32 pipe (FP64 accumulation into Z)
     // (with deflation the restart happens in the next cycle's prologue, after V_m P_k)
     const bool defl = P->opts.k_defl > 0;
-    LAUNCH(EXPM_STAGE_UPDATE, launch_update_z(P->V, ld, mp + p, p, n, sm(P, kOffWc), P->Zacc, ld, defl ? 0 : 1, s,
+    if (P->mma)
+        LAUNCH(EXPM_STAGE_UPDATE, launch_updz_mma(P->V, P->V32, ld, mp + p, P->Zacc, ld, p, n, sm(P, kOffWc), P->colexp,
+                                                  flags_of(P->stat), defl ? 0 : 1, P->sms_rows, s));
+    else LAUNCH(EXPM_STAGE_UPDATE, launch_update_z(P->V, ld, mp + p, p, n, sm(P, kOffWc), P->Zacc, ld, defl ? 0 : 1, s,
                                               P->nblk, P->opts.precision == EXPM_PREC_MIXED ? 1 : 0));
     if (!d2h) return EXPM_OK;   // the batch graph's stop test reads the status on the device
     CK(cudaMemcpyAsync(P->hpin, P->stat, sizeof(double) * kStatDoubles, cudaMemcpyDeviceToHost, s));
@@ -579,6 +634,7 @@ expm_status run_begin(expm_plan* P, RunState& r) {
     LAUNCH(EXPM_STAGE_OTHER, launch_copy(r.dB, r.ldb, P->W, ld, n, p, s));
     expm_status st = qr_block(P, p, P->V, ld, false, 0, 0, P->stat + 16, false);
     if (st != EXPM_OK) return st;
+    if (P->mma) LAUNCH(EXPM_STAGE_QR, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
     if (fused_qr(P, p))   // the fused QR leaves R in Rt2, or in Rt3 when its third pass ran
         LAUNCH(EXPM_STAGE_OTHER, launch_init_S(sm(P, kOffRt2), p, P->npoles, P->S, s, sm(P, kOffRt3),
                                                flags_of(P->stat) + 2));
@@ -801,6 +857,10 @@ void free_plan(expm_plan* P) {
     delete[] P->hcert;
     cudaFree(P->H);
     cudaFree(P->part);
+    cudaFree(P->V32);
+    cudaFree(P->colexp);
+    cudaFree(P->partG);
+    cudaFree(P->fac);
     cudaFree(P->small);
     cudaFree(P->poles);
     cudaFree(P->S);
@@ -1298,6 +1358,9 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         // shape (see block_step).  Test switch: "1" for every block step it fits, "0" never
         const char* ptc = std::getenv("EXPM_PROJ_TC");
         P->proj_tc = opts->precision != EXPM_PREC_MIXED ? 0 : !ptc ? 2 : ptc[0] == '1' ? 1 : 0;
+        // mixed plans run the register-streamed passes (k_mma.cu); either switch above keeps a plan
+        // on the kernels it names
+        P->mma = opts->precision == EXPM_PREC_MIXED && !tc && !ptc && mma_fit(opts->m * p_max, p_max);
         // test switch: the bound of the tensor-core kernel's waits (0 makes every wait run out)
         const char* sl = std::getenv("EXPM_TC_SPIN_LIMIT");
         if (sl) P->tc_spin = std::strtol(sl, nullptr, 10);
@@ -1370,6 +1433,9 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         // first CGS pass; for the other row passes, the share of it that the plan was given.
         int per_sm = opts->row_ctas_per_sm > 0 ? opts->row_ctas_per_sm : 2;
         const int sms_rows = opts->grid_sms > 0 ? std::min(sms, (int)opts->grid_sms) : sms;
+        P->sms = sms;
+        P->sms_rows = sms_rows;
+        P->nblkG = 4 * sms;
         P->nblk = consistent_blocks(n, std::max(1, std::min<int>(per_sm * sms_rows, (int)((n + 63) / 64))));
         // the first CGS pass (projection, update) may use more CTAs than the other row passes
         const int per_sm_cgs = opts->cgs_ctas_per_sm > 0 ? opts->cgs_ctas_per_sm : 2 * per_sm;
@@ -1453,6 +1519,13 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
             ok = ok && dalloc(&P->R64, (size_t)ld * p_max);
         }
     }
+    if (P->mma) {
+        const size_t v32 = (size_t)ld * (m + 1) * p_max;
+        ok = ok && dalloc(&P->V32, v32) && dalloc(&P->colexp, (size_t)(m + 2) * p_max) &&
+             dalloc(&P->partG, (size_t)P->nblkG * p_max * p_max) && dalloc(&P->fac, 2 * kMaxP * kMaxP + 2 * kMaxP) &&
+             cudaMemsetAsync(P->V32, 0, sizeof(float) * v32, P->stream) == cudaSuccess &&
+             cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, P->stream) == cudaSuccess;
+    }
     if (!ok) {
         cudaGetLastError();
         free_plan(P);
@@ -1460,7 +1533,8 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
     }
     cudaStream_t s = P->stream;
     bool cuda_ok = krylov_set_smem_limits() == cudaSuccess && poles_set_smem_limits() == cudaSuccess &&
-                   operator_set_smem_limits() == cudaSuccess && cgs_tc_set_smem_limits() == cudaSuccess;
+                   operator_set_smem_limits() == cudaSuccess && cgs_tc_set_smem_limits() == cudaSuccess &&
+                   mma_set_smem_limits() == cudaSuccess;
     if (csr && cuda_ok) {
         CsrOp& c = P->cs;
         cuda_ok = cudaMemcpyAsync(c.rowptr, op->csr_rowptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice, s) == cudaSuccess &&
@@ -1899,6 +1973,7 @@ expm_status expm_arnoldi(expm_plan* plan, double t, const double* dV1, int64_t l
     CK(cudaMemsetAsync(plan->H, 0, sizeof(double) * (size_t)plan->ldH * m * plan->p_max, s));
     expm_plan* P = plan;
     LAUNCH(EXPM_STAGE_OTHER, launch_copy(dV1, ldv1, plan->V, ld, n, p, s));
+    if (P->mma) LAUNCH(EXPM_STAGE_OTHER, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
     for (int j = 0; j < m; ++j) {
         st = block_step(plan, t, j, p, EXPM_ALG_PSBFOM);
         if (st != EXPM_OK) return st;

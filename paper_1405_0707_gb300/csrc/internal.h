@@ -233,6 +233,13 @@ struct expm_plan_s {
     int cgs_tc = 0;            // mixed path, first CGS update on the tensor cores: 0 never, 1 always, 2 by shape
     int proj_tc = 0;           // mixed path, first CGS projection on the tensor cores: 0 never, 1 always, 2 by shape
     int stencil_df = 0;        // mixed path: the stencil in double-float (k_cd_apply_df)
+    bool mma = false;          // mixed path: the register-streamed tensor-core passes (k_mma.cu)
+    int sms = 0, sms_rows = 0; // SMs of the device, and the share the row passes are sized for
+    float* V32 = nullptr;      // ld x (m+1) p_max   FP32 copy of V (rows n .. ld - 1 zero)
+    int* colexp = nullptr;     // (m+2) p_max        largest biased exponent of each column of V
+    double* partG = nullptr;   // nblkG x p_max x p_max Gram partials of the update
+    int nblkG = 0;
+    float* fac = nullptr;      // the block's factor for k_qr_apply
     long tc_spin = 1L << 24;   // bound of the tensor-core kernel's mbarrier waits (iterations)
     // deflated restart (opts.k_defl > 0)
     int kdefl_max = 0;         // columns of Vk and Pkd
@@ -286,7 +293,7 @@ cudaError_t launch_reduce_h(const double* part, int nblk, int cols, int p, doubl
 cudaError_t launch_update_proj(const double* V, int64_t ldv, int cols, double* W, int64_t ldw,
                                int p, int64_t n, const double* h, double* part, int nblk,
                                int gram, cudaStream_t s, int f32 = 0, int upd32 = 0, double* G = nullptr,
-                               unsigned* ctr = nullptr);
+                               unsigned* ctr = nullptr, const int* skip = nullptr);
 // Mixed path, p <= 8: Cholesky-QR pass with an FP32 factorisation (mode 0: of G; modes 1
 // and 2: of the deviation G - I), corrections in FP32, W and the R product in FP64.
 cudaError_t launch_qr_mixed_rows(double* W, int64_t ldw, int p, int64_t n, int nblk, double* G, double* part,
@@ -294,7 +301,8 @@ cudaError_t launch_qr_mixed_rows(double* W, int64_t ldw, int p, int64_t n, int n
                                  double* Rtot_out, double* H, int ldH, int hrow, int hcol, double* normsq_out,
                                  int* flags, double* out, int64_t ldo, cudaStream_t s,
                                  const double* Vc = nullptr, int64_t ldvc = 0, int ccols = 0,
-                                 const double* h2 = nullptr, double* fin = nullptr, int64_t ldfin = 0);
+                                 const double* h2 = nullptr, double* fin = nullptr, int64_t ldfin = 0,
+                                 float* out32 = nullptr, int* colexp = nullptr, int skip_done = 0);
 constexpr int kRowsMaxP = 16;  // widths handled by the row-per-thread kernels
 // The first CGS pass's update W <- W - V h on the tensor cores (k_cgs_tc.cu): p <= 16,
 // cols <= 160.  The second projection and the Gram matrix follow from launch_cgs_rows(0, ...,
@@ -311,14 +319,35 @@ int proj_tc_blocks(int64_t n, int cols, int max_blocks);
 cudaError_t launch_proj_tc(const double* V, int64_t ldv, int cols, const double* W, int64_t ldw, int p, int64_t n,
                            double* part, int nb, int* flags, long spin_limit, cudaStream_t s);
 cudaError_t cgs_tc_set_smem_limits();
+// The register-streamed tensor-core passes of the mixed path (k_mma.cu), p <= 32: projection from
+// the FP32 basis copy (nb partials of cols x p), update with the Gram partials (nb of p x p) and
+// the rounded h recorded in H, Z update with the restart copy; V32 and colexp of other blocks.
+bool mma_fit(int mp, int p);
+cudaError_t launch_proj_mma(const float* V32, int64_t ldv, int cols, const double* W, int64_t ldw, int p, int64_t n,
+                            double* part, int max_blocks, int sms, int* nb, cudaStream_t s);
+cudaError_t launch_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,
+                           int* colexp, double* partG, double* H, int ldH, int hcol, int* flags, int max_blocks, int sms,
+                           int* nb, cudaStream_t s);
+cudaError_t launch_updz_mma(double* V, float* V32, int64_t ldv, int cols, double* Z, int64_t ldz, int p, int64_t n,
+                            const double* Wc, int* colexp, int* flags, int restart, int sms, cudaStream_t s);
+cudaError_t launch_pack_block(const double* V, float* V32, int64_t ld, int64_t n, int p, int* colexp, const int* skip,
+                              cudaStream_t s);
+cudaError_t mma_set_smem_limits();
+// The Cholesky-QR step after the second projection (rows_qr.cuh)
+cudaError_t launch_reduce_factor(const double* part, int nblk, const double* partG, int nblkG, int cols, int p, double* h,
+                                 double* H, int ldH, int hrow, int hcol, double* R, double* Rtot, float* fac,
+                                 unsigned* ctr, int* flags, int allow, cudaStream_t s);
+cudaError_t launch_qr_apply(const double* W, int64_t ldw, int p, int64_t n, const float* V32, int64_t ldv, int cols,
+                            const double* h2, const float* fac, double* out, float* out32, int64_t ldo, int* colexp,
+                            const int* flags, int sms, cudaStream_t s);
 // Cholesky-QR passes: mode 0 (unshifted, shifted on ill-conditioning, sets flags[2] when a
 // third pass is needed), mode 1, mode 2 (no-op unless flags[2]); see k_krylov.cu.
 cudaError_t launch_chol(const double* part, int nblk, int p, double shift_rel, double* R,
                         double* Rinv, double* Rtot, int mode, double* H, int ldH, int hrow,
-                        int hcol, double* normsq_out, int* flags, cudaStream_t s);
+                        int hcol, double* normsq_out, int* flags, cudaStream_t s, const int* skip = nullptr);
 cudaError_t launch_trsm(double* W, int64_t ldw, int p, int64_t n, const double* Rinv,
                         double* out, int64_t ldo, double* part, int nblk, int gram,
-                        const int* extra, int tmode, cudaStream_t s);
+                        const int* extra, int tmode, cudaStream_t s, const int* skip = nullptr);
 // projected solves / update
 cudaError_t launch_poles(const double* H, int ldH, int mp, int p, int npoles,
                          const double* tau_re, const double* tau_im, const double* om_re,

@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(NT) k_update(const double* __restrict__ V, int
                                                double* __restrict__ W, int64_t ldw, int p,
                                                int64_t n, int64_t rpb,
                                                const double* __restrict__ h,
-                                               double* __restrict__ part, int gram) {
+                                               double* __restrict__ part, int gram, const int* skip) {
+    if (skip && *skip) return;            // the fused pass finished the block
     extern __shared__ double sm[];
     const int cs = cols | 1;
     double* hs = sm;                      // cols x p
@@ -440,7 +441,9 @@ constexpr int CHOL_T = 1024;
 __global__ void __launch_bounds__(CHOL_T) k_chol(const double* __restrict__ part, int nblk, int p,
                                                  double shift_rel, double* R, double* Rinv,
                                                  double* Rtot, int mode, double* H, int ldH,
-                                                 int hrow, int hcol, double* normsq_out, int* flags) {
+                                                 int hrow, int hcol, double* normsq_out, int* flags,
+                                                 const int* skip) {
+    if (skip && *skip) return;
     int* extra = flags + 2;
     if (mode == 2 && *extra == 0) return;
     __shared__ double G[kMaxP * kMaxP], G0[kMaxP * kMaxP], Rs[kMaxP * kMaxP], Ri[kMaxP * kMaxP],
@@ -588,7 +591,8 @@ __global__ void __launch_bounds__(NT) k_trsm(double* W, int64_t ldw, int p, int6
                                              int64_t rpb, const double* __restrict__ Rinv,
                                              double* out_, int64_t ldo_,
                                              double* __restrict__ part, int gram_,
-                                             const int* extra, int tmode) {
+                                             const int* extra, int tmode, const int* skip) {
+    if (skip && *skip) return;
     const TrsmPass ps = trsm_pass(W, ldw, out_, ldo_, gram_, extra, tmode);
     if (ps.skip) return;
     double* out = ps.dest;
@@ -753,15 +757,31 @@ cudaError_t launch_qr_mixed_rows(double* W, int64_t ldw, int p, int64_t n, int n
                                  unsigned* ctr, int mode, double* R, double* Rinv, const double* Rtot_in,
                                  double* Rtot_out, double* H, int ldH, int hrow, int hcol, double* normsq_out,
                                  int* flags, double* out, int64_t ldo, cudaStream_t s, const double* Vc,
-                                 int64_t ldvc, int ccols, const double* h2, double* fin, int64_t ldfin) {
+                                 int64_t ldvc, int ccols, const double* h2, double* fin, int64_t ldfin, float* out32,
+                                 int* colexp, int skip_done) {
     if (p < 1 || p > kRowsMaxP) return cudaErrorInvalidValue;
     return EXPM_ROWS_CALL(p, qr(W, ldw, p, n, nblk, G, part, ctr, mode, R, Rinv, Rtot_in, Rtot_out, H, ldH, hrow,
-                                hcol, normsq_out, flags, out, ldo, s, Vc, ldvc, ccols, h2, fin, ldfin));
+                                hcol, normsq_out, flags, out, ldo, s, Vc, ldvc, ccols, h2, fin, ldfin, out32, colexp,
+                                skip_done));
+}
+
+cudaError_t launch_reduce_factor(const double* part, int nblk, const double* partG, int nblkG, int cols, int p, double* h,
+                                 double* H, int ldH, int hrow, int hcol, double* R, double* Rtot, float* fac,
+                                 unsigned* ctr, int* flags, int allow, cudaStream_t s) {
+    return EXPM_ROWS_QR_CALL(p, reduce_factor(part, nblk, partG, nblkG, cols, p, h, H, ldH, hrow, hcol, R, Rtot, fac, ctr,
+                                              flags, allow, s));
+}
+
+cudaError_t launch_qr_apply(const double* W, int64_t ldw, int p, int64_t n, const float* V32, int64_t ldv, int cols,
+                            const double* h2, const float* fac, double* out, float* out32, int64_t ldo, int* colexp,
+                            const int* flags, int sms, cudaStream_t s) {
+    return EXPM_ROWS_QR_CALL(p, qr_apply(W, ldw, p, n, V32, ldv, cols, h2, fac, out, out32, ldo, colexp, flags, sms, s));
 }
 
 cudaError_t launch_update_proj(const double* V, int64_t ldv, int cols, double* W, int64_t ldw,
                                int p, int64_t n, const double* h, double* part, int nblk,
-                               int gram, cudaStream_t s, int f32, int upd32, double* G, unsigned* ctr) {
+                               int gram, cudaStream_t s, int f32, int upd32, double* G, unsigned* ctr,
+                               const int* skip) {
     const int64_t rpb = rows_per_block(n, nblk);
     const int g = blocks_for(n, nblk);
     size_t shm = sizeof(double) * ((size_t)cols * p + TR * (cols | 1) + TR * p);
@@ -772,33 +792,33 @@ cudaError_t launch_update_proj(const double* V, int64_t ldv, int cols, double* W
         return EXPM_ROWS_CALL(p, upd_gram(V, ldv, cols, W, ldw, p, n, h, part, nblk, G, ctr, upd32, s));
     if (upd32 && gram)
         EXPM_OPT_DISPATCH(nout, (k_update<O, false, true><<<g, NT, shm, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part,
-                                                                             gram)));
+                                                                             gram, skip)));
     else if (f32 && !gram && f32 == 2) {
         const size_t shm_df = sizeof(float) * (2 * (size_t)cols * p + 2 * TR * (cols | 1) + TR * p + 2 * NT);
         EXPM_OPT_DISPATCH(nout, (k_update_df<O><<<g, NT, shm_df, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part)));
     } else if (f32)
-        EXPM_OPT_DISPATCH(nout, (k_update<O, true><<<g, NT, shm, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part, gram)));
+        EXPM_OPT_DISPATCH(nout, (k_update<O, true><<<g, NT, shm, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part, gram, skip)));
     else
-        EXPM_OPT_DISPATCH(nout, (k_update<O, false><<<g, NT, shm, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part, gram)));
+        EXPM_OPT_DISPATCH(nout, (k_update<O, false><<<g, NT, shm, s>>>(V, ldv, cols, W, ldw, p, n, rpb, h, part, gram, skip)));
     return cudaGetLastError();
 }
 
 cudaError_t launch_chol(const double* part, int nblk, int p, double shift_rel, double* R,
                         double* Rinv, double* Rtot, int mode, double* H, int ldH, int hrow,
-                        int hcol, double* normsq_out, int* flags, cudaStream_t s) {
+                        int hcol, double* normsq_out, int* flags, cudaStream_t s, const int* skip) {
     k_chol<<<1, CHOL_T, 0, s>>>(part, nblk, p, shift_rel, R, Rinv, Rtot, mode, H, ldH, hrow, hcol,
-                                normsq_out, flags);
+                                normsq_out, flags, skip);
     return cudaGetLastError();
 }
 
 cudaError_t launch_trsm(double* W, int64_t ldw, int p, int64_t n, const double* Rinv,
                         double* out, int64_t ldo, double* part, int nblk, int gram,
-                        const int* extra, int tmode, cudaStream_t s) {
+                        const int* extra, int tmode, cudaStream_t s, const int* skip) {
     const int64_t rpb = rows_per_block(n, nblk);
     const int g = blocks_for(n, nblk);
-    if (p <= kRowsMaxP) return EXPM_ROWS_CALL(p, trsm(W, ldw, p, n, Rinv, out, ldo, part, nblk, gram, extra, tmode, s));
+    if (p <= kRowsMaxP && !skip) return EXPM_ROWS_CALL(p, trsm(W, ldw, p, n, Rinv, out, ldo, part, nblk, gram, extra, tmode, s));
     EXPM_OPT_DISPATCH(p * p, (k_trsm<O><<<g, NT, 0, s>>>(W, ldw, p, n, rpb, Rinv, out, ldo, part, gram,
-                                                       extra, tmode)));
+                                                       extra, tmode, skip)));
     return cudaGetLastError();
 }
 
@@ -877,6 +897,11 @@ cudaError_t krylov_set_smem_limits() {
     if (e == cudaSuccess) e = rows8::set_smem(optin);
     if (e == cudaSuccess) e = rows12::set_smem(optin);
     if (e == cudaSuccess) e = rows16::set_smem(optin);
+    if (e == cudaSuccess) e = rows4::qr_set_smem();
+    if (e == cudaSuccess) e = rows8::qr_set_smem();
+    if (e == cudaSuccess) e = rows12::qr_set_smem();
+    if (e == cudaSuccess) e = rows16::qr_set_smem();
+    if (e == cudaSuccess) e = rows32::qr_set_smem();
 #undef EXPM_SET
     return e;
 }

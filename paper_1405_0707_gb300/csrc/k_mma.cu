@@ -1,0 +1,651 @@
+// k_mma.cu -- the tall-skinny products of the mixed path as register-streamed tensor-core
+// passes (mma.sync): the Gram-Schmidt projections h = V^T W, the update W <- W - V h, and the
+// solution update Z <- Z + V Wc, for blocks of p <= 32 columns against any number of basis
+// columns.
+//
+// What bounds these passes: each reads the n x cols basis once and does 2 n cols p useful flop
+// on it, so their floor is the basis's bytes at the memory rate.  Earlier forms staged every
+// element through shared memory (FP64 bytes, an integer FP64 -> FP32 conversion, a store, a
+// barrier, a load per FMA) and were bound by issue slots and latency at 0.2-0.4 of that rate.
+// Here the operands go from global memory straight into MMA fragments: a fragment's K (or M)
+// index may be any permutation of the rows as long as both operands use the same one, so each
+// lane loads 16 contiguous bytes of a column and no shared-memory pass or barrier remains.
+//
+//  * The projections read an FP32 copy of the basis (V32, written with every new block; the
+//    FP32 rounding is the one the CUDA-core projection applied on each read), half the bytes.
+//    Each FP32 value is split exactly enough into three bf16 parts, and the six products
+//    v0w0 | v0w1 v1w0 v1w1 v0w2 v2w0 go to two accumulators (the second 2^-8 smaller), so the
+//    product error is ~2^-25, below the FP32 rounding of the operands.  Every few hundred rows
+//    the main accumulator is added to a float pair, so summation error does not grow with n.
+//  * The update must hold to FP64 rounding (the Arnoldi relation of eq. (4.5)).  Both operands
+//    are cut into balanced base-256 digits held exactly in fp16, products of digits are summed
+//    by level (digit positions i + j) in FP32 accumulators that stay below 2^24, hence exact,
+//    and the level sums are combined in float pairs.  V's digits are scaled per column by the
+//    exponent of its largest entry (colexp, kept with each block): seven digits then resolve
+//    2^-55 of that entry.
+//  * h of the first pass only seeds the second pass, so the update rounds it to four digits
+//    (2^-32 of the largest scaled entry of its column, finer than the FP32 projection it came
+//    from), subtracts V times exactly that h and records exactly that h in H: the relation does
+//    not see the rounding, and 22 digit products replace 27.  The Z update keeps six digits.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "df.cuh"
+#include "internal.h"
+#include "mma.cuh"
+
+namespace expm {
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// ---------------------------------------------------------------- projection
+constexpr int kProjKb = 8;                       // 16-row blocks per unit: 128 rows
+constexpr size_t proj_smem(int NT, int MTW) {
+    return std::max((size_t)NT * MTW * 4 * 8 * 32 * sizeof(float2), (size_t)2 * kProjKb * NT * 3 * 32 * sizeof(uint2));
+}
+
+// v rounded to FP32 (nearest, ties away), below 2^-126 flushed to zero; not for inf and NaN, whose
+// blocks the Gram matrix of the update flags
+__device__ __forceinline__ float f32_fast(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t f = __funnelshift_l(lo, hi, 3) - (384u << 23) + ((lo >> 28) & 1u);
+    return ((hi & 0x7FFFFFFFu) >> 20) < 897u ? 0.f : __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// partial[bx][a][c] = sum over the rows of row group bx of V[r, a] W[r, c].
+// MMA: M = 16 basis columns, N = 8 block columns, K = 16 rows.  A warp owns up to MTW M tiles
+// (a = 16 (cg + CG i)) and every N tile; the CTA's 8 warps are CG column groups x 8 / CG row
+// groups; grid.y covers bases wider than CG MTW tiles.  Rows are taken in units of 128: W's unit
+// is converted to fragments in shared memory once per CTA (its conversion from FP64 costs more
+// instructions than the products it feeds when every warp repeats it), two buffers, one barrier
+// per unit; V's next block is loaded while the current one is multiplied.
+template <int NT, int MTW>
+__global__ void __launch_bounds__(256, (NT * MTW <= 4) ? 2 : 1)
+k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __restrict__ W, int64_t ldw, int p,
+           int64_t n, double* __restrict__ part, int CG) {
+    extern __shared__ __align__(16) unsigned char smp[];
+    uint2* wf = reinterpret_cast<uint2*>(smp);             // [buf][kb][nt][split][lane]
+    constexpr int WBUF = kProjKb * NT * 3 * 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int cg = warp % CG, rg = warp / CG, RG = 8 / CG;
+    const int mt_all = (cols + 15) >> 4, mt0 = blockIdx.y * CG * MTW + cg;
+    float cm[MTW][NT][4], cc[MTW][NT][4], ch[MTW][NT][4];
+#pragma unroll
+    for (int i = 0; i < MTW; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cm[i][j][q] = cc[i][j][q] = ch[i][j][q] = 0.f;
+    const int nmt = mt0 < mt_all ? min(MTW, (mt_all - mt0 + CG - 1) / CG) : 0;   // tiles this warp owns
+    const int64_t nblk = (n + 15) >> 4, units = (nblk + kProjKb - 1) / kProjKb;
+    auto loadv = [&](float4* v, int i, int64_t blk) {
+        const int a = (mt0 + i * CG) * 16 + g;
+        const int64_t r0 = blk * 16 + 4 * t;
+        v[0] = *reinterpret_cast<const float4*>(V + (int64_t)min(a, cols - 1) * ldv + r0);
+        v[1] = *reinterpret_cast<const float4*>(V + (int64_t)min(a + 8, cols - 1) * ldv + r0);
+    };
+    double2 w[NT][2];
+    auto loadw = [&](int64_t u) {                          // item k: block kb = warp, N tile k
+        const int64_t r = (u * kProjKb + warp) * 16 + 4 * t;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            w[j][0] = w[j][1] = make_double2(0.0, 0.0);
+            const double* src = W + (int64_t)min(8 * j + g, p - 1) * ldw + r;
+            if (r < n) {                                   // columns are padded to 32 rows
+                w[j][0] = *reinterpret_cast<const double2*>(src);
+                w[j][1] = *reinterpret_cast<const double2*>(src + 2);
+                if (r + 1 >= n) w[j][0].y = 0.0;           // the padding is not W's
+                if (r + 2 >= n) w[j][1].x = 0.0;
+                if (r + 3 >= n) w[j][1].y = 0.0;
+            }
+        }
+    };
+    auto storew = [&](int buf) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            uint32_t s0[3], s1[3];
+            split3(f32_fast(w[j][0].x), f32_fast(w[j][0].y), s0);
+            split3(f32_fast(w[j][1].x), f32_fast(w[j][1].y), s1);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) wf[buf * WBUF + ((warp * NT + j) * 3 + k) * 32 + lane] = make_uint2(s0[k], s1[k]);
+        }
+    };
+    int64_t u = blockIdx.x;
+    float4 v[MTW][2];
+    int buf = 0;
+    if (u < units) {
+        loadw(u);
+        const int64_t b0 = u * kProjKb + rg;
+#pragma unroll
+        for (int i = 0; i < MTW; ++i)
+            if (i < nmt && b0 < nblk) loadv(v[i], i, b0);
+        storew(0);
+    }
+    __syncthreads();
+    for (; u < units; u += gridDim.x) {
+        const int64_t un = u + gridDim.x;
+        if (un < units) loadw(un);
+        const int64_t bend = min(nblk, (u + 1) * kProjKb);
+        for (int64_t b = u * kProjKb + rg; b < bend; b += RG) {
+            int64_t bn = b + RG;
+            if (bn >= bend) bn = un * kProjKb + rg;
+            const bool more = bn < nblk;
+            const uint2* wq = wf + buf * WBUF + (int)(b - u * kProjKb) * NT * 3 * 32 + lane;
+            uint2 wb[NT][3];
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) wb[j][k] = wq[(j * 3 + k) * 32];
+#pragma unroll
+            for (int i = 0; i < MTW; ++i)
+                if (i < nmt) {
+                    uint32_t a[3][4];
+                    {
+                        uint32_t s[3];
+                        split3(v[i][0].x, v[i][0].y, s);
+                        a[0][0] = s[0]; a[1][0] = s[1]; a[2][0] = s[2];
+                        split3(v[i][1].x, v[i][1].y, s);
+                        a[0][1] = s[0]; a[1][1] = s[1]; a[2][1] = s[2];
+                        split3(v[i][0].z, v[i][0].w, s);
+                        a[0][2] = s[0]; a[1][2] = s[1]; a[2][2] = s[2];
+                        split3(v[i][1].z, v[i][1].w, s);
+                        a[0][3] = s[0]; a[1][3] = s[1]; a[2][3] = s[2];
+                    }
+                    if (more) loadv(v[i], i, bn);
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        mma_bf16(cc[i][j], a[2], wb[j][0].x, wb[j][0].y);
+                        mma_bf16(cm[i][j], a[0], wb[j][0].x, wb[j][0].y);
+                        mma_bf16(cc[i][j], a[0], wb[j][2].x, wb[j][2].y);
+                        mma_bf16(cc[i][j], a[1], wb[j][1].x, wb[j][1].y);
+                        mma_bf16(cc[i][j], a[1], wb[j][0].x, wb[j][0].y);
+                        mma_bf16(cc[i][j], a[0], wb[j][1].x, wb[j][1].y);
+                    }
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < MTW; ++i)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    df_add(ch[i][j][q], cc[i][j][q], cm[i][j][q]);
+                    cm[i][j][q] = 0.f;
+                }
+        buf ^= 1;
+        if (un < units) storew(buf);
+        __syncthreads();
+    }
+    // the row groups' sums in float pairs (FP64 adds here cost more than the products above: one
+    // FP64 warp instruction occupies its scheduler for ~64 clocks), one FP64 value per output
+    float2* red = reinterpret_cast<float2*>(smp);          // [tile][q][warp][lane]
+#pragma unroll
+    for (int i = 0; i < MTW; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                red[(((i * NT + j) * 4 + q) * 8 + warp) * 32 + lane] = make_float2(ch[i][j][q], cc[i][j][q]);
+    __syncthreads();
+    double* out = part + (int64_t)blockIdx.x * cols * p;
+    const int tiles_y = min(CG * MTW, mt_all - (int)blockIdx.y * CG * MTW);   // M tiles of this CTA
+    for (int e = threadIdx.x; e < tiles_y * NT * 128; e += 256) {
+        const int ln = e & 31, q = (e >> 5) & 3, mj = e >> 7, j = mj % NT, m = mj / NT;
+        const int i = m / CG, w0 = m - i * CG;
+        const int aa = (blockIdx.y * CG * MTW + m) * 16 + (ln >> 2) + (q >> 1) * 8, c = 8 * j + 2 * (ln & 3) + (q & 1);
+        if (aa >= cols || c >= p) continue;
+        const float2* src = red + ((i * NT + j) * 4 + q) * 256 + w0 * 32 + ln;
+        float sh = src[0].x, sl = src[0].y;
+        for (int k = 1; k < RG; ++k) {
+            const float2 x = src[k * CG * 32];
+            df_add(sh, sl, x.x);
+            sl += x.y;
+        }
+        out[(int64_t)aa * p + c] = f64_of_f32_i(sh) + f64_of_f32_i(sl);
+    }
+}
+
+// ---------------------------------------------------------------- digits
+// The seven balanced base-256 digits of v 2^(1022 - emax) (magnitude below 1; c9 = 9 + emax), as
+// the bytes of Y = X + bias with X the two's-complement value times 2^55: the top 16 bits of Y
+// read as fp16 are 1152 + d_0, and 0x6400 | byte is 1152 + d_i below.
+__device__ __forceinline__ void digits_y(double v, int c9, uint32_t& yl, uint32_t& yh) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t s = (uint32_t)(c9 - (int)((hi >> 20) & 0x7FFu));
+    const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
+    unsigned long long X = ((unsigned long long)mh << 32) | ml;
+    asm("shr.u64 %0, %0, %1;" : "+l"(X) : "r"(s));            // shifts of 64 and more give zero
+    const int sg = (int)hi >> 31;
+    const unsigned long long S = (unsigned long long)(long long)sg;
+    X = (X ^ S) + (0x6480808080808080ull - S);
+    yl = (uint32_t)X;
+    yh = (uint32_t)(X >> 32);
+}
+
+__device__ __forceinline__ uint32_t unbias(uint32_t x) {      // (1152 + d) - 1152 in both halves
+    uint32_t r;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(0xE480E480u));
+    return r;
+}
+// digit I of the pair (x in the low half, y in the high half)
+template <int I>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t xl, uint32_t xh, uint32_t yl, uint32_t yh) {
+    if constexpr (I == 0) return unbias(__byte_perm(xh, yh, 0x7632));
+    const uint32_t z = I <= 2 ? __byte_perm(xh, yh, 0x5410) : I <= 4 ? __byte_perm(xl, yl, 0x7632) : __byte_perm(xl, yl, 0x5410);
+    if constexpr (I % 2 == 0) return unbias((z & 0x00FF00FFu) | 0x64006400u);
+    return unbias(__byte_perm(z, 0x64646464u, 0x4341));
+}
+
+// x 2^k by an add to the exponent field (integer operations only); a result below the normal
+// range flushes to a signed zero and one above it becomes inf
+__device__ __forceinline__ double scale2_e(double x, int k) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7FF);
+    long long r = b + ((long long)k << 52);
+    if (e == 0 || e + k <= 0) r = b & (1LL << 63);
+    if (e != 0 && e + k >= 0x7FF) r = (b & (1LL << 63)) | (0x7FFLL << 52);
+    return __longlong_as_double(r);
+}
+
+// X 2^k as a double, |X| <= 2^52, built from its bit pattern (results below 2^-1022 flush to zero)
+__device__ __forceinline__ double scaled_int(long long X, int k) {
+    if (X == 0) return 0.0;
+    const unsigned long long m = (unsigned long long)(X < 0 ? -X : X);
+    const int lead = 63 - __clzll((long long)m), e = lead + k + 1023;
+    if (e <= 0) return 0.0;
+    const unsigned long long b = ((unsigned long long)e << 52) | ((m << (52 - lead)) & 0xFFFFFFFFFFFFFull);
+    return __longlong_as_double((long long)(b | (X < 0 ? 1ull << 63 : 0ull)));
+}
+
+constexpr int kUpdThreads = 128;
+__host__ __device__ constexpr int upd_seg(int NH) { return NH == 4 ? 15 : 10; }   // 16-column chunks per exact segment
+__host__ __device__ constexpr int gram_rounds(int NT) { return NT == 1 ? 5 : NT == 2 ? 5 : 17; }
+__host__ __device__ constexpr int gram_split(int NT) { return NT == 1 ? 4 : 1; }   // lanes sharing one Gram entry
+
+constexpr size_t upd_smem(int cols, int NT, int NH, bool gram) {
+    const size_t nk = (size_t)((cols + 15) / 16);
+    return nk * (NH / 2) * NT * 32 * 16 + nk * 16 * sizeof(int) +
+           (gram ? sizeof(float2) * (size_t)std::max((kUpdThreads / 32) * 16 * (8 * NT + 1), gram_rounds(NT) * 128) : 0);
+}
+
+// GS (NH = 4): W <- W - V h with h rounded as described at the top; CTA 0 records the rounded h in
+// H (columns hcol .., rows 0 .. cols - 1) and clears the next block's colexp; the Gram matrix of
+// the updated W in float pairs goes to partG[blk][p][p].
+// Z (NH = 6): Z <- Z + V Wc (sgn = 1), then the restart copy V[:, 0:p] <- V[:, cols-p:cols] of this
+// CTA's rows (and of V32) when asked.
+// MMA: M = 16 rows (lane group g holds rows 2g and 2g + 1, one 16-byte load per column), N = 8
+// block columns, K = 16 basis columns (lane t holds columns 4t .. 4t + 3).  One warp per 16-row
+// tile, the next chunk's loads in flight.  44 MMAs per 256 basis elements at p = 16 take about as
+// long as the elements' 8 bytes at the memory rate.
+template <int NT, int NH, bool GS>
+__global__ void __launch_bounds__(kUpdThreads, NT == 4 ? 2 : NT == 2 ? 3 : 4)
+k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* __restrict__ h,
+          int* __restrict__ colexp, double* __restrict__ partG, double* __restrict__ H, int ldH, int hcol,
+          int* flags, float* V32, int restart) {
+    extern __shared__ __align__(16) unsigned char smu[];
+    const int nk = (cols + 15) >> 4;
+    const int64_t ntiles = (n + 15) >> 4;
+    const int64_t tstep = (int64_t)gridDim.x * (kUpdThreads / 32);
+    int64_t tile = (int64_t)blockIdx.x * (kUpdThreads / 32) + (threadIdx.x >> 5);
+    double2 v[4];
+    auto load = [&](int64_t tl, int kc) {
+        const int64_t r = tl * 16 + 2 * ((threadIdx.x & 31) >> 2);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = *reinterpret_cast<const double2*>(V + (int64_t)min(kc * 16 + 4 * (int)(threadIdx.x & 3) + q, cols - 1) * ldv + r);
+    };
+    if (tile < ntiles) load(tile, 0);            // in flight while the digits of h are formed
+    __half* Bh = reinterpret_cast<__half*>(smu);
+    int* c9s = reinterpret_cast<int*>(smu + (size_t)nk * (NH / 2) * NT * 512);
+    float2* gbuf = reinterpret_cast<float2*>(c9s + nk * 16);
+    __shared__ int fmax_s[8 * NT], bad_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    constexpr int NCOL = 8 * NT;
+    for (int a = tid; a < nk * 16; a += kUpdThreads) c9s[a] = 9 + (a < cols ? colexp[a] : 0);
+    if (tid < NCOL) fmax_s[tid] = -100000;
+    if (tid == 0) bad_s = 0;
+    __syncthreads();
+    if (GS && blockIdx.x == 0 && tid < p) colexp[cols + tid] = 0;
+    // exponent f_c of column c of the scaled h: |h[a, c]| 2^(emax_a - 1022) < 2^f_c
+    for (int e = tid; e < cols * NCOL; e += kUpdThreads) {
+        const int a = e / NCOL, c = e - a * NCOL;
+        if (c < p) {
+            const int E = (int)(((unsigned)__double2hiint(h[a * p + c]) >> 20) & 0x7FFu);
+            if (E == 0x7FF) bad_s = 1;
+            const int em = c9s[a] - 9;
+            if (E > 0 && em > 0) atomicMax(&fmax_s[c], E - 1022 + em - 1022);
+        }
+    }
+    __syncthreads();
+    if (tid == 0 && bad_s) atomicOr(&flags[0], 1);
+    constexpr int SC = 8 * NH - 1;
+    for (int e = tid; e < nk * 16 * NCOL; e += kUpdThreads) {
+        const int a = e / NCOL, c = e - a * NCOL;
+        long long X = 0;
+        int sh = 0;
+        if (a < cols && c < p) {
+            const double hv = h[a * p + c];
+            const unsigned long long b = (unsigned long long)__double_as_longlong(hv);
+            const int E = (int)((b >> 52) & 0x7FF), em = c9s[a] - 9, f = fmax_s[c];
+            // |h| 2^(em - 1022) 2^(SC - f) = m 2^-sh, rounded to nearest
+            sh = 1075 - E + 1022 - em + f - SC;
+            if (E > 0 && em > 0 && sh <= 54) {
+                const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+                X = (long long)((m + (1ull << (sh - 1))) >> sh);
+                if (b >> 63) X = -X;
+            }
+            if (GS && blockIdx.x == 0) {
+                // the h that is applied, exactly: X 2^(f - SC) 2^(1022 - em)
+                H[(int64_t)(hcol + c) * ldH + a] = scaled_int(X, f - SC + 1022 - em);
+            }
+        }
+        const int kc = a >> 4, kk = a & 15;
+        const int ln = (c & 7) * 4 + (kk >> 2);
+#pragma unroll
+        for (int j = NH - 1; j >= 0; --j) {
+            int d;
+            if (j > 0) {
+                d = (int)((X + 128) & 255) - 128;
+                X = (X - d) >> 8;
+            } else {
+                d = (int)X;
+            }
+            Bh[((((size_t)kc * (NH / 2) + (j >> 1)) * NT + (c >> 3)) * 32 + ln) * 8 + (j & 1) * 4 + (kk & 3)] =
+                __int2half_rn(d);
+        }
+    }
+    __syncthreads();
+
+    constexpr int GK = GS ? gram_rounds(NT) : 1, GSP = gram_split(NT);
+    const int ne = p * (p + 1) / 2;
+    float gh[GK], gl[GK];
+    int gi[GK];                                  // packed (row group << 16 | i << 8 | j), -1 none
+    if (GS) {
+#pragma unroll
+        for (int k = 0; k < GK; ++k) {
+            gh[k] = gl[k] = 0.f;
+            const int it = lane + 32 * k;
+            gi[k] = -1;
+            if (it < ne * GSP) {
+                int i = 0, rem = it % ne;
+                while (rem >= p - i) {
+                    rem -= p - i;
+                    ++i;
+                }
+                gi[k] = ((it / ne) << 16) | (i << 8) | (i + rem);
+            }
+        }
+    }
+    float2* gw = gbuf + (size_t)warp * 16 * (NCOL + 1);
+    for (; tile < ntiles; tile += tstep) {
+        const int64_t r = tile * 16 + 2 * g;
+        double w[NT][4];                         // [nt]: (2g, c) (2g, c + 1) (2g + 1, c) (2g + 1, c + 1)
+        for (int k0 = 0; k0 < nk; k0 += upd_seg(NH)) {
+            const int k1 = min(nk, k0 + upd_seg(NH));
+            float acc[7][NT][4];
+#pragma unroll
+            for (int l = 0; l < 7; ++l)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[l][j][q] = 0.f;
+            for (int kc = k0; kc < k1; ++kc) {
+                uint32_t yl[4][2], yh[4][2];
+                const int4 c9 = *reinterpret_cast<const int4*>(c9s + kc * 16 + 4 * t);
+                digits_y(v[0].x, c9.x, yl[0][0], yh[0][0]);
+                digits_y(v[0].y, c9.x, yl[0][1], yh[0][1]);
+                digits_y(v[1].x, c9.y, yl[1][0], yh[1][0]);
+                digits_y(v[1].y, c9.y, yl[1][1], yh[1][1]);
+                digits_y(v[2].x, c9.z, yl[2][0], yh[2][0]);
+                digits_y(v[2].y, c9.z, yl[2][1], yh[2][1]);
+                digits_y(v[3].x, c9.w, yl[3][0], yh[3][0]);
+                digits_y(v[3].y, c9.w, yl[3][1], yh[3][1]);
+                if (kc + 1 < nk) load(tile, kc + 1);
+                else if (tile + tstep < ntiles) load(tile + tstep, 0);
+                uint4 b[NH / 2][NT];
+                const uint4* Bq = reinterpret_cast<const uint4*>(Bh) + (size_t)kc * (NH / 2) * NT * 32;
+#pragma unroll
+                for (int jp = 0; jp < NH / 2; ++jp)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) b[jp][j] = Bq[(jp * NT + j) * 32 + lane];
+                auto level = [&](auto ic) {
+                    constexpr int I = decltype(ic)::value;
+                    uint32_t a[4];
+                    a[0] = digit_pair<I>(yl[0][0], yh[0][0], yl[1][0], yh[1][0]);
+                    a[1] = digit_pair<I>(yl[0][1], yh[0][1], yl[1][1], yh[1][1]);
+                    a[2] = digit_pair<I>(yl[2][0], yh[2][0], yl[3][0], yh[3][0]);
+                    a[3] = digit_pair<I>(yl[2][1], yh[2][1], yl[3][1], yh[3][1]);
+#pragma unroll
+                    for (int jj = 0; jj < NH; ++jj)
+                        if (I + jj <= 6) {
+#pragma unroll
+                            for (int j = 0; j < NT; ++j) {
+                                const uint4 bq = b[jj >> 1][j];
+                                mma_f16(acc[I + jj][j], a, (jj & 1) ? bq.z : bq.x, (jj & 1) ? bq.w : bq.y);
+                            }
+                        }
+                };
+                level(std::integral_constant<int, 0>{});
+                level(std::integral_constant<int, 1>{});
+                level(std::integral_constant<int, 2>{});
+                level(std::integral_constant<int, 3>{});
+                level(std::integral_constant<int, 4>{});
+                level(std::integral_constant<int, 5>{});
+                level(std::integral_constant<int, 6>{});
+            }
+            if (k0 == 0) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int c = 8 * j + 2 * t + q;
+                        double2 x = make_double2(0.0, 0.0);
+                        if (c < p) {
+                            if (r + 1 < n) x = *reinterpret_cast<const double2*>(W + (int64_t)c * ldw + r);
+                            else if (r < n) x.x = W[(int64_t)c * ldw + r];
+                        }
+                        w[j][q] = x.x;
+                        w[j][2 + q] = x.y;
+                    }
+            }
+            // S = sum_l L_l 2^(-8 l) by Horner in a float pair; the product is S 2^(f - 14)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float sh = acc[6][j][q], sl = 0.f;
+#pragma unroll
+                    for (int l = 5; l >= 0; --l) {
+                        sh *= 0x1p-8f;
+                        sl *= 0x1p-8f;
+                        df_add(sh, sl, acc[l][j][q]);
+                    }
+                    const int k = fmax_s[8 * j + 2 * t + (q & 1)] - 14;
+                    const double x = scale2_e(f64_of_f32_i(sh), k), y = scale2_e(f64_of_f32_i(sl), k);
+                    w[j][q] = GS ? (w[j][q] - x) - y : (w[j][q] + x) + y;
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int c = 8 * j + 2 * t + q;
+                if (c < p) {
+                    double* dst = W + (int64_t)c * ldw + r;
+                    if (r + 1 < n) *reinterpret_cast<double2*>(dst) = make_double2(w[j][q], w[j][2 + q]);
+                    else if (r < n) *dst = w[j][q];
+                }
+            }
+        if (GS) {
+            // Gram entries of the tile's 16 rows (zero past n and p) from float pairs
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    float wh, wl;
+                    split_df_i(w[j][q], wh, wl);
+                    gw[(2 * g + (q >> 1)) * (NCOL + 1) + 8 * j + 2 * t + (q & 1)] = make_float2(wh, wl);
+                }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < GK; ++k)
+                if (gi[k] >= 0) {
+                    const float2* rowp = gw + (gi[k] >> 16) * (16 / GSP) * (NCOL + 1);
+                    const int i = (gi[k] >> 8) & 0xFF, j = gi[k] & 0xFF;
+                    float sh = 0.f, sl = 0.f;
+#pragma unroll 4
+                    for (int rr = 0; rr < 16 / GSP; ++rr) {
+                        const float2 x = rowp[rr * (NCOL + 1) + i], y = rowp[rr * (NCOL + 1) + j];
+                        df_fma(sh, sl, x.x, x.y, y.x, y.y);
+                    }
+                    df_add(gh[k], gl[k], sh);
+                    gl[k] += sl;
+                }
+        } else if (restart) {
+            __syncwarp();
+            const int64_t rr = tile * 16 + 2 * (lane & 7);
+            for (int c = lane >> 3; c < p; c += 4) {
+                const int64_t so = (int64_t)(cols - p + c) * ldv + rr, dof = (int64_t)c * ldv + rr;
+                *reinterpret_cast<double2*>(V + dof) = *reinterpret_cast<const double2*>(V + so);
+                *reinterpret_cast<float2*>(V32 + dof) = *reinterpret_cast<const float2*>(V32 + so);
+            }
+        }
+    }
+    if (GS) {
+        __syncthreads();
+        // the warps' pairs, then one FP64 value per entry
+        float2* red = gbuf;                                  // [k][warp][lane]
+#pragma unroll
+        for (int k = 0; k < GK; ++k)
+            if (32 * k < ne * GSP) red[(k * 4 + warp) * 32 + lane] = make_float2(gh[k], gl[k]);
+        __syncthreads();
+        double* out = partG + (int64_t)blockIdx.x * p * p;
+        for (int e = tid; e < p * p; e += kUpdThreads) {
+            int i = e / p, j = e % p;
+            if (i > j) {
+                const int x = i;
+                i = j;
+                j = x;
+            }
+            const int k = i * p - i * (i - 1) / 2 + (j - i);
+            float sh = 0.f, sl = 0.f;
+            for (int q = 0; q < GSP; ++q) {
+                const int it = q * ne + k;
+#pragma unroll
+                for (int wi = 0; wi < kUpdThreads / 32; ++wi) {
+                    const float2 x = red[((it >> 5) * 4 + wi) * 32 + (it & 31)];
+                    df_add(sh, sl, x.x);
+                    sl += x.y;
+                }
+            }
+            out[e] = f64_of_f32_i(sh) + f64_of_f32_i(sl);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- the FP32 copy and colexp
+// V32 and colexp of columns c0 .. c0 + p - 1 of V (blocks that no fused pass wrote: the first
+// block, Ritz vectors).  skip: the fused pass wrote them (device flag).
+__global__ void k_pack_block(const double* __restrict__ V, float* __restrict__ V32, int64_t ld, int64_t n,
+                             int* __restrict__ colexp, const int* skip) {
+    if (skip && *skip) return;
+    const int c = blockIdx.y;
+    unsigned mx = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double v = V[c * ld + i];
+        V32[c * ld + i] = f32_rn_i(v);
+        mx = max(mx, (unsigned)__double2hiint(v) & 0x7FFFFFFFu);
+    }
+    mx = __reduce_max_sync(kFull, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&colexp[c], (int)(mx >> 20));
+}
+
+__global__ void k_zero_int(int* p, int n, const int* skip) {
+    if (skip && *skip) return;
+    if ((int)threadIdx.x < n) p[threadIdx.x] = 0;
+}
+
+}  // namespace
+
+// h = V^T W partials: returns the number of partials (row groups) through nb
+cudaError_t launch_proj_mma(const float* V32, int64_t ldv, int cols, const double* W, int64_t ldw, int p, int64_t n,
+                            double* part, int max_blocks, int sms, int* nb, cudaStream_t s) {
+    const int mt = (cols + 15) / 16, NT = p <= 8 ? 1 : p <= 16 ? 2 : 4, MTW = NT == 1 ? 4 : 2;
+    int CG = 1;
+    while (CG < 8 && CG * MTW < mt) CG *= 2;
+    const int gy = (mt + CG * MTW - 1) / (CG * MTW);
+    const int64_t units = (n + 16 * kProjKb - 1) / (16 * kProjKb);
+    const int ctas_sm = NT * MTW <= 4 ? 2 : 1;
+    const int64_t gmax = std::max(1, std::min(max_blocks, ctas_sm * sms / gy));
+    const int64_t per = (units + gmax - 1) / gmax;         // units per CTA, the CTAs evenly loaded
+    const int gx = (int)((units + per - 1) / per);
+    *nb = gx;
+    const dim3 grid(gx, gy);
+    if (NT == 1) k_proj_mma<1, 4><<<grid, 256, proj_smem(1, 4), s>>>(V32, ldv, cols, W, ldw, p, n, part, CG);
+    else if (NT == 2) k_proj_mma<2, 2><<<grid, 256, proj_smem(2, 2), s>>>(V32, ldv, cols, W, ldw, p, n, part, CG);
+    else k_proj_mma<4, 2><<<grid, 256, proj_smem(4, 2), s>>>(V32, ldv, cols, W, ldw, p, n, part, CG);
+    return cudaGetLastError();
+}
+
+template <int NT, int NH, bool GS>
+static cudaError_t upd_launch(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n,
+                              const double* h, int* colexp, double* partG, double* H, int ldH, int hcol, int* flags,
+                              float* V32, int restart, int max_blocks, int sms, int* nb, cudaStream_t s) {
+    const size_t shm = upd_smem(cols, NT, NH, GS);
+    int per_sm = NT == 4 ? 2 : NT == 2 ? 3 : 4;
+    while (per_sm > 1 && shm * per_sm > 200 * 1024) --per_sm;
+    const int64_t tiles = (n + 15) / 16;
+    const int g = (int)std::min<int64_t>({(int64_t)per_sm * sms, (tiles + 3) / 4, (int64_t)max_blocks});
+    if (nb) *nb = g;
+    k_upd_mma<NT, NH, GS><<<g, kUpdThreads, shm, s>>>(V, ldv, cols, W, ldw, p, n, h, colexp, partG, H, ldH, hcol, flags,
+                                                      V32, restart);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,
+                           int* colexp, double* partG, double* H, int ldH, int hcol, int* flags, int max_blocks, int sms,
+                           int* nb, cudaStream_t s) {
+#define EXPM_UPD(NT) upd_launch<NT, 4, true>(V, ldv, cols, W, ldw, p, n, h, colexp, partG, H, ldH, hcol, flags, nullptr, 0, max_blocks, sms, nb, s)
+    return p <= 8 ? EXPM_UPD(1) : p <= 16 ? EXPM_UPD(2) : EXPM_UPD(4);
+#undef EXPM_UPD
+}
+
+cudaError_t launch_updz_mma(double* V, float* V32, int64_t ldv, int cols, double* Z, int64_t ldz, int p, int64_t n,
+                            const double* Wc, int* colexp, int* flags, int restart, int sms, cudaStream_t s) {
+#define EXPM_UPZ(NT) upd_launch<NT, 6, false>(V, ldv, cols, Z, ldz, p, n, Wc, colexp, nullptr, nullptr, 0, 0, flags, V32, restart, 1 << 20, sms, nullptr, s)
+    cudaError_t e = p <= 8 ? EXPM_UPZ(1) : p <= 16 ? EXPM_UPZ(2) : EXPM_UPZ(4);
+#undef EXPM_UPZ
+    if (e == cudaSuccess && restart)
+        e = cudaMemcpyAsync(colexp, colexp + cols - p, sizeof(int) * p, cudaMemcpyDeviceToDevice, s);
+    return e;
+}
+
+bool mma_fit(int mp, int p) {
+    const int NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
+    return p >= 1 && p <= kMaxP && upd_smem(mp, NT, 4, true) <= 220 * 1024 && upd_smem(mp + p, NT, 6, false) <= 220 * 1024;
+}
+
+cudaError_t launch_pack_block(const double* V, float* V32, int64_t ld, int64_t n, int p, int* colexp, const int* skip,
+                              cudaStream_t s) {
+    for (int c = 0; c < p; c += 1024) k_zero_int<<<1, 1024, 0, s>>>(colexp + c, std::min(1024, p - c), skip);
+    const int gx = (int)std::min<int64_t>((n + 255) / 256, 512);
+    k_pack_block<<<dim3(gx, p), 256, 0, s>>>(V, V32, ld, n, colexp, skip);
+    return cudaGetLastError();
+}
+
+cudaError_t mma_set_smem_limits() {
+    cudaError_t e = cudaSuccess;
+#define EXPM_SET(K) \
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024)
+    EXPM_SET((k_proj_mma<4, 2>));
+    EXPM_SET((k_upd_mma<1, 4, true>)); EXPM_SET((k_upd_mma<2, 4, true>)); EXPM_SET((k_upd_mma<4, 4, true>));
+    EXPM_SET((k_upd_mma<1, 6, false>)); EXPM_SET((k_upd_mma<2, 6, false>)); EXPM_SET((k_upd_mma<4, 6, false>));
+#undef EXPM_SET
+    return e;
+}
+
+}  // namespace expm

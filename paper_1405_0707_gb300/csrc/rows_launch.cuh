@@ -36,7 +36,8 @@ cudaError_t cgs(int upd, const double* V, int64_t ldv, int cols, double* W, int6
 cudaError_t qr(double* W, int64_t ldw, int p, int64_t n, int nblk, double* G, double* part, unsigned* ctr, int mode,
                double* R, double* Rinv, const double* Rtot_in, double* Rtot_out, double* H, int ldH, int hrow,
                int hcol, double* normsq_out, int* flags, double* out, int64_t ldo, cudaStream_t s, const double* Vc,
-               int64_t ldvc, int ccols, const double* h2, double* fin, int64_t ldfin) {
+               int64_t ldvc, int ccols, const double* h2, double* fin, int64_t ldfin, float* out32, int* colexp,
+               int skip_done) {
     if (p > RP) return cudaErrorInvalidValue;
     if (Vc && (mode != 0 || !h2 || ccols < 1 || ccols > kMaxMP)) return cudaErrorInvalidValue;
     const int64_t rpb = rows_per_block(n, nblk);
@@ -47,15 +48,15 @@ cudaError_t qr(double* W, int64_t ldw, int p, int64_t n, int nblk, double* G, do
     if (mode == 0 && Vc)
         k_qr_mixed_rows<3><<<g, NTR, 2 * sizeof(float) * (size_t)ccols * RP, s>>>(
             W, ldw, p, n, rpb, G, part, ctr, mode, R, Rinv, Rtot_in, Rtot_out, H, ldH, hrow, hcol, normsq_out,
-            flags, out, ldo, Vc, ldvc, ccols, h2, lead_blk, fin, ldfin);
+            flags, out, ldo, Vc, ldvc, ccols, h2, lead_blk, fin, ldfin, out32, colexp, skip_done);
     else if (mode == 0)
         k_qr_mixed_rows<1><<<g, NTR, 0, s>>>(W, ldw, p, n, rpb, G, part, ctr, mode, R, Rinv, Rtot_in, Rtot_out, H,
                                              ldH, hrow, hcol, normsq_out, flags, out, ldo, nullptr, 0, 0, nullptr,
-                                             lead_blk, nullptr, 0);
+                                             lead_blk, nullptr, 0, out32, colexp, skip_done);
     else
         k_qr_mixed_rows<2><<<g, NTR, 0, s>>>(W, ldw, p, n, rpb, G, part, ctr, mode, R, Rinv, Rtot_in, Rtot_out, H,
                                              ldH, hrow, hcol, normsq_out, flags, out, ldo, nullptr, 0, 0, nullptr,
-                                             lead_blk, nullptr, 0);
+                                             lead_blk, nullptr, 0, out32, colexp, skip_done);
     return cudaGetLastError();
 }
 

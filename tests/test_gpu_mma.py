@@ -1,0 +1,72 @@
+"""The register-streamed tensor-core passes of the mixed path (k_mma.cu, rows_qr.cuh), through the
+C ABI, against the CUDA-core row kernels and the oracle.
+
+The sizes cover each N-tile width (p <= 8, <= 16, <= 32) and its edges, bases that end inside a
+16-column chunk or pass the 240-column segment of the exact sums, row counts below one 16-row tile
+and ragged against 16, 32 and 128 rows, and starting blocks that are localised (unit vectors, one
+digit scale for every column) or spread out.
+
+Tolerances, from the arithmetic: W - V h is exact to 2^-55 of each column's largest entry and the
+forward substitution to ~2^-48 per product with the factor's condition below 300, so the relation
+(tA)^{-1} V_m = V_{m+1} H~_m holds to 1e-12 relative; the projections carry 2^-25 per product, so
+orthogonality and the agreement of H~ with the CUDA-core passes stay at FP32 level (1e-5, 1e-6, the
+bounds of those passes' own tests).
+"""
+import numpy as np
+import pytest
+
+from oracle import cf, operators as ops, psbfom as ps
+from paper_1405_0707_gb300 import inputs
+from tests.gpu_util import need_gpu, rel, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+def _arnoldi(sides, p, m, V1, t):
+    from paper_1405_0707_gb300 import Plan
+    vel = (1.0, -0.5, 0.3)[:len(sides)]
+    plan = Plan(sides, 0.1, vel, p_max=p, m=m, precision="mixed")
+    Vg, Hg = plan.arnoldi(t, to_dev(V1))
+    W = np.column_stack([to_np(plan.prec_apply(t, Vg[:, j * p:(j + 1) * p])) for j in range(m)])
+    out = to_np(Vg), to_np(Hg), W
+    plan.close()
+    return out
+
+
+@pytest.mark.parametrize("local", [False, True])
+@pytest.mark.parametrize("sides,p,m", [((13,), 1, 3), ((47, 3), 3, 8), ((61, 59), 8, 10), ((33, 31, 29), 9, 5),
+                                       ((97, 83), 16, 10), ((64, 40), 17, 6), ((130, 65), 32, 10), ((40, 41), 24, 3),
+                                       ((70, 66), 16, 30), ((129, 127), 1, 40)])
+def test_relation_orthogonality_and_h(sides, p, m, local, monkeypatch):
+    need_gpu()
+    n, t = int(np.prod(sides)), 0.05
+    if local:
+        V1 = np.zeros((n, p), order="F")
+        V1[np.linspace(0, n - 1, p).astype(int), np.arange(p)] = 1.0
+    else:
+        V1, _ = ps.qr_positive(inputs.rhs(n, p, 8))
+    V, H, W = _arnoldi(sides, p, m, V1, t)
+    assert np.linalg.norm(W - V @ H) <= 1e-12 * np.linalg.norm(W)
+    assert np.linalg.norm(V.T @ V - np.eye((m + 1) * p)) <= 1e-5
+    monkeypatch.setenv("EXPM_CGS_TC", "0")
+    Hr = _arnoldi(sides, p, m, V1, t)[1]
+    k = p * min(m, 6)       # later columns amplify either side's FP32-level differences
+    assert np.linalg.norm(H[:, :k] - Hr[:, :k]) <= 1e-6 * np.linalg.norm(Hr[:, :k])
+
+
+@pytest.mark.parametrize("sides,p,t", [((256, 256), 8, 0.1), ((90, 77), 32, 0.03), ((40, 37, 35), 13, 0.02),
+                                       ((300,), 5, 0.1)])
+@pytest.mark.parametrize("repeated", [False, True])
+def test_converged_solve_matches_closed_form(sides, p, t, repeated):
+    """repeated: equal right-hand-side columns, which keep every block on the fallback passes."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    n, d = int(np.prod(sides)), len(sides)
+    diff, vel = (0.1, (1.0, 1.0)) if d == 2 else (1.0, (2.0, -1.0, 1.5)[:d])
+    B = inputs.rhs(n, p, 44)
+    if repeated:
+        B[:, -1] = B[:, 0]
+    Z, info = Plan(sides, diff, vel, p_max=p, m=10, tol=1e-11, max_cycles=400, precision="mixed").expm_block(t, to_dev(B))
+    assert info.converged == 1
+    ref = ops.exact_r_of_A_B(sides, diff, vel, t, cf.load_table(), B)
+    assert rel(to_np(Z), ref) <= 1e-9, rel(to_np(Z), ref)
