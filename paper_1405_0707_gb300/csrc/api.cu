@@ -135,36 +135,33 @@ expm_status qr_block(expm_plan* P, int p, double* out, int64_t ldo, bool withH, 
     return EXPM_OK;
 }
 
-// One FP32 application of (tA)^{-1} to R (FP64 in), written (acc = 0) or added (acc = 1)
-// to X (FP64).  Same transforms and layouts as the FP64 path.
-expm_status inv32_apply(expm_plan* P, double t, const void* R, int64_t ldr, int p, double* X,
-                        int64_t ldx, int acc, int r_f64 = 1) {
+// One FP32 application of (tA)^{-1} to R (FP32), written (acc = 0) or added (acc = 1) to X (FP64).
+// Same transforms and layouts as the FP64 path.
+expm_status inv32_apply(expm_plan* P, double t, const float* R, int64_t ldr, int p, double* X,
+                        int64_t ldx, int acc) {
     cudaStream_t s = P->stream;
     const int nx = P->ax[0].N, ny = P->ax[1].N, nz = P->ax[2].N;
     const int64_t ld = P->ld;
     const float lsub = (float)P->ax[0].l, inv_t = (float)(1.0 / t);
     if (P->ndim == 2) {
-        GemmArgsMixed g1{R, P->Qf32[1], P->T1f, nx, ny, ny, 1, nx, ldr, 0, ny, 1, ld, 0, ny, p, 1, r_f64, 0, 0};
-        LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g1, s));
+        const TransformArgs g1{R, P->QfF[1], P->T1f, nx, ny, ny, 1, nx, ldr, ny, 1, ld, 0, 0};
+        LAUNCH(EXPM_STAGE_GEMM, launch_transform(g1, p, P->sms, s));
         LAUNCH(EXPM_STAGE_TRIDIAG, launch_tridiag_lines32(P->T1f, ld, p, nx, ny, lsub, P->th_m32, P->th_c32, inv_t, s));
-        GemmArgsMixed g2{P->T1f, P->Qi32[1], X, nx, ny, ny, ny, 1, ld, 0, 1, nx, ldx, 0, ny, p, 1, 0, 1, acc};
-        LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g2, s));
+        const TransformArgs g2{P->T1f, P->QiF[1], X, nx, ny, ny, ny, 1, ld, 1, nx, ldx, 1, acc};
+        LAUNCH(EXPM_STAGE_GEMM, launch_transform(g2, p, P->sms, s));
         return EXPM_OK;
     }
-    const int64_t nxy = (int64_t)nx * ny;
-    GemmArgsMixed g1{R, P->Qf32[2], P->T2f, (int)nxy, nz, nz, 1, nxy, ldr, 0, 1, nxy, ld, 0, nz, p, 1, r_f64, 0, 0};
-    LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g1, s));
+    const int64_t nxy = (int64_t)nx * ny, nyz = (int64_t)ny * nz;
+    const TransformArgs g1{R, P->QfF[2], P->T2f, (int)nxy, nz, nz, 1, nxy, ldr, 1, nxy, ld, 0, 0};
+    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g1, p, P->sms, s));
     // the y transforms take (x, z) as one row index of nx nz rows (no padding per x line)
-    GemmArgsMixed g2{P->T2f, P->Qf32[1], P->T1f, nx * nz, ny, ny, 1, nx, ld, 0, (int64_t)ny * nz, 1, ld, 0, ny, p, 1,
-                     0, 0, 0, nx, nxy, ny};
-    LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g2, s));
-    LAUNCH(EXPM_STAGE_TRIDIAG, launch_tridiag_lines32(P->T1f, ld, p, nx, (int64_t)ny * nz, lsub, P->th_m32,
-                                                      P->th_c32, inv_t, s));
-    GemmArgsMixed g3{P->T1f, P->Qi32[1], P->T2f, nx * nz, ny, ny, (int64_t)ny * nz, 1, ld, 0, 1, nx, ld, 0, ny, p, 1,
-                     0, 0, 0, nx, ny, nxy};
-    LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g3, s));
-    GemmArgsMixed g4{P->T2f, P->Qi32[2], X, (int)nxy, nz, nz, 1, nxy, ld, 0, 1, nxy, ldx, 0, nz, p, 1, 0, 1, acc};
-    LAUNCH(EXPM_STAGE_GEMM, launch_gemm32(g4, s));
+    const TransformArgs g2{P->T2f, P->QfF[1], P->T1f, nx * nz, ny, ny, 1, nx, ld, nyz, 1, ld, 0, 0, nx, nxy, ny};
+    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g2, p, P->sms, s));
+    LAUNCH(EXPM_STAGE_TRIDIAG, launch_tridiag_lines32(P->T1f, ld, p, nx, nyz, lsub, P->th_m32, P->th_c32, inv_t, s));
+    const TransformArgs g3{P->T1f, P->QiF[1], P->T2f, nx * nz, ny, ny, nyz, 1, ld, 1, nx, ld, 0, 0, nx, ny, nxy};
+    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g3, p, P->sms, s));
+    const TransformArgs g4{P->T2f, P->QiF[2], X, (int)nxy, nz, nz, 1, nxy, ld, 1, nxy, ldx, 1, acc};
+    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g4, p, P->sms, s));
     return EXPM_OK;
 }
 
@@ -172,18 +169,23 @@ expm_status inv32_apply(expm_plan* P, double t, const void* R, int64_t ldr, int 
 // inverse: x_0 = inv32(V), x_{k+1} = x_k + inv32(V - tA x_k) with the residual in FP64
 // (Theorem 4.3: the inverse's accuracy is what the shifted solutions inherit).  Each step
 // multiplies the backward error by about eps_32 * rho^-N (diagonal similarity).
+// V32, when given, is V's FP32 copy (leading dimension P->ld), which the first transform reads.
 expm_status prec_apply_mixed(expm_plan* P, double t, const double* V, int64_t ldv, int p,
-                             double* W, int64_t ldw) {
+                             double* W, int64_t ldw, const float* V32) {
     cudaStream_t s = P->stream;
-    expm_status st = inv32_apply(P, t, V, ldv, p, W, ldw, 0);
+    float* R32 = reinterpret_cast<float*>(P->R64);
+    if (!V32) {
+        LAUNCH(EXPM_STAGE_GEMM, launch_d2f(V, R32, P->n, s, ldv, P->ld, p));
+        V32 = R32;
+    }
+    expm_status st = inv32_apply(P, t, V32, P->ld, p, W, ldw, 0);
     if (st != EXPM_OK) return st;
     for (int k = 0; k < P->refine; ++k) {
         // the residual V - tA x in FP64, stored in FP32 (the R64 buffer): the transforms read
         // it as FP32 either way
-        float* R32 = reinterpret_cast<float*>(P->R64);
         LAUNCH(EXPM_STAGE_STENCIL, launch_cd_apply(W, ldw, nullptr, P->ld, p, P->ndim, P->ax[0].N, P->ax[1].N,
                                                    P->ax[2].N, P->ax, -t, s, V, ldv, 1.0, R32, P->stencil_df & 2));
-        st = inv32_apply(P, t, R32, P->ld, p, W, ldw, 1, 0);
+        st = inv32_apply(P, t, R32, P->ld, p, W, ldw, 1);
         if (st != EXPM_OK) return st;
     }
     return EXPM_OK;
@@ -288,7 +290,7 @@ expm_status op_apply_internal(expm_plan* P, double t, const double* V, int64_t l
 }
 
 expm_status prec_apply_internal(expm_plan* P, double t, const double* V, int64_t ldv, int p,
-                                double* W, int64_t ldw) {
+                                double* W, int64_t ldw, const float* V32 = nullptr) {
     cudaStream_t s = P->stream;
     if (P->toeplitz) {
         if (!P->tz.gsf) return EXPM_INVALID_ARG;
@@ -305,7 +307,7 @@ expm_status prec_apply_internal(expm_plan* P, double t, const double* V, int64_t
         P->inner_iters += iters;
         return conv ? EXPM_OK : EXPM_NOT_CONVERGED;
     }
-    if (P->opts.precision == EXPM_PREC_MIXED && P->ndim > 1) return prec_apply_mixed(P, t, V, ldv, p, W, ldw);
+    if (P->opts.precision == EXPM_PREC_MIXED && P->ndim > 1) return prec_apply_mixed(P, t, V, ldv, p, W, ldw, V32);
     const double inv_t = 1.0 / t;
     const int nx = P->ax[0].N, ny = P->ax[1].N, nz = P->ax[2].N;
     const int64_t ld = P->ld;
@@ -393,7 +395,8 @@ expm_status block_step(expm_plan* P, double t, int j, int p, int alg) {
     double* h = sm(P, kOffH);
     const double* Vj = P->V + (int64_t)j * p * ld;
     if (alg == 2) {
-        expm_status st = prec_apply_internal(P, t, Vj, ld, p, P->W, ld);
+        expm_status st = prec_apply_internal(P, t, Vj, ld, p, P->W, ld,
+                                             P->mma ? P->V32 + (int64_t)j * p * ld : nullptr);
         if (st != EXPM_OK) return st;
     } else {
         expm_status st = op_apply_internal(P, t, Vj, ld, p, P->W, ld);
@@ -811,8 +814,8 @@ void free_plan(expm_plan* P) {
     cudaFree(P->th_m);
     cudaFree(P->th_c);
     for (int d = 0; d < 3; ++d) {
-        cudaFree(P->Qf32[d]);
-        cudaFree(P->Qi32[d]);
+        cudaFree(P->QfF[d]);
+        cudaFree(P->QiF[d]);
     }
     cudaFree(P->th_m32);
     cudaFree(P->th_c32);
@@ -1511,7 +1514,7 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         if (mixed) {
             for (int d = 1; d < P->ndim; ++d) {
                 const int N = P->ax[d].N;
-                ok = ok && dalloc(&P->Qf32[d], (size_t)N * N) && dalloc(&P->Qi32[d], (size_t)N * N);
+                ok = ok && dalloc(&P->QfF[d], table_frag_count(N)) && dalloc(&P->QiF[d], table_frag_count(N));
             }
             ok = ok && dalloc(&P->th_m32, (size_t)P->ax[0].N * nmodes) &&
                  dalloc(&P->th_c32, (size_t)P->ax[0].N * nmodes);
@@ -1534,7 +1537,7 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
     cudaStream_t s = P->stream;
     bool cuda_ok = krylov_set_smem_limits() == cudaSuccess && poles_set_smem_limits() == cudaSuccess &&
                    operator_set_smem_limits() == cudaSuccess && cgs_tc_set_smem_limits() == cudaSuccess &&
-                   mma_set_smem_limits() == cudaSuccess;
+                   mma_set_smem_limits() == cudaSuccess && transform_set_smem() == cudaSuccess;
     if (csr && cuda_ok) {
         CsrOp& c = P->cs;
         cuda_ok = cudaMemcpyAsync(c.rowptr, op->csr_rowptr, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice, s) == cudaSuccess &&
@@ -1553,9 +1556,8 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
                                           P->ndim > 2 ? P->lam[2] : nullptr, P->ax[2].N, s) == cudaSuccess;
         if (cuda_ok && mixed) {
             for (int d = 1; d < P->ndim && cuda_ok; ++d) {
-                const int64_t NN = (int64_t)P->ax[d].N * P->ax[d].N;
-                cuda_ok = launch_d2f(P->Qf[d], P->Qf32[d], NN, s) == cudaSuccess &&
-                          launch_d2f(P->Qi[d], P->Qi32[d], NN, s) == cudaSuccess;
+                cuda_ok = launch_table_frags(P->Qf[d], P->ax[d].N, P->QfF[d], s) == cudaSuccess &&
+                          launch_table_frags(P->Qi[d], P->ax[d].N, P->QiF[d], s) == cudaSuccess;
             }
             const int64_t nt = (int64_t)P->ax[0].N * nmodes;
             if (cuda_ok)

@@ -32,18 +32,17 @@ struct GemmArgs {
     int nb1, nb2;
 };
 
-// Mixed-precision variant: A and C may be FP64 or FP32 (a_f64 / c_f64), B is FP32,
-// arithmetic FP32; accumulate != 0 adds into C.
-struct GemmArgsMixed {
-    const void* A;
-    const float* B;
+// One sine transform of the mixed path (k_transform.cu), per block column b: C[m, n] = sum_k A[m, k]
+// Q[k, n] in FP32 accuracy; A FP32, C FP32 or FP64 (c_f64), element (m, k) of A at a_b b + m a_rs +
+// k a_cs; accumulate != 0 adds into an FP64 C.
+struct TransformArgs {
+    const float* A;
+    const uint4* Q;      // the table in fragment order (launch_table_frags)
     void* C;
     int M, N, K;
-    int64_t a_rs, a_cs, a_b1, a_b2;
-    int64_t c_rs, c_cs, c_b1, c_b2;
-    int ldb;
-    int nb1, nb2;
-    int a_f64, c_f64, accumulate;
+    int64_t a_rs, a_cs, a_b;
+    int64_t c_rs, c_cs, c_b;
+    int c_f64, accumulate;
     // ms > 0: the row index m is a pair (m % ms, m / ms) with strides (a_rs, a_ms2) in A and
     // (c_rs, c_ms2) in C, so two grid axes form one long M dimension (no padding per line)
     int ms = 0;
@@ -180,8 +179,8 @@ struct expm_plan_s {
     double* th_c = nullptr;                          // Thomas c',      [x * nmodes + mode]
     int64_t nmodes = 1;
     // mixed precision: FP32 copies of the tables and FP32 transform buffers
-    float* Qf32[3] = {nullptr, nullptr, nullptr};
-    float* Qi32[3] = {nullptr, nullptr, nullptr};
+    uint4* QfF[3] = {nullptr, nullptr, nullptr};   // Qf, Qi split for the tensor cores, fragment order
+    uint4* QiF[3] = {nullptr, nullptr, nullptr};
     float* th_m32 = nullptr;
     float* th_c32 = nullptr;
     float* T1f = nullptr;      // ld x p_max
@@ -273,11 +272,15 @@ cudaError_t launch_cd_apply(const double* V, int64_t ldv, double* W, int64_t ldw
                             int ndim, int nx, int ny, int nz, const Axis* ax, double t,
                             cudaStream_t s, const double* Y = nullptr, int64_t ldy = 0,
                             double beta = 0.0, float* W32 = nullptr, int df = 0);
-cudaError_t launch_gemm32(const GemmArgsMixed& g, cudaStream_t s);
+size_t table_frag_count(int N);
+cudaError_t launch_table_frags(const double* Q, int N, uint4* F, cudaStream_t s);
+cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s);
+cudaError_t transform_set_smem();
 cudaError_t launch_tridiag_lines32(float* y, int64_t ld, int p, int L, int64_t nmodes, float l_sub,
                                    const float* th_m, const float* th_c, float inv_t,
                                    cudaStream_t s);
-cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s);
+cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, int64_t ldin = 0, int64_t ldout = 0,
+                       int cols = 1);
 
 // block Gram-Schmidt / Cholesky-QR pieces
 cudaError_t launch_proj_partial(const double* V, int64_t ldv, int cols, const double* W,

@@ -115,6 +115,8 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
     };
     int64_t u = blockIdx.x;
     float4 v[MTW][2];
+#pragma unroll
+    for (int i = 0; i < MTW; ++i) v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);   // tiles past nmt
     int buf = 0;
     if (u < units) {
         loadw(u);
@@ -139,31 +141,36 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
             for (int j = 0; j < NT; ++j)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) wb[j][k] = wq[(j * 3 + k) * 32];
+            // two M tiles at a time: their splits, the next block's loads, then the products
+            // interleaved over the tiles and N tiles
 #pragma unroll
-            for (int i = 0; i < MTW; ++i)
-                if (i < nmt) {
-                    uint32_t a[3][4];
-                    {
+            for (int i0 = 0; i0 < MTW; i0 += 2)
+                if (i0 < nmt) {
+                    uint32_t a[2][3][4];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const float4 x = v[i0 + i][0], y = v[i0 + i][1];
                         uint32_t s[3];
-                        split3(v[i][0].x, v[i][0].y, s);
-                        a[0][0] = s[0]; a[1][0] = s[1]; a[2][0] = s[2];
-                        split3(v[i][1].x, v[i][1].y, s);
-                        a[0][1] = s[0]; a[1][1] = s[1]; a[2][1] = s[2];
-                        split3(v[i][0].z, v[i][0].w, s);
-                        a[0][2] = s[0]; a[1][2] = s[1]; a[2][2] = s[2];
-                        split3(v[i][1].z, v[i][1].w, s);
-                        a[0][3] = s[0]; a[1][3] = s[1]; a[2][3] = s[2];
+                        split3(x.x, x.y, s);
+                        a[i][0][0] = s[0]; a[i][1][0] = s[1]; a[i][2][0] = s[2];
+                        split3(y.x, y.y, s);
+                        a[i][0][1] = s[0]; a[i][1][1] = s[1]; a[i][2][1] = s[2];
+                        split3(x.z, x.w, s);
+                        a[i][0][2] = s[0]; a[i][1][2] = s[1]; a[i][2][2] = s[2];
+                        split3(y.z, y.w, s);
+                        a[i][0][3] = s[0]; a[i][1][3] = s[1]; a[i][2][3] = s[2];
                     }
-                    if (more) loadv(v[i], i, bn);
 #pragma unroll
-                    for (int j = 0; j < NT; ++j) {
-                        mma_bf16(cc[i][j], a[2], wb[j][0].x, wb[j][0].y);
-                        mma_bf16(cm[i][j], a[0], wb[j][0].x, wb[j][0].y);
-                        mma_bf16(cc[i][j], a[0], wb[j][2].x, wb[j][2].y);
-                        mma_bf16(cc[i][j], a[1], wb[j][1].x, wb[j][1].y);
-                        mma_bf16(cc[i][j], a[1], wb[j][0].x, wb[j][0].y);
-                        mma_bf16(cc[i][j], a[0], wb[j][1].x, wb[j][1].y);
-                    }
+                    for (int i = 0; i < 2; ++i)
+                        if (more && i0 + i < nmt) loadv(v[i0 + i], i0 + i, bn);
+#pragma unroll
+                    for (int pr = 0; pr < 6; ++pr)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int j = 0; j < NT; ++j)
+                                mma_bf16(pr == 0 ? cm[i0 + i][j] : cc[i0 + i][j], a[i][kProdA[pr]], wb[j][kProdB[pr]].x,
+                                         wb[j][kProdB[pr]].y);
                 }
         }
 #pragma unroll

@@ -330,251 +330,8 @@ __global__ void k_cd_apply_df(const double* __restrict__ V, int64_t ldv, double*
 }
 
 // ---------------------------------------------------------------- mixed precision
-// FP32 arithmetic for the DST-I transforms of the exact inverse; the result is refined
-// in FP64 by the caller (residual with the FP64 stencil, Theorem 4.3 bounds what an
-// inexact inverse costs).  TA / TC: element types of A and C; acc: C += A B.
-constexpr int BK32 = 32;   // k-depth of one FP32 tile
-
-// FP32 tiles of 64 x 64 outputs, 4 x 4 per thread; the next k-tile's global loads are
-// issued into registers before the current tile's FMAs (software pipelining), so each
-// barrier round overlaps its loads with arithmetic.  FP64 operands are converted from the
-// bit pattern (f32_rn_i) and FP64 results formed with an exact float -> double widening,
-// keeping the transforms off GB300's FP64 pipe except for the one accumulating add.
-__device__ __forceinline__ int64_t gemm_row_off(int m, int ms, int64_t rs, int64_t ms2) {
-    return ms ? (int64_t)(m % ms) * rs + (int64_t)(m / ms) * ms2 : (int64_t)m * rs;
-}
-
-__device__ __forceinline__ float gemm_in(double x) { return f32_rn_i(x); }
-__device__ __forceinline__ float gemm_in(float x) { return x; }
-
-template <typename TC>
-__device__ __forceinline__ void gemm_out(TC* dst, float v, int acc) {
-    if constexpr (sizeof(TC) == 8) *dst = acc ? *dst + f64_of_f32_i(v) : f64_of_f32_i(v);
-    else *dst = acc ? *dst + v : v;
-}
-
-template <bool CM, typename TA, typename TC>
-__global__ void __launch_bounds__(256) k_gemm32(GemmArgsMixed g) {
-    // rows padded to BM + 4 floats: 16-byte aligned rows for the float4 operand loads
-    __shared__ __align__(16) float As[BK32][BM + 4];
-    __shared__ __align__(16) float Bs[BK32][BN];
-    const int b1 = blockIdx.z % g.nb1, b2 = blockIdx.z / g.nb1;
-    const TA* A = reinterpret_cast<const TA*>(g.A) + b1 * g.a_b1 + b2 * g.a_b2;
-    TC* C = reinterpret_cast<TC*>(g.C) + b1 * g.c_b1 + b2 * g.c_b2;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const bool a_mfast = (g.a_rs == 1);
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    constexpr int NQ = BK32 * BM / 256;   // elements of each tile per thread (8)
-    // A-row offset of each of this thread's fetched elements (-1 past M), fixed over k
-    int64_t aoff[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int e = tid + q * 256;
-        const int gm = m0 + (a_mfast ? e % BM : e / BK32);
-        aoff[q] = gm < g.M ? gemm_row_off(gm, g.ms, g.a_rs, g.a_ms2) : -1;
-    }
-    float ra[NQ], rb[NQ];
-    auto fetch = [&](int k0) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int e = tid + q * 256;
-            const int gk = k0 + (a_mfast ? e / BM : e % BK32);
-            ra[q] = (aoff[q] >= 0 && gk < g.K) ? gemm_in(A[aoff[q] + (int64_t)gk * g.a_cs]) : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int e = tid + q * 256;
-            const int nn = e % BN, kk = e / BN;
-            const int gn = n0 + nn, gk = k0 + kk;
-            rb[q] = (gn < g.N && gk < g.K) ? g.B[(int64_t)gk * g.ldb + gn] : 0.f;
-        }
-    };
-    fetch(0);
-    for (int k0 = 0; k0 < g.K; k0 += BK32) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int e = tid + q * 256;
-            int mm, kk;
-            if (a_mfast) { mm = e % BM; kk = e / BM; }
-            else { kk = e % BK32; mm = e / BK32; }
-            As[kk][mm] = ra[q];
-            Bs[e / BN][e % BN] = rb[q];
-        }
-        __syncthreads();
-        if (k0 + BK32 < g.K) fetch(k0 + BK32);
-        // each thread owns 4 consecutive rows m and 4 consecutive columns n: one float4 load
-        // per operand per k (the fastest-varying thread index walks C's contiguous dimension)
-        const int mi = 4 * (CM ? tx : ty), nj = 4 * (CM ? ty : tx);
-#pragma unroll
-        for (int kk = 0; kk < BK32; ++kk) {
-            const float4 av = *reinterpret_cast<const float4*>(&As[kk][mi]);
-            const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][nj]);
-            const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    const int mi = 4 * (CM ? tx : ty), nj = 4 * (CM ? ty : tx);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + mi + i;
-        if (m >= g.M) continue;
-        TC* crow = C + gemm_row_off(m, g.ms, g.c_rs, g.c_ms2);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int nn = n0 + nj + j;
-            if (nn < g.N) gemm_out(crow + (int64_t)nn * g.c_cs, acc[i][j], g.accumulate);
-        }
-    }
-}
-
-// Transforms along a short axis (K, N <= 96: every axis of the 3-D grids): the whole K x N
-// DST matrix and a slab of SBM rows of A (all K) sit in shared memory, so one barrier
-// separates staging from arithmetic and no k-tile padding is read.  A thread owns 8 rows
-// (two runs of 4 consecutive rows, 64 apart) and NJ columns (16 apart): per k two float4 of
-// A and NJ floats of B feed 8 NJ FMAs.  The row runs (CM: C's contiguous dimension is m) or
-// the columns (otherwise) walk consecutive threads, so the stores coalesce.
-constexpr int SBM = 128, SMAX = 96;
-constexpr int SAS = SBM + 4;   // row stride of the staged A (float4-aligned)
-
-// one 4-byte asynchronous global -> shared copy (zero-filled when !ok: no bytes are read,
-// and src is then any valid address)
-__device__ __forceinline__ void cp_async4(float* dst, const float* src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-                 "l"(src), "r"(ok ? 4 : 0)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__host__ __device__ constexpr size_t gemm_small_smem(int K, int NJ) {
-    return sizeof(float) * ((size_t)K * 16 * NJ + (size_t)K * SAS);
-}
-
-template <bool CM, typename TA, typename TC, int NJ>
-__global__ void __launch_bounds__(256) k_gemm_small(GemmArgsMixed g) {
-    extern __shared__ __align__(16) float sgm[];
-    constexpr int NP = 16 * NJ;
-    const int K = g.K;
-    float* Bs = sgm;                  // K x NP, columns past N zero
-    float* As = Bs + K * NP;          // K x SAS: As[k * SAS + mm]
-    const int b1 = blockIdx.y % g.nb1, b2 = blockIdx.y / g.nb1;
-    const TA* A = reinterpret_cast<const TA*>(g.A) + b1 * g.a_b1 + b2 * g.a_b2;
-    TC* C = reinterpret_cast<TC*>(g.C) + b1 * g.c_b1 + b2 * g.c_b2;
-    const int m0 = blockIdx.x * SBM, tid = threadIdx.x;
-    // staging: every float operand is copied with cp.async, so all of a thread's copies are in
-    // flight at once and the CTA waits for one round trip; an FP64 A is converted on the way
-    // and goes through registers, in batches of loads issued before any is stored
-    for (int e = tid; e < K * NP; e += 256) {
-        const int k = e / NP, n = e - k * NP;
-        const bool ok = n < g.N;
-        cp_async4(Bs + e, ok ? g.B + (int64_t)k * g.ldb + n : g.B, ok);
-    }
-    if constexpr (sizeof(TA) == 4) {
-        if (g.a_rs == 1) {
-            const int mm = tid & (SBM - 1), m = m0 + mm;
-            const bool ok = m < g.M;
-            const int64_t ro = ok ? gemm_row_off(m, g.ms, g.a_rs, g.a_ms2) : 0;
-            for (int k = tid >> 7; k < K; k += 2)
-                cp_async4(As + k * SAS + mm, ok ? (const float*)A + ro + (int64_t)k * g.a_cs : (const float*)A, ok);
-        } else {
-            const int warp = tid >> 5, lane = tid & 31;
-            for (int mm0 = warp; mm0 < SBM; mm0 += 32)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int m = m0 + mm0 + 8 * r;
-                    const bool ok = m < g.M;
-                    const int64_t ro = ok ? gemm_row_off(m, g.ms, g.a_rs, g.a_ms2) : 0;
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const int k = lane + 32 * j;
-                        if (k < K)
-                            cp_async4(As + k * SAS + mm0 + 8 * r,
-                                      ok ? (const float*)A + ro + (int64_t)k * g.a_cs : (const float*)A, ok);
-                    }
-                }
-        }
-    } else if (g.a_rs == 1) {
-        // m fastest in memory: thread t keeps row mm = t % SBM (one row offset) and walks k
-        const int mm = tid & (SBM - 1), m = m0 + mm;
-        const bool ok = m < g.M;
-        const int64_t ro = ok ? gemm_row_off(m, g.ms, g.a_rs, g.a_ms2) : 0;
-        for (int k0 = tid >> 7; k0 < K; k0 += 16) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int k = k0 + 2 * u;
-                v[u] = (ok && k < K) ? gemm_in(A[ro + (int64_t)k * g.a_cs]) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (k0 + 2 * u < K) As[(k0 + 2 * u) * SAS + mm] = v[u];
-        }
-    } else {
-        // k fastest in memory: a warp takes 4 rows at a time, lane l the entries k = l + 32 j
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int mm0 = warp; mm0 < SBM; mm0 += 32) {
-            float v[4][3];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int m = m0 + mm0 + 8 * r;
-                const bool ok = m < g.M;
-                const int64_t ro = ok ? gemm_row_off(m, g.ms, g.a_rs, g.a_ms2) : 0;
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const int k = lane + 32 * j;
-                    v[r][j] = (ok && k < K) ? gemm_in(A[ro + (int64_t)k * g.a_cs]) : 0.f;
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (lane + 32 * j < K) As[(lane + 32 * j) * SAS + mm0 + 8 * r] = v[r][j];
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    const int tm = CM ? (tid & 15) : (tid >> 4), tn = CM ? (tid >> 4) : (tid & 15);
-    float acc[8][NJ];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
-    const float* ap = As + 4 * tm;
-    const float* bp = Bs + tn;
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-        const float4 a0 = *reinterpret_cast<const float4*>(ap + k * SAS);
-        const float4 a1 = *reinterpret_cast<const float4*>(ap + k * SAS + 64);
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        float b[NJ];
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) b[j] = bp[k * NP + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int m = m0 + 4 * tm + (i & 3) + 64 * (i >> 2);
-        if (m >= g.M) continue;
-        TC* crow = C + gemm_row_off(m, g.ms, g.c_rs, g.c_ms2);
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int n = tn + 16 * j;
-            if (n < g.N) gemm_out(crow + (int64_t)n * g.c_cs, acc[i][j], g.accumulate);
-        }
-    }
-}
-
+// FP32 line solves of the exact inverse (its transforms are in k_transform.cu); the result is refined in
+// FP64 by the caller (residual with the FP64 stencil, Theorem 4.3 bounds what an inexact inverse costs).
 // The FP32 line solves with the lines staged in shared memory: a CTA takes TK consecutive
 // modes of one column (16 x L values of f, thm and thc, loaded once with coalesced reads),
 // runs the same segmented affine scans as tridiag_seg from shared memory and writes y back.
@@ -823,9 +580,9 @@ __global__ void k_true_resid(const double* __restrict__ X, int64_t ldx, const do
     if (threadIdx.x == 0) part[(int64_t)pole * gridDim.x + blockIdx.x] = red[0];
 }
 
-__global__ void k_d2f(const double* __restrict__ in, float* __restrict__ out, int64_t n) {
+__global__ void k_d2f(const double* __restrict__ in, float* __restrict__ out, int64_t n, int64_t ldin, int64_t ldout) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = (float)in[i];
+    if (i < n) out[blockIdx.y * ldout + i] = f32_rn_i(in[blockIdx.y * ldin + i]);
 }
 
 }  // namespace
@@ -895,51 +652,6 @@ cudaError_t launch_cd_apply(const double* V, int64_t ldv, double* W, int64_t ldw
     return cudaGetLastError();
 }
 
-template <typename TA, typename TC, int NJ>
-static void launch_gemm_small_nj(const GemmArgsMixed& g, bool cm, cudaStream_t s) {
-    const dim3 grid((unsigned)((g.M + SBM - 1) / SBM), (unsigned)(g.nb1 * g.nb2));
-    const size_t shm = gemm_small_smem(g.K, NJ);
-    if (cm) k_gemm_small<true, TA, TC, NJ><<<grid, 256, shm, s>>>(g);
-    else k_gemm_small<false, TA, TC, NJ><<<grid, 256, shm, s>>>(g);
-}
-
-template <typename TA, typename TC>
-static void launch_gemm_small_t(const GemmArgsMixed& g, bool cm, cudaStream_t s) {
-    const int nj = (g.N + 15) / 16;
-    if (nj <= 2) launch_gemm_small_nj<TA, TC, 2>(g, cm, s);
-    else if (nj == 3) launch_gemm_small_nj<TA, TC, 3>(g, cm, s);
-    else if (nj == 4) launch_gemm_small_nj<TA, TC, 4>(g, cm, s);
-    else if (nj == 5) launch_gemm_small_nj<TA, TC, 5>(g, cm, s);
-    else launch_gemm_small_nj<TA, TC, 6>(g, cm, s);
-}
-
-cudaError_t launch_gemm32(const GemmArgsMixed& g, cudaStream_t s) {
-    const bool small = g.K <= SMAX && g.N <= SMAX;
-    if (small) {
-        const bool cm = (g.c_rs == 1);
-        if (g.a_f64 && !g.c_f64) launch_gemm_small_t<double, float>(g, cm, s);
-        else if (!g.a_f64 && !g.c_f64) launch_gemm_small_t<float, float>(g, cm, s);
-        else if (!g.a_f64 && g.c_f64) launch_gemm_small_t<float, double>(g, cm, s);
-        else return cudaErrorInvalidValue;
-        return cudaGetLastError();
-    }
-    dim3 grid((g.M + BM - 1) / BM, (g.N + BN - 1) / BN, g.nb1 * g.nb2);
-    const bool cm = (g.c_rs == 1);
-    if (g.a_f64 && !g.c_f64) {
-        if (cm) k_gemm32<true, double, float><<<grid, 256, 0, s>>>(g);
-        else k_gemm32<false, double, float><<<grid, 256, 0, s>>>(g);
-    } else if (!g.a_f64 && !g.c_f64) {
-        if (cm) k_gemm32<true, float, float><<<grid, 256, 0, s>>>(g);
-        else k_gemm32<false, float, float><<<grid, 256, 0, s>>>(g);
-    } else if (!g.a_f64 && g.c_f64) {
-        if (cm) k_gemm32<true, float, double><<<grid, 256, 0, s>>>(g);
-        else k_gemm32<false, float, double><<<grid, 256, 0, s>>>(g);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
 cudaError_t launch_tridiag_lines32(float* y, int64_t ld, int p, int L, int64_t nmodes, float l_sub,
                                    const float* th_m, const float* th_c, float inv_t,
                                    cudaStream_t s) {
@@ -960,32 +672,9 @@ cudaError_t launch_tridiag_lines32(float* y, int64_t ld, int p, int L, int64_t n
     return cudaGetLastError();
 }
 
-template <typename TA, typename TC, int NJ>
-static cudaError_t set_gemm_small_smem() {
-    const int mx = (int)gemm_small_smem(SMAX, NJ);
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_small<true, TA, TC, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_gemm_small<false, TA, TC, NJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    return e;
-}
-
-template <typename TA, typename TC>
-static cudaError_t set_gemm_small_smem_t() {
-    cudaError_t e = set_gemm_small_smem<TA, TC, 2>();
-    if (e == cudaSuccess) e = set_gemm_small_smem<TA, TC, 3>();
-    if (e == cudaSuccess) e = set_gemm_small_smem<TA, TC, 4>();
-    if (e == cudaSuccess) e = set_gemm_small_smem<TA, TC, 5>();
-    if (e == cudaSuccess) e = set_gemm_small_smem<TA, TC, 6>();
-    return e;
-}
-
 cudaError_t operator_set_smem_limits() {
-    cudaError_t e = cudaFuncSetAttribute(k_tridiag_tile32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kTridiagTileSmemMax);
-    if (e == cudaSuccess) e = set_gemm_small_smem_t<double, float>();
-    if (e == cudaSuccess) e = set_gemm_small_smem_t<float, float>();
-    if (e == cudaSuccess) e = set_gemm_small_smem_t<float, double>();
-    return e;
+    return cudaFuncSetAttribute(k_tridiag_tile32, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kTridiagTileSmemMax);
 }
 
 int true_resid_blocks(int64_t n) { return (int)((n + 255) / 256); }
@@ -1001,8 +690,8 @@ cudaError_t launch_true_resid(const double* X, int64_t ldx, const double* B, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s) {
-    k_d2f<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, out, n);
+cudaError_t launch_d2f(const double* in, float* out, int64_t n, cudaStream_t s, int64_t ldin, int64_t ldout, int cols) {
+    k_d2f<<<dim3((unsigned)((n + 255) / 256), (unsigned)cols), 256, 0, s>>>(in, out, n, ldin, ldout);
     return cudaGetLastError();
 }
 

@@ -377,20 +377,18 @@ k_qr_apply(const double* __restrict__ W, int64_t ldw, int p, int64_t n, const fl
             }
             if (kc + 1 < nk) load(tile, kc + 1);
             else if (tile + tstep < ntiles) load(tile + tstep, 0);
+            uint2 hq[NT][3];
 #pragma unroll
-            for (int j = 0; j < NT; ++j) {
-                const uint2* hq = hb + ((kc * NT + j) * 3) * 32 + lane;
-                const uint2 b0 = hq[0], b1 = hq[32], b2 = hq[64];
+            for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    mma_bf16(cm[i][j], a[i][0], b0.x, b0.y);
-                    mma_bf16(cc[i][j], a[i][2], b0.x, b0.y);
-                    mma_bf16(cc[i][j], a[i][0], b2.x, b2.y);
-                    mma_bf16(cc[i][j], a[i][1], b1.x, b1.y);
-                    mma_bf16(cc[i][j], a[i][1], b0.x, b0.y);
-                    mma_bf16(cc[i][j], a[i][0], b1.x, b1.y);
-                }
-            }
+                for (int k = 0; k < 3; ++k) hq[j][k] = hb[((kc * NT + j) * 3 + k) * 32 + lane];
+#pragma unroll
+            for (int pr = 0; pr < 6; ++pr)
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        mma_bf16(pr == 0 ? cm[i][j] : cc[i][j], a[i][kProdA[pr]], hq[j][kProdB[pr]].x, hq[j][kProdB[pr]].y);
         }
         __syncwarp();
 #pragma unroll
