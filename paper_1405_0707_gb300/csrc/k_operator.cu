@@ -14,12 +14,16 @@
 namespace expm {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16;
+constexpr int BK = 16;
 
-// C = A * B, FP64.  256 threads, 4x4 outputs per thread.  CM selects the thread layout
-// so that the fastest-varying thread index walks C's contiguous dimension.
-template <bool CM>
+// C = A * B, FP64.  256 threads, TM x TM outputs per thread (tiles of 16 TM).  CM selects the thread
+// layout so that the fastest-varying thread index walks C's contiguous dimension.  The FP64 pipe (2 FMAs
+// per SM and clock) is the bound, whatever the tile: a 64 x 64 tile keeps one SM busy for 100 us at
+// K = 99, so small problems take smaller tiles and spread over the SMs (launch_gemm picks the tile with
+// the least work on the fullest SM; 99 x 99, 3 columns: 127 us with 12 CTAs, 10 us with 147).
+template <bool CM, int TM>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
+    constexpr int BM = 16 * TM, BN = 16 * TM;
     __shared__ double As[BK][BM + 1];
     __shared__ double Bs[BK][BN];
     const int b1 = blockIdx.z % g.nb1, b2 = blockIdx.z / g.nb1;
@@ -28,14 +32,14 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const bool a_mfast = (g.a_rs == 1);
-    double acc[4][4];
+    double acc[TM][TM];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < TM; ++j) acc[i][j] = 0.0;
     for (int k0 = 0; k0 < g.K; k0 += BK) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < TM; ++q) {
             const int e = tid + q * 256;
             int mm, kk;
             if (a_mfast) { mm = e % BM; kk = e / BM; }
@@ -44,7 +48,7 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
             As[kk][mm] = (gm < g.M && gk < g.K) ? A[(int64_t)gm * g.a_rs + (int64_t)gk * g.a_cs] : 0.0;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < TM; ++q) {
             const int e = tid + q * 256;
             const int nn = e % BN, kk = e / BN;
             const int gn = n0 + nn, gk = k0 + kk;
@@ -53,22 +57,22 @@ __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            double a[4], b[4];
+            double a[TM], b[TM];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][(CM ? tx : ty) + 16 * i];
+            for (int i = 0; i < TM; ++i) a[i] = As[kk][(CM ? tx : ty) + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][(CM ? ty : tx) + 16 * j];
+            for (int j = 0; j < TM; ++j) b[j] = Bs[kk][(CM ? ty : tx) + 16 * j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TM; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < TM; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TM; ++j) {
             const int m = m0 + (CM ? tx : ty) + 16 * i, nn = n0 + (CM ? ty : tx) + 16 * j;
             if (m < g.M && nn < g.N) C[(int64_t)m * g.c_rs + (int64_t)nn * g.c_cs] = acc[i][j];
         }
@@ -197,6 +201,116 @@ __global__ void k_tridiag_lines(const double* in, int64_t ld_in, double* out, in
     const int c = active ? (int)(line / nmodes) : 0;
     tridiag_seg<double>(in + c * ld_in + k, out + c * ld_out + k, L, nmodes, k, l_sub, thm, thc, inv_t, seg,
                         active);
+}
+
+// A single long line per column (1-D problems): one CTA per line.  Thread t owns kLineE consecutive
+// points of each chunk of kLineT kLineE; it composes their affine maps keeping the partial results, the
+// CTA scans the threads' maps, and each point is corrected with the value that enters its segment
+// (y = y_local + P y_in), so every point is read once per sweep and costs nine FP64 operations.  With the
+// warp-per-four-lines kernel above, 2000 points were 250 dependent FP64 steps per lane: 178 us a solve,
+// now 11 us, most of it the one SM's FP64 pipe.
+constexpr int kLineT = 256, kLineE = 8;
+
+struct Affine {
+    double a, b;     // v -> a v + b
+};
+
+// exclusive scan over the CTA of the maps in thread order (rev: descending), the total in *tot; red:
+// one slot per warp
+__device__ inline Affine line_scan(Affine m, bool rev, Affine* red, Affine* tot) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pos = rev ? 31 - lane : lane;
+    const int nw = kLineT / 32, wpos = rev ? nw - 1 - warp : warp;
+    Affine x = m;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int src = rev ? lane + d : lane - d;
+        const double pa = __shfl_sync(full, x.a, src & 31), pb = __shfl_sync(full, x.b, src & 31);
+        if (pos >= d) {
+            x.b = fma(x.a, pb, x.b);
+            x.a = x.a * pa;
+        }
+    }
+    __syncthreads();
+    if (pos == 31) red[wpos] = x;
+    const int prev = rev ? lane + 1 : lane - 1;
+    Affine e;
+    e.a = __shfl_sync(full, x.a, prev & 31);
+    e.b = __shfl_sync(full, x.b, prev & 31);
+    if (pos == 0) e = Affine{1.0, 0.0};
+    __syncthreads();
+    Affine w{1.0, 0.0}, all{1.0, 0.0};
+    for (int k = 0; k < nw; ++k) {
+        if (k == wpos) w = all;
+        all = Affine{red[k].a * all.a, fma(red[k].a, all.b, red[k].b)};
+    }
+    *tot = all;
+    return Affine{e.a * w.a, fma(e.a, w.b, e.b)};
+}
+
+__global__ void __launch_bounds__(kLineT) k_line_solve(const double* in, int64_t ld_in, double* out, int64_t ld_out,
+                                                       int L, double l_sub, const double* __restrict__ thm,
+                                                       const double* __restrict__ thc, double inv_t) {
+    __shared__ Affine red[kLineT / 32];
+    const double* f = in + (int64_t)blockIdx.x * ld_in;
+    double* y = out + (int64_t)blockIdx.x * ld_out;
+    constexpr int CH = kLineT * kLineE;
+    const int nch = (L + CH - 1) / CH;
+    double yv[kLineE], pv[kLineE];
+    double carry = 0.0;
+    for (int ch = 0; ch < nch; ++ch) {
+        const int x0 = ch * CH + threadIdx.x * kLineE;
+        double mv[kLineE];
+#pragma unroll
+        for (int q = 0; q < kLineE; ++q) {
+            yv[q] = x0 + q < L ? f[x0 + q] : 0.0;
+            mv[q] = x0 + q < L ? thm[x0 + q] : 0.0;
+        }
+        Affine m{1.0, 0.0};
+#pragma unroll
+        for (int q = 0; q < kLineE; ++q) {
+            const double a = -l_sub * mv[q];
+            m.b = fma(a, m.b, yv[q] * inv_t * mv[q]);
+            m.a *= a;
+            yv[q] = m.b;
+            pv[q] = m.a;
+        }
+        Affine tot;
+        const Affine ex = line_scan(m, false, red, &tot);
+        const double yin = fma(ex.a, carry, ex.b);
+        carry = fma(tot.a, carry, tot.b);
+#pragma unroll
+        for (int q = 0; q < kLineE; ++q) {
+            yv[q] = fma(pv[q], yin, yv[q]);
+            if (x0 + q < L && ch + 1 < nch) y[x0 + q] = yv[q];      // the last chunk stays in registers
+        }
+    }
+    carry = 0.0;
+    for (int ch = nch - 1; ch >= 0; --ch) {
+        const int x0 = ch * CH + threadIdx.x * kLineE;
+        double cv[kLineE];
+#pragma unroll
+        for (int q = 0; q < kLineE; ++q) {
+            if (ch + 1 < nch) yv[q] = x0 + q < L ? y[x0 + q] : 0.0;
+            else if (x0 + q >= L) yv[q] = 0.0;
+            cv[q] = x0 + q < L - 1 ? thc[x0 + q] : 0.0;
+        }
+        Affine m{1.0, 0.0};
+#pragma unroll
+        for (int q = kLineE - 1; q >= 0; --q) {
+            m.b = fma(-cv[q], m.b, yv[q]);
+            m.a *= -cv[q];
+            yv[q] = m.b;
+            pv[q] = m.a;
+        }
+        Affine tot;
+        const Affine ex = line_scan(m, true, red, &tot);
+        const double zin = fma(ex.a, carry, ex.b);
+        carry = fma(tot.a, carry, tot.b);
+#pragma unroll
+        for (int q = 0; q < kLineE; ++q)
+            if (x0 + q < L) y[x0 + q] = fma(pv[q], zin, yv[q]);
+    }
 }
 
 // Thomas factors for every mode (one thread per mode): pivots b - l c'_{x-1}, stored as
@@ -588,15 +702,40 @@ __global__ void k_d2f(const double* __restrict__ in, float* __restrict__ out, in
 }  // namespace
 
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
-    dim3 grid((g.M + BM - 1) / BM, (g.N + BN - 1) / BN, g.nb1 * g.nb2);
-    if (g.c_rs == 1) k_gemm<true><<<grid, 256, 0, s>>>(g);
-    else k_gemm<false><<<grid, 256, 0, s>>>(g);
+    // FP64 work of the fullest SM per tile side: CTAs per SM times tile area; larger tiles (fewer
+    // shared-memory loads per FMA) at equal work
+    constexpr int64_t kSms = 152;
+    int best = 4;
+    int64_t cost = INT64_MAX;
+    for (int tm = 4; tm >= 1; tm /= 2) {
+        const int64_t b = 16 * tm, ctas = ((g.M + b - 1) / b) * ((g.N + b - 1) / b) * (int64_t)(g.nb1 * g.nb2);
+        const int64_t c = (ctas + kSms - 1) / kSms * b * b;
+        if (c < cost) {
+            cost = c;
+            best = tm;
+        }
+    }
+    const int b = 16 * best;
+    const dim3 grid((g.M + b - 1) / b, (g.N + b - 1) / b, g.nb1 * g.nb2);
+    if (g.c_rs == 1) {
+        if (best == 4) k_gemm<true, 4><<<grid, 256, 0, s>>>(g);
+        else if (best == 2) k_gemm<true, 2><<<grid, 256, 0, s>>>(g);
+        else k_gemm<true, 1><<<grid, 256, 0, s>>>(g);
+    } else {
+        if (best == 4) k_gemm<false, 4><<<grid, 256, 0, s>>>(g);
+        else if (best == 2) k_gemm<false, 2><<<grid, 256, 0, s>>>(g);
+        else k_gemm<false, 1><<<grid, 256, 0, s>>>(g);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_tridiag_lines(const double* in, int64_t ld_in, double* out, int64_t ld_out,
                                  int p, int L, int64_t nmodes, double l_sub, const double* th_m,
                                  const double* th_c, double inv_t, cudaStream_t s) {
+    if (nmodes == 1) {
+        k_line_solve<<<p, kLineT, 0, s>>>(in, ld_in, out, ld_out, L, l_sub, th_m, th_c, inv_t);
+        return cudaGetLastError();
+    }
     const int64_t lines = nmodes * p, per_block = 128 / TSEG;
     k_tridiag_lines<<<(unsigned)((lines + per_block - 1) / per_block), 128, 0, s>>>(in, ld_in, out, ld_out, p, L,
                                                                                  nmodes, l_sub, th_m, th_c, inv_t);
