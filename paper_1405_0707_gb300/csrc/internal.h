@@ -200,7 +200,7 @@ struct expm_plan_s {
     int nblk = 0;
     int nblk_cgs = 0;          // CTAs of the first CGS pass (projection, update)
     double* small = nullptr;   // small scratch (see api.cu for the map)
-    double* poles = nullptr;   // per-pole elimination workspace (global fallback)
+    double* poles = nullptr;   // per-pole elimination workspace
     double* S = nullptr;       // per-pole restart factors, npoles x p x p complex
     double* Wc_slots = nullptr;// per-pole (m+1)p x p update coefficients
     double* stat = nullptr;    // device status block: res[16], normsq, flags (ints)
@@ -395,6 +395,7 @@ cudaError_t operator_set_smem_limits();
 cudaError_t krylov_set_smem_limits();
 cudaError_t poles_set_smem_limits();
 size_t poles_smem_bytes(int mp, int p);
+size_t poles_work_doubles(int mp, int p);   // workspace of one pole
 cudaError_t launch_init_S(const double* R, int p, int npoles, double* S, cudaStream_t s,
                           const double* R_alt = nullptr, const int* use_alt = nullptr);
 cudaError_t launch_axpby(double a, const double* X, int64_t ldx, double b, const double* Y,

@@ -17,6 +17,8 @@
 // at rows j..kk+p-1.  The
 // matrix lives in shared memory when (mp)^2 + mp p complex numbers fit, else in a global
 // workspace (L2-resident).
+#include <algorithm>
+
 #include "internal.h"
 
 namespace expm {
@@ -266,6 +268,367 @@ __global__ void __launch_bounds__(kPoleThreads) k_poles(const double* __restrict
     }
 }
 
+// ---------------------------------------------------------------- one cluster per pole
+//
+// The same blocked elimination by a cluster of kPc CTAs per pole (plans without a deflated block).
+// The FP64 pipe of one SM (2 FMAs per clock) is what bounds the one-CTA kernel below, so the trailing
+// columns and the right-hand sides are dealt out over the cluster's SMs; M and X live in global memory
+// (L2), each column is only ever touched by its owner, and the p-wide panel is factored in shared
+// memory by CTA 0 of the cluster and handed on through global memory between cluster barriers:
+//
+//   panel    CTA 0: rows r0 .. rend-1 of block column J, pivoted, two barriers per column; the unit
+//            lower block is inverted by doubling (log2 p steps instead of p^2 / 2 dependent ones)
+//   update   every CTA, its columns 32 at a time in shared memory: swaps, U = L^-1 top, below -= L U
+//   back     X's columns are independent: each CTA substitutes its own
+//
+// Values that another CTA wrote are read past L1 (__ldcg).  Measured per launch (7 poles), one CTA per
+// pole -> cluster: m = 10, p = 8 288 -> 256 us, p = 12 580 -> 412 us, p = 16 1008 -> 578 us, p = 32
+// 5541 -> 2270 us; m = 30, p = 8 1196 -> 780 us, p = 16 5887 -> 2192 us.  Each block column costs ~8 us
+// of barriers and L2 round trips, so narrow blocks (p = 4, m = 10: 123 -> 162 us) stay on one CTA.
+constexpr int kPc = 8;            // CTAs per cluster
+constexpr int kPcT = 256;
+
+// |v|^2 for the pivot search from the operands' leading bits (truncated to FP32 with integer
+// operations: a conversion occupies the FP64 pipe like an FMA)
+__device__ __forceinline__ float lead32(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7FFu) - 896;
+    const uint32_t f = (e <= 0 ? 0u : e >= 255 ? 0x7F800000u : ((uint32_t)e << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+    return __uint_as_float(f);
+}
+__device__ __forceinline__ cplx ldc(const cplx* p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2*>(p));
+    return cplx{v.x, v.y};
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// complex numbers of the workspace of one pole: M, X, U_JJ^{-1}, the panel in flight, |S|^2 partials
+__host__ __device__ constexpr size_t poles_work(int mp, int p) {
+    return (size_t)mp * mp + 2 * (size_t)mp * p + 3 * (size_t)p * p + (size_t)p + kPc;
+}
+constexpr size_t poles_cluster_smem(int mp, int p) {
+    return sizeof(cplx) * std::max(3 * (size_t)p * p + 2 * (size_t)p * 32, (size_t)mp * ((p + kPc - 1) / kPc));
+}
+
+__global__ void __launch_bounds__(kPcT) __cluster_dims__(kPc, 1, 1)
+k_poles_cluster(const double* __restrict__ H, int ldH, int mp, int p, const double* __restrict__ tau_re,
+                const double* __restrict__ tau_im, const double* __restrict__ om_re, const double* __restrict__ om_im,
+                double* __restrict__ S, double* work, double* __restrict__ Y_slots, double* res, int* flags, int alg,
+                double* __restrict__ Zout) {
+    extern __shared__ __align__(16) unsigned char smp[];
+    cplx* P = reinterpret_cast<cplx*>(smp);              // 2p x p panel
+    cplx* Li = P + 2 * (size_t)p * p;                    // p x p inverse of its unit lower block
+    cplx* Tl = Li + (size_t)p * p;                       // 2p x 32 columns being updated (CTA 0: scratch)
+    __shared__ int piv_s[kMaxP];
+    __shared__ cplx inv_s;
+    __shared__ double red[kPcT];
+    const int rank = blockIdx.x % kPc, i = blockIdx.x / kPc, tid = threadIdx.x, lane = tid & 31;
+    const cplx tau{tau_re[i], tau_im[i]}, om{om_re[i], om_im[i]};
+    cplx* M = reinterpret_cast<cplx*>(work) + (size_t)i * poles_work(mp, p);
+    cplx* X = M + (size_t)mp * mp;
+    cplx* Ui = X + (size_t)mp * p;
+    cplx* pan = Ui + (size_t)mp * p;                     // 2p x p panel, p x p inverse
+    cplx* rdg = pan + 3 * (size_t)p * p;                 // pivots as integers (re)
+    double* parts = reinterpret_cast<double*>(rdg + p);
+    cplx* Si = reinterpret_cast<cplx*>(S) + (size_t)i * p * p;
+    const int gt = rank * kPcT + tid, gn = kPc * kPcT;
+    // M = I - tau H_m (eq. (3236)) or H_m - tau I (eq. (3.3)); X = E_1 S_i
+    for (int e = gt; e < mp * mp; e += gn) {
+        const int c = e / mp, r = e - c * mp;            // H column-major: r fastest
+        const double h = H[(int64_t)c * ldH + r], d = r == c ? 1.0 : 0.0;
+        M[(size_t)r * mp + c] = alg == 2 ? cplx{d - tau.re * h, -tau.im * h} : cplx{h - d * tau.re, -d * tau.im};
+    }
+    for (int e = gt; e < mp * p; e += gn) X[e] = e / p < p ? Si[e] : cplx{0.0, 0.0};
+    cluster_sync();
+    const int nbc = mp / p;
+    // U_JJ^{-1} from the panel in shared memory, by doubling as for the unit lower block: run by one of
+    // the CTAs that wait while CTA 0 factors the next panel
+    auto invert_upper = [&](int J) {
+        for (int e = tid; e < p * p; e += kPcT) {
+            const int a = e / p, b = e - a * p;
+            cplx v{0.0, 0.0};
+            if (a == b) {
+                const cplx d = P[e];
+                const double x = 1.0 / (d.re * d.re + d.im * d.im);
+                v = cplx{d.re * x, -d.im * x};
+            }
+            Li[e] = v;
+        }
+        __syncthreads();
+        for (int s = 1; s < p; s *= 2) {
+            for (int ph = 0; ph < 2; ++ph) {
+                for (int e = tid; e < p * s; e += kPcT) {          // rows a of the upper block, columns c of the lower
+                    const int b = e / (2 * s * s) * 2 * s, o = e % (2 * s * s), a = b + o / s, c = b + s + o % s;
+                    if (o < s * s && c < p) {
+                        cplx t{0.0, 0.0};
+                        if (ph == 0) {                             // T = -B C^-1
+                            for (int k = b + s; k <= c; ++k) cmsub(t, P[a * p + k], Li[k * p + c]);
+                            Tl[a * p + c] = t;
+                        } else {                                   // A^-1 T
+                            for (int k = a; k < b + s; ++k) {
+                                const cplx l = Li[a * p + k], x = Tl[k * p + c];
+                                t.re = fma(l.re, x.re, fma(-l.im, x.im, t.re));
+                                t.im = fma(l.re, x.im, fma(l.im, x.re, t.im));
+                            }
+                            Li[a * p + c] = t;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        for (int e = tid; e < p * p; e += kPcT) Ui[(size_t)J * p * p + e] = Li[e];
+        __syncthreads();
+    };
+    for (int J = 0; J < nbc; ++J) {
+        const int r0 = J * p, rows = min(2 * p, mp - r0);
+        if (J > 0 && rank == 1 + (J - 1) % (kPc - 1)) invert_upper(J - 1);
+        if (rank == 0) {
+            for (int e = tid; e < rows * p; e += kPcT) P[e] = ldc(M + (size_t)(r0 + e / p) * mp + r0 + e % p);
+            __syncthreads();
+            constexpr int kEl = (2 * kMaxP * kMaxP + kPcT - 1) / kPcT;
+            int er[kEl], ek[kEl];                        // this thread's panel entries
+#pragma unroll
+            for (int q = 0; q < kEl; ++q) {
+                const int e = tid + q * kPcT;
+                er[q] = e < rows * p ? e / p : -1;
+                ek[q] = e - max(er[q], 0) * p;
+            }
+            for (int jj = 0; jj < p; ++jj) {
+                // pivot: arg-max of the magnitudes in FP32, by every warp for itself
+                float best = -1.f;
+                int piv = jj;
+                for (int r = jj + lane; r < rows; r += 32) {
+                    const cplx v = P[r * p + jj];
+                    const float fr = lead32(v.re), fi = lead32(v.im), m = fmaf(fr, fr, fi * fi);
+                    if (m > best) {
+                        best = m;
+                        piv = r;
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int op = __shfl_xor_sync(0xffffffffu, piv, o);
+                    if (ob > best || (ob == best && op < piv)) {
+                        best = ob;
+                        piv = op;
+                    }
+                }
+                if (tid == 0) {
+                    const cplx d = P[piv * p + jj];
+                    const double n2 = d.re * d.re + d.im * d.im;
+                    if (!(n2 > 0.0)) atomicOr(&flags[0], 2);
+                    const double x = 1.0 / n2;
+                    inv_s = cplx{d.re * x, -d.im * x};
+                    piv_s[jj] = piv;
+                }
+                __syncthreads();
+                const cplx inv = inv_s;
+                // rows jj .. with the pivot row moved up, the others eliminated; all reads, then all
+                // writes.  Columns left of jj (stored multipliers) only swap.
+                cplx nv[kEl];
+#pragma unroll
+                for (int q = 0; q < kEl; ++q) {
+                    if (q * kPcT >= rows * p) break;
+                    const int r = er[q], k = ek[q];
+                    if (r >= jj) {
+                        const int src = r == jj ? piv : r == piv ? jj : r;
+                        cplx v = P[src * p + k];
+                        if (r > jj && k >= jj) {
+                            const cplx mlt = cmul(P[src * p + jj], inv);
+                            if (k == jj) v = mlt;
+                            else cmsub(v, mlt, P[piv * p + k]);
+                        }
+                        nv[q] = v;
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < kEl; ++q) {
+                    if (q * kPcT >= rows * p) break;
+                    if (er[q] >= jj) P[tid + q * kPcT] = nv[q];
+                }
+                __syncthreads();
+            }
+            // inverse of the unit lower block by doubling: the off-diagonal blocks of size s from the
+            // inverses of the two diagonal blocks of size s
+            for (int e = tid; e < p * p; e += kPcT) Li[e] = cplx{e / p == e % p ? 1.0 : 0.0, 0.0};
+            __syncthreads();
+            for (int s = 1; s < p; s *= 2) {
+                for (int e = tid; e < p * s; e += kPcT) {          // T = B A^-1, rows of the lower blocks
+                    const int b = e / (2 * s * s) * 2 * s, o = e % (2 * s * s), a = b + s + o / s, c = b + o % s;
+                    if (o < s * s && a < p) {
+                        cplx t{0.0, 0.0};
+                        for (int k = c; k < b + s; ++k) cmsub(t, P[a * p + k], Li[k * p + c]);
+                        Tl[a * p + c] = t;                         // -B A^-1
+                    }
+                }
+                __syncthreads();
+                for (int e = tid; e < p * s; e += kPcT) {
+                    const int b = e / (2 * s * s) * 2 * s, o = e % (2 * s * s), a = b + s + o / s, c = b + o % s;
+                    if (o < s * s && a < p) {
+                        cplx t = Tl[a * p + c];                    // C^-1 (-B A^-1), C^-1 unit lower
+                        for (int k = b + s; k < a; ++k) {
+                            const cplx l = Li[a * p + k], x = Tl[k * p + c];
+                            t.re = fma(l.re, x.re, fma(-l.im, x.im, t.re));
+                            t.im = fma(l.re, x.im, fma(l.im, x.re, t.im));
+                        }
+                        Li[a * p + c] = t;
+                    }
+                }
+                __syncthreads();
+            }
+            for (int e = tid; e < rows * p; e += kPcT) {
+                pan[e] = P[e];
+                M[(size_t)(r0 + e / p) * mp + r0 + e % p] = P[e];
+            }
+            for (int e = tid; e < p * p; e += kPcT) pan[2 * (size_t)p * p + e] = Li[e];
+            if (tid < p) rdg[tid] = cplx{(double)piv_s[tid], 0.0};
+        }
+        cluster_sync();
+        if (rank != 0) {
+            for (int e = tid; e < rows * p; e += kPcT) P[e] = ldc(pan + e);
+            for (int e = tid; e < p * p; e += kPcT) Li[e] = ldc(pan + 2 * (size_t)p * p + e);
+            if (tid < p) piv_s[tid] = (int)ldc(rdg + tid).re;
+        }
+        // this CTA's columns: every kPc-th of M's trailing ones and of X's, 32 at a time
+        const int ncm = mp - r0 - p, ncol = ncm + p, mine = (ncol - rank + kPc - 1) / kPc;
+        for (int q0 = 0; q0 < mine; q0 += 32) {
+            const int nc = min(32, mine - q0);
+            auto at = [&](int r, int q) -> cplx* {       // row r0 + r of this chunk's column q
+                const int c = rank + (q0 + q) * kPc;
+                return c < ncm ? M + (size_t)(r0 + r) * mp + r0 + p + c : X + (size_t)(r0 + r) * p + (c - ncm);
+            };
+            __syncthreads();
+            for (int e = tid; e < rows * nc; e += kPcT) Tl[(e / nc) * 32 + e % nc] = ldc(at(e / nc, e % nc));
+            __syncthreads();
+            if (tid < nc)
+                for (int jj = 0; jj < p; ++jj) {
+                    const int pv = piv_s[jj];
+                    if (pv != jj) {
+                        const cplx a = Tl[jj * 32 + tid];
+                        Tl[jj * 32 + tid] = Tl[pv * 32 + tid];
+                        Tl[pv * 32 + tid] = a;
+                    }
+                }
+            __syncthreads();
+            constexpr int kUo = (kMaxP * 32 + kPcT - 1) / kPcT;
+            cplx u[kUo];
+#pragma unroll
+            for (int q = 0; q < kUo; ++q) {
+                const int e = tid + q * kPcT, a = e / nc, c = e - a * nc;
+                if (e < p * nc) {
+                    cplx s = Tl[a * 32 + c];
+                    for (int k = 0; k < a; ++k) {
+                        const cplx l = Li[a * p + k], x = Tl[k * 32 + c];
+                        s.re = fma(l.re, x.re, fma(-l.im, x.im, s.re));
+                        s.im = fma(l.re, x.im, fma(l.im, x.re, s.im));
+                    }
+                    u[q] = s;
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < kUo; ++q) {
+                const int e = tid + q * kPcT, a = e / nc, c = e - a * nc;
+                if (e < p * nc) {
+                    Tl[a * 32 + c] = u[q];
+                    *at(a, c) = u[q];
+                }
+            }
+            __syncthreads();
+            for (int e = tid; e < (rows - p) * nc; e += kPcT) {
+                const int a = e / nc, c = e - a * nc;
+                cplx s = Tl[(p + a) * 32 + c];
+                for (int k = 0; k < p; ++k) cmsub(s, P[(p + a) * p + k], Tl[k * 32 + c]);
+                *at(p + a, c) = s;
+            }
+        }
+        cluster_sync();
+    }
+    if (rank == 1 + (nbc - 1) % (kPc - 1)) invert_upper(nbc - 1);
+    cluster_sync();
+    // blocked back substitution of this CTA's columns of X (c = rank + kPc q), held in shared memory;
+    // U's entries are loaded eight at a time
+    const int nx = rank < p ? (p - rank + kPc - 1) / kPc : 0;
+    cplx* Xl = P;                                        // mp x nx (P, Li and Tl are free now)
+    for (int e = tid; e < mp * nx; e += kPcT) Xl[e] = ldc(X + (size_t)(e / nx) * p + rank + (e % nx) * kPc);
+    __syncthreads();
+    auto dot = [&](cplx s, const cplx* m, int k0, int k1, const cplx* x) {   // s - sum_k m[k] x[k nx]
+        for (int k = k0; k < k1; k += 8) {
+            cplx v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k + u < k1) v[u] = ldc(m + k + u);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k + u < k1) cmsub(s, v[u], x[(size_t)(k + u) * nx]);
+        }
+        return s;
+    };
+    for (int J = nbc - 1; J >= 0; --J) {
+        const int r0 = J * p;
+        constexpr int kXo = (kMaxP * ((kMaxP + kPc - 1) / kPc) + kPcT - 1) / kPcT;
+        cplx xn[kXo];
+#pragma unroll
+        for (int q = 0; q < kXo; ++q) {
+            const int e = tid + q * kPcT;
+            if (e < p * nx) xn[q] = dot(cplx{0.0, 0.0}, Ui + ((size_t)J * p + e / nx) * p, e / nx, p, Xl + (size_t)r0 * nx + e % nx);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kXo; ++q) {
+            const int e = tid + q * kPcT;
+            if (e < p * nx) Xl[(size_t)r0 * nx + e] = cplx{-xn[q].re, -xn[q].im};
+        }
+        __syncthreads();
+        for (int e = tid; e < r0 * nx; e += kPcT)
+            Xl[e] = dot(Xl[e], M + (size_t)(e / nx) * mp + r0, 0, p, Xl + (size_t)r0 * nx + e % nx);
+        __syncthreads();
+    }
+    // S_i, its norm, Y_i = 2 Re(omega_i Z_i) for this CTA's columns
+    double ss = 0.0;
+    for (int e = tid; e < p * nx; e += kPcT) {
+        const int a = e / nx, c = rank + (e % nx) * kPc;
+        cplx s{0.0, 0.0};
+        for (int b = 0; b < p; ++b) {
+            const double h = H[(int64_t)(mp - p + b) * ldH + mp + a];
+            const cplx x = Xl[(size_t)(mp - p + b) * nx + e % nx];
+            s.re += h * x.re;
+            s.im += h * x.im;
+        }
+        const cplx snew = (alg == 2) ? cmul(tau, s) : cplx{-s.re, -s.im};
+        Si[a * p + c] = snew;
+        ss += cabs2(snew);
+    }
+    red[tid] = ss;
+    __syncthreads();
+    for (int st = kPcT / 2; st > 0; st >>= 1) {
+        if (tid < st) red[tid] += red[tid + st];
+        __syncthreads();
+    }
+    if (tid == 0) parts[rank] = red[0];
+    double* Yi = Y_slots + (size_t)i * mp * p;
+    cplx* Zi = Zout ? reinterpret_cast<cplx*>(Zout) + (size_t)i * mp * p : nullptr;
+    for (int e = tid; e < mp * nx; e += kPcT) {
+        const int r = e % mp, c = rank + (e / mp) * kPc;
+        const cplx x = Xl[(size_t)r * nx + e / mp];
+        Yi[(size_t)c * mp + r] = 2.0 * (om.re * x.re - om.im * x.im);
+        if (Zi) Zi[(size_t)r * p + c] = x;
+    }
+    cluster_sync();
+    if (rank == 0 && tid == 0) {
+        double s = 0.0;
+        for (int k = 0; k < kPc; ++k) s += __ldcg(parts + k);
+        res[i] = sqrt(s);
+        if (!isfinite(s)) atomicOr(&flags[0], 4);
+    }
+}
+
 // Wc = H~ sum_i Y_i (Algorithm 2) or [sum_i Y_i; 0] (Algorithm 1), (mp+p) x p, row-major
 // [r][c] as k_update_z reads it.  One thread per output, r fastest (coalesced H~ columns).
 __global__ void k_combine2(const double* __restrict__ H, int ldH, int mp, int p, int npoles,
@@ -326,6 +689,10 @@ cudaError_t launch_certify_coeffs(const double* H, int ldH, int mp, int p, int n
     return cudaGetLastError();
 }
 
+size_t poles_work_doubles(int mp, int p) {
+    return 2 * std::max(poles_work(mp, p), (size_t)mp * mp + 2 * (size_t)mp * p);
+}
+
 size_t poles_smem_bytes(int mp, int p) {
     const size_t b = ((size_t)mp * mp + 2 * (size_t)mp * p) * sizeof(cplx);
     return b <= kSmemLimit ? b : 0;
@@ -337,6 +704,13 @@ cudaError_t launch_poles(const double* H, int ldH, int mp, int p, int npoles,
                          const double* tau_re, const double* tau_im, const double* om_re,
                          const double* om_im, double* S, double* work, double* Y_slots,
                          double* res, int* flags, int alg, cudaStream_t s, double* Zout, int kk) {
+    // where the elimination outweighs the cluster's exchanges (p = 6: 189 against 221 us at mp = 60, 723
+    // against 647 us at mp = 180; p = 8: 288 against 256 us at mp = 80)
+    if (kk == 0 && p >= 6 && mp * p >= 600) {
+        k_poles_cluster<<<npoles * kPc, kPcT, poles_cluster_smem(mp, p), s>>>(H, ldH, mp, p, tau_re, tau_im, om_re, om_im, S, work,
+                                                                         Y_slots, res, flags, alg, Zout);
+        return cudaGetLastError();
+    }
     size_t shm = poles_smem_bytes(mp, p);
     int h_in = 0;
     if (shm > 0 && shm + poles_h_bytes(mp, p) <= kSmemLimit) {
@@ -361,6 +735,8 @@ cudaError_t poles_set_smem_limits() {
     // kSmemLimit (200 KB) of dynamic memory plus the kernel's few KB of static memory stays
     // below the 227 KB per-block opt-in maximum
     cudaError_t e = cudaFuncSetAttribute(k_poles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_poles_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)poles_cluster_smem(kMaxMP, kMaxP));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_combine2, cudaFuncAttributeMaxDynamicSharedMemorySize, 140 * 1024);
     return e;
