@@ -561,10 +561,35 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
 // Capture (once) and return the graph of one cycle for (alg, p, t); nullptr if capture is
 // not possible, in which case the caller launches directly.
 GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int prologue = 0) {
+    // the legacy default stream cannot capture: the cycle is captured on a stream of the plan's own and
+    // the graph launched into the default stream.  A cycle is launched directly the first time there
+    // (a solve of one cycle, as on small or stiff problems, does not pay for a capture it uses once)
+    const bool legacy = P->stream == nullptr;
+    GraphEntry* seen = nullptr;
     for (auto& g : P->graphs)
-        if (g.alg == alg && g.p == p && g.t == t && g.kk == kk && g.prologue == prologue) return &g;
-    if (P->graphs.size() >= 16) return nullptr;
-    cudaStream_t s = P->stream;
+        if (g.alg == alg && g.p == p && g.t == t && g.kk == kk && g.prologue == prologue) {
+            if (g.exec) return &g;
+            seen = &g;
+        }
+    if (!seen) {
+        if (P->graphs.size() >= 16) return nullptr;
+        if (legacy) {
+            GraphEntry e;
+            e.alg = alg;
+            e.p = p;
+            e.t = t;
+            e.kk = kk;
+            e.prologue = prologue;
+            P->graphs.push_back(e);
+            return nullptr;
+        }
+    }
+    if (legacy && !P->cap && cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        P->cap = nullptr;
+        return nullptr;
+    }
+    cudaStream_t s = legacy ? P->cap : P->stream;
     const int64_t l0 = P->launches;
     int64_t sl0[EXPM_NSTAGES];
     for (int k = 0; k < EXPM_NSTAGES; ++k) sl0[k] = P->stage_launches[k];
@@ -572,7 +597,10 @@ GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int pr
         cudaGetLastError();
         return nullptr;
     }
+    const cudaStream_t own = P->stream;
+    P->stream = s;
     expm_status st = issue_cycle(P, t, p, alg, kk, prologue);
+    P->stream = own;
     cudaGraph_t graph = nullptr;
     cudaError_t ec = cudaStreamEndCapture(s, &graph);
     GraphEntry e;
@@ -597,6 +625,10 @@ GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int pr
     if (ei != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
+    }
+    if (seen) {
+        *seen = e;
+        return seen;
     }
     P->graphs.push_back(e);
     return &P->graphs.back();
@@ -655,7 +687,8 @@ expm_status run_issue(expm_plan* P, RunState& r) {
     r.steps += P->opts.m - r.kk / r.p;
     // graph of one restart cycle, cached per (algorithm, p, t, restart kind)
     r.ge = nullptr;
-    if (P->use_graphs && !P->prof && P->stream != nullptr) r.ge = graph_for(P, r.t, r.p, r.alg, r.kk, r.prologue);
+    // (the sparse operator's inexact inverse synchronises inside a block step: no graph)
+    if (P->use_graphs && !P->prof && !(P->csr && r.alg == EXPM_ALG_PSBFOM)) r.ge = graph_for(P, r.t, r.p, r.alg, r.kk, r.prologue);
     if (r.ge) {
         CK(cudaGraphLaunch(r.ge->exec, s));
         P->launches += r.ge->launches;
@@ -881,7 +914,9 @@ void free_plan(expm_plan* P) {
     if (P->cycle_ev) cudaEventDestroy(P->cycle_ev);
     if (P->adj) free_plan(P->adj);
     for (auto& e : P->ev) cudaEventDestroy(e);
-    for (auto& g : P->graphs) cudaGraphExecDestroy(g.exec);
+    for (auto& g : P->graphs)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (P->cap) cudaStreamDestroy(P->cap);
     delete P;
 }
 
@@ -1345,7 +1380,7 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
     P->stream = reinterpret_cast<cudaStream_t>(stream);
     {
         const char* ng = std::getenv("EXPM_DISABLE_GRAPHS");   // debugging switch
-        P->use_graphs = !(ng && ng[0] == '1') && !csr;
+        P->use_graphs = !(ng && ng[0] == '1');
         // test switch: "0" keeps the mixed path on the three-pass FP32 Cholesky-QR for every
         // block (the fallback of the single accurate pass)
         const char* sq = std::getenv("EXPM_QR_SINGLE_PASS");

@@ -148,7 +148,7 @@ struct GraphEntry {
     int alg = 0, p = 0;
     double t = 0.0;
     int kk = 0, prologue = 0;   // deflated restart: kept Ritz vectors, kind of restart prologue
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec = nullptr;   // null: seen once, not captured yet
     int64_t launches = 0;
     int64_t stage_launches[EXPM_NSTAGES] = {};
 };
@@ -248,6 +248,7 @@ struct expm_plan_s {
     double* hPk = nullptr;     // pinned: staging of Pkd
     double* hHnew = nullptr;   // pinned: the leading (kk + p) x kk block of H~ after the restart
     std::vector<GraphEntry> graphs;
+    cudaStream_t cap = nullptr;   // capture stream of plans on the legacy default stream (which cannot capture)
 };
 
 // ---------------------------------------------------------------- launchers
