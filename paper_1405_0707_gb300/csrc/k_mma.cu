@@ -114,6 +114,7 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
         }
     };
     int64_t u = blockIdx.x;
+    int since = 0;
     float4 v[MTW][2];
 #pragma unroll
     for (int i = 0; i < MTW; ++i) v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);   // tiles past nmt
@@ -173,15 +174,22 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
                                          wb[j][kProdB[pr]].y);
                 }
         }
+        // every eight blocks of this warp (CG of them per unit), and at the end
+        since += CG;
+        if (since >= kProjKb || un >= units) {
+            since = 0;
 #pragma unroll
-        for (int i = 0; i < MTW; ++i)
+            for (int i = 0; i < MTW; ++i)
+                if (i < nmt) {
 #pragma unroll
-            for (int j = 0; j < NT; ++j)
+                    for (int j = 0; j < NT; ++j)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    df_add(ch[i][j][q], cc[i][j][q], cm[i][j][q]);
-                    cm[i][j][q] = 0.f;
+                        for (int q = 0; q < 4; ++q) {
+                            df_add(ch[i][j][q], cc[i][j][q], cm[i][j][q]);
+                            cm[i][j][q] = 0.f;
+                        }
                 }
+        }
         buf ^= 1;
         if (un < units) storew(buf);
         __syncthreads();

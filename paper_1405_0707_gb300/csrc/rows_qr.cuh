@@ -51,7 +51,7 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
     __shared__ float sh_[AC * RP], sl_[AC * RP];
     __shared__ float2 Gs[RP * RP], Us[RP * RP], Is[RP], comb[PAD];
     __shared__ float trd[RP];
-    __shared__ double hn2[RP], combd[kRedT];
+    __shared__ float hn2[RP], combf[kRedT];
     __shared__ unsigned ticket;
     __shared__ int kexp_s, sgl_s;
     const int nh = cols * p, nout = nh + p * p, tid = threadIdx.x;
@@ -85,24 +85,26 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
     if (tid == 0) *ctr = 0u;
     // ---- the last CTA.  Its chain is serial, so loads are issued together and the arithmetic
     // stays off the FP64 pipe where it can.
-    // squared norms of the new entries of H above the block (the breakdown test)
-    {
-        const int stripes = kRedT / p, c = tid % p, st = tid / p;
-        double v2 = 0.0;
-        if (st < stripes)
-#pragma unroll 4
-            for (int a = st; a < hrow; a += stripes) {
-                const double v = __ldcg(H + (int64_t)(hcol + c) * ldH + a);
-                v2 = fma(v, v, v2);
-            }
-        combd[tid] = v2;
-    }
     // G is factored as G 2^-kexp (kexp even), kexp from the largest diagonal entry
     if (tid < 32) {
         int e = 0;
         if (tid < p) e = (__double2hiint(__ldcg(h + nh + tid * p + tid)) >> 20) & 0x7FF;
         e = __reduce_max_sync(0xffffffffu, e);
         if (tid == 0) kexp_s = (e - 1022) & ~1;
+    }
+    __syncthreads();
+    const int kexp = kexp_s;
+    // squared norms of the new entries of H above the block, in units of 2^kexp (the breakdown test: FP32)
+    {
+        const int stripes = min(8, kRedT / p), c = tid % p, st = tid / p;
+        float v2 = 0.f;
+        if (st < stripes)
+#pragma unroll 4
+            for (int a = st; a < hrow; a += stripes) {
+                const float v = f32_rn_i(scale_pow2(__ldcg(H + (int64_t)(hcol + c) * ldH + a), -(kexp / 2)));
+                v2 = fmaf(v, v, v2);
+            }
+        combf[tid] = v2;
     }
     const int ne = p * (p + 1) / 2, S = max(1, min(8, kRedT / ne));
     constexpr int KI = (RP * (RP + 1) / 2 + kRedT - 1) / kRedT + 1;
@@ -123,8 +125,6 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
             jj[k] = i + rem;
         }
     }
-    __syncthreads();
-    const int kexp = kexp_s;
     // G - h2^T h2.  The correction is ~2^-40 of G unless the first pass cancelled almost all of W,
     // so its products are formed in FP32 first; only when a diagonal entry's correction passes
     // 2^-20 of it are they formed again in float pairs (G needs ~2^-48).
@@ -177,9 +177,9 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
     }
     if (tid < p) trd[tid] = Gs[tid * p + tid].x;
     if (tid < p) {
-        const int stripes = kRedT / p;
-        double s = 0.0;
-        for (int k = 0; k < stripes; ++k) s += combd[k * p + tid];
+        const int stripes = min(8, kRedT / p);
+        float s = 0.f;
+        for (int k = 0; k < stripes; ++k) s += combf[k * p + tid];
         hn2[tid] = s;
     }
     // Cholesky factor by all threads, thread t holding entries t, t + kRedT, .. of the upper
@@ -290,10 +290,9 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
     }
     if (tid < p) {
         // breakdown: R_cc against the column's norm before orthogonalisation
-        float n0 = 0.f;
+        float n0 = hn2[tid];
         for (int a = 0; a <= tid; ++a) n0 = fmaf(Us[a * p + tid].x, Us[a * p + tid].x, n0);
-        const double nn = scale_pow2(hn2[tid], -kexp) + (double)n0;
-        if ((double)Us[tid * p + tid].x <= 1e-14 * sqrt(nn)) atomicOr(&flags[1], 1);
+        if (Us[tid * p + tid].x <= 1e-14f * sqrtf(n0)) atomicOr(&flags[1], 1);
     }
     if (bad) atomicOr(&flags[0], 1);
 }
