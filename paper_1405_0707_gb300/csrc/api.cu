@@ -387,6 +387,50 @@ expm_status ortho_mma(expm_plan* P, int j, int p) {
     return EXPM_OK;
 }
 
+// FP64 plans take the digit passes on blocks of at least kUse64 entries: they need more launches, and on
+// small blocks the FP64 pipe is not the bound (99 x 99, p = 3, 29403 entries: 4.2 ms with the FP64 kernels,
+// 4.4 with the digit passes; n = 50021, p = 5: 7.0 against 6.4; 256 x 256, p = 8: 54.4 against 34.7).
+constexpr int64_t kUse64 = 100000;
+inline bool use64(const expm_plan* P, int p) { return P->mma64 && P->n * p >= kUse64; }
+
+// The FP64 path's Gram-Schmidt and Cholesky-QR of block step j by exact digit products (k_mma.cu): the
+// column scales of W, projection and update twice, then two Cholesky-QR passes (a third one when the first
+// asks for it), every tall product on the tensor cores and every result rounded once to FP64.  wexp holds
+// two sets of five p-column exponent arrays; a step uses one and clears the other.
+expm_status ortho64(expm_plan* P, int j, int p) {
+    cudaStream_t s = P->stream;
+    const int64_t n = P->n, ld = P->ld;
+    const int cols = (j + 1) * p, hrow = (j + 1) * p, hcol = j * p;
+    double* h = sm(P, kOffH);
+    int* flags = flags_of(P->stat);
+    double* out = P->V + (int64_t)cols * ld;
+    int* w = P->wexp + (j & 1) * 5 * P->p_max;
+    int* other = P->wexp + ((j + 1) & 1) * 5 * P->p_max;
+    int *w1 = w + P->p_max, *w2 = w1 + P->p_max, *w3 = w2 + P->p_max, *w4 = w3 + P->p_max, *vnext = P->colexp + cols;
+    const int maxb = std::max(P->nblk, P->nblk_cgs), sms = P->sms;
+    const double shift = 11.0 * ((double)n * p + (double)p * (p + 1)) * std::ldexp(1.0, -53);
+    int nb = 0;
+    LAUNCH(EXPM_STAGE_CGS, launch_colmax(P->W, ld, p, n, w, other, 5 * P->p_max, vnext, p, s));
+    for (int pass = 0; pass < 2; ++pass) {
+        LAUNCH(EXPM_STAGE_CGS, launch_proj64(P->V, ld, cols, P->colexp, P->W, ld, p, pass ? w1 : w, n, P->part, maxb, sms, &nb,
+                                             nullptr, s));
+        LAUNCH(EXPM_STAGE_REDUCE, launch_reduce_h(P->part, nb, cols, p, h, P->H, P->ldH, 0, hcol, pass, s));
+        LAUNCH(EXPM_STAGE_CGS, launch_upd64(P->V, ld, cols, P->W, ld, p, n, h, P->colexp, pass ? w2 : w1, flags, sms, s));
+    }
+    const int* extra = flags + 2;
+    double *R = sm(P, kOffR), *Ri = sm(P, kOffRi), *Rt = sm(P, kOffRt);
+    LAUNCH(EXPM_STAGE_QR, launch_proj64(P->W, ld, p, w2, P->W, ld, p, w2, n, P->part, maxb, sms, &nb, nullptr, s));
+    LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, nb, p, shift, R, Ri, Rt, 0, P->H, P->ldH, hrow, hcol, nullptr, flags, s));
+    LAUNCH(EXPM_STAGE_QR, launch_mul64(P->W, ld, p, n, Ri, w2, P->W, ld, w3, nullptr, 0, nullptr, 0, flags, sms, s));
+    LAUNCH(EXPM_STAGE_QR, launch_proj64(P->W, ld, p, w3, P->W, ld, p, w3, n, P->part, maxb, sms, &nb, nullptr, s));
+    LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, nb, p, 0.0, R, Ri, Rt, 1, P->H, P->ldH, hrow, hcol, nullptr, flags, s));
+    LAUNCH(EXPM_STAGE_QR, launch_mul64(P->W, ld, p, n, Ri, w3, out, ld, vnext, P->W, ld, w4, 0, flags, sms, s));
+    LAUNCH(EXPM_STAGE_QR, launch_proj64(P->W, ld, p, w4, P->W, ld, p, w4, n, P->part, maxb, sms, &nb, extra, s));
+    LAUNCH(EXPM_STAGE_QR, launch_chol(P->part, nb, p, 0.0, R, Ri, Rt, 2, P->H, P->ldH, hrow, hcol, nullptr, flags, s));
+    LAUNCH(EXPM_STAGE_QR, launch_mul64(P->W, ld, p, n, Ri, w4, out, ld, vnext, nullptr, 0, nullptr, 1, flags, sms, s));
+    return EXPM_OK;
+}
+
 // Block step j (0-based): V_j -> W = Op V_j -> V_{j+1}, H column block j.
 // Op = (tA)^{-1} (Algorithm 2) or tA (Algorithm 1).
 expm_status block_step(expm_plan* P, double t, int j, int p, int alg) {
@@ -404,6 +448,7 @@ expm_status block_step(expm_plan* P, double t, int j, int p, int alg) {
     }
     const int cols = (j + 1) * p;
     if (P->mma) return ortho_mma(P, j, p);
+    if (use64(P, p)) return ortho64(P, j, p);
     const int f32 = P->opts.precision == EXPM_PREC_MIXED ? 1 : 0;
     const int nbc = P->nblk_cgs;
     // first pass: FP64, or in the mixed path FP32 projection and double-float update (the
@@ -497,7 +542,7 @@ expm_status restart_prologue(expm_plan* P, int p, int kk, int prologue) {
     double* Vnext = P->V + (int64_t)mp * ld;
     if (prologue == 1) {
         LAUNCH(EXPM_STAGE_UPDATE, launch_copy(Vnext, ld, P->V, ld, n, p, s));
-        if (P->mma) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
+        if (P->mma || use64(P, p)) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
         return EXPM_OK;
     }
     CK(cudaMemcpyAsync(P->Pkd, P->hPk, sizeof(double) * (size_t)mp * kk, cudaMemcpyHostToDevice, s));
@@ -509,7 +554,7 @@ expm_status restart_prologue(expm_plan* P, int p, int kk, int prologue) {
     }
     LAUNCH(EXPM_STAGE_UPDATE, launch_copy(Vnext, ld, P->V + (int64_t)kk * ld, ld, n, p, s));
     LAUNCH(EXPM_STAGE_UPDATE, launch_copy(P->Vk, ld, P->V, ld, n, kk, s));
-    if (P->mma) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, kk + p, P->colexp, nullptr, s));
+    if (P->mma || use64(P, p)) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, kk + p, P->colexp, nullptr, s));
     CK(cudaMemsetAsync(P->H, 0, sizeof(double) * (size_t)P->ldH * P->opts.m * P->p_max, s));
     CK(cudaMemcpy2DAsync(P->H, sizeof(double) * P->ldH, P->hHnew, sizeof(double) * P->ldH,
                          sizeof(double) * (size_t)(kk + p), kk, cudaMemcpyHostToDevice, s));
@@ -528,6 +573,7 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
         expm_status st = restart_prologue(P, p, kk, prologue);
         if (st != EXPM_OK) return st;
     }
+    if (use64(P, p)) CK(cudaMemsetAsync(P->wexp, 0, sizeof(int) * 10 * (size_t)P->p_max, s));
     for (int j = kk / p; j < m; ++j) {
         expm_status st = block_step(P, t, j, p, alg);
         if (st != EXPM_OK) return st;
@@ -547,7 +593,7 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
     // mixed path: the product V Wc in double-float on the FP32 pipe (FP64 accumulation into Z)
     // (with deflation the restart happens in the next cycle's prologue, after V_m P_k)
     const bool defl = P->opts.k_defl > 0;
-    if (P->mma)
+    if (P->mma || use64(P, p))
         LAUNCH(EXPM_STAGE_UPDATE, launch_updz_mma(P->V, P->V32, ld, mp + p, P->Zacc, ld, p, n, sm(P, kOffWc), P->colexp,
                                                   flags_of(P->stat), defl ? 0 : 1, P->sms_rows, s));
     else LAUNCH(EXPM_STAGE_UPDATE, launch_update_z(P->V, ld, mp + p, p, n, sm(P, kOffWc), P->Zacc, ld, defl ? 0 : 1, s,
@@ -669,7 +715,7 @@ expm_status run_begin(expm_plan* P, RunState& r) {
     LAUNCH(EXPM_STAGE_OTHER, launch_copy(r.dB, r.ldb, P->W, ld, n, p, s));
     expm_status st = qr_block(P, p, P->V, ld, false, 0, 0, P->stat + 16, false);
     if (st != EXPM_OK) return st;
-    if (P->mma) LAUNCH(EXPM_STAGE_QR, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
+    if (P->mma || use64(P, p)) LAUNCH(EXPM_STAGE_QR, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
     if (fused_qr(P, p))   // the fused QR leaves R in Rt2, or in Rt3 when its third pass ran
         LAUNCH(EXPM_STAGE_OTHER, launch_init_S(sm(P, kOffRt2), p, P->npoles, P->S, s, sm(P, kOffRt3),
                                                flags_of(P->stat) + 2));
@@ -895,6 +941,7 @@ void free_plan(expm_plan* P) {
     cudaFree(P->part);
     cudaFree(P->V32);
     cudaFree(P->colexp);
+    cudaFree(P->wexp);
     cudaFree(P->partG);
     cudaFree(P->fac);
     cudaFree(P->small);
@@ -1398,6 +1445,7 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         P->proj_tc = opts->precision != EXPM_PREC_MIXED ? 0 : !ptc ? 2 : ptc[0] == '1' ? 1 : 0;
         // mixed plans run the register-streamed passes (k_mma.cu); either switch above keeps a plan
         // on the kernels it names
+        P->mma64 = opts->precision == EXPM_PREC_FP64 && mma64_fit(opts->m * p_max, p_max);
         P->mma = opts->precision == EXPM_PREC_MIXED && !tc && !ptc && mma_fit(opts->m * p_max, p_max);
         // test switch: the bound of the tensor-core kernel's waits (0 makes every wait run out)
         const char* sl = std::getenv("EXPM_TC_SPIN_LIMIT");
@@ -1556,6 +1604,8 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
             ok = ok && dalloc(&P->R64, (size_t)ld * p_max);
         }
     }
+    if (P->mma64)
+        ok = ok && dalloc(&P->colexp, (size_t)(m + 2) * p_max) && dalloc(&P->wexp, 10 * (size_t)p_max);
     if (P->mma) {
         const size_t v32 = (size_t)ld * (m + 1) * p_max;
         ok = ok && dalloc(&P->V32, v32) && dalloc(&P->colexp, (size_t)(m + 2) * p_max) &&
@@ -2009,7 +2059,10 @@ expm_status expm_arnoldi(expm_plan* plan, double t, const double* dV1, int64_t l
     CK(cudaMemsetAsync(plan->H, 0, sizeof(double) * (size_t)plan->ldH * m * plan->p_max, s));
     expm_plan* P = plan;
     LAUNCH(EXPM_STAGE_OTHER, launch_copy(dV1, ldv1, plan->V, ld, n, p, s));
-    if (P->mma) LAUNCH(EXPM_STAGE_OTHER, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
+    if (P->mma || use64(P, p)) {
+        LAUNCH(EXPM_STAGE_OTHER, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
+        if (P->wexp) CK(cudaMemsetAsync(P->wexp, 0, sizeof(int) * 10 * (size_t)P->p_max, s));
+    }
     for (int j = 0; j < m; ++j) {
         st = block_step(plan, t, j, p, EXPM_ALG_PSBFOM);
         if (st != EXPM_OK) return st;

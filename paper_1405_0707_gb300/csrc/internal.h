@@ -236,6 +236,8 @@ struct expm_plan_s {
     int sms = 0, sms_rows = 0; // SMs of the device, and the share the row passes are sized for
     float* V32 = nullptr;      // ld x (m+1) p_max   FP32 copy of V (rows n .. ld - 1 zero)
     int* colexp = nullptr;     // (m+2) p_max        largest biased exponent of each column of V
+    bool mma64 = false;        // FP64 plans: the digit passes fit (use64 decides by size)
+    int* wexp = nullptr;       // FP64 plans: 2 x 5 p_max largest exponents of W's columns
     double* partG = nullptr;   // nblkG x p_max x p_max Gram partials of the update
     int nblkG = 0;
     float* fac = nullptr;      // the block's factor for k_qr_apply
@@ -337,6 +339,17 @@ cudaError_t launch_updz_mma(double* V, float* V32, int64_t ldv, int cols, double
 cudaError_t launch_pack_block(const double* V, float* V32, int64_t ld, int64_t n, int p, int* colexp, const int* skip,
                               cudaStream_t s);
 cudaError_t mma_set_smem_limits();
+// The same passes to FP64 rounding for FP64 plans (k_mma.cu)
+bool mma64_fit(int mp, int p);
+cudaError_t launch_upd64(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,
+                         int* colexp, int* oexp, int* flags, int sms, cudaStream_t s);
+cudaError_t launch_mul64(double* W, int64_t ldw, int p, int64_t n, const double* Rinv, int* wexp, double* out, int64_t ldo,
+                         int* oexp, double* alt, int64_t ldalt, int* altexp, int third, int* flags, int sms, cudaStream_t s);
+cudaError_t launch_proj64(const double* V, int64_t ldv, int cols, const int* vexp, const double* W, int64_t ldw, int p,
+                          const int* wexp, int64_t n, double* part, int max_blocks, int sms, int* nb, const int* only,
+                          cudaStream_t s);
+cudaError_t launch_colmax(const double* W, int64_t ldw, int p, int64_t n, int* wexp, int* zero0, int n0, int* zero1, int n1,
+                          cudaStream_t s);
 // The Cholesky-QR step after the second projection (rows_qr.cuh)
 cudaError_t launch_reduce_factor(const double* part, int nblk, const double* partG, int nblkG, int cols, int p, double* h,
                                  double* H, int ldH, int hrow, int hcol, double* R, double* Rtot, float* fac,

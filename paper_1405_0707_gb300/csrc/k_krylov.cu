@@ -23,6 +23,7 @@ namespace {
 
 constexpr int NT = 256;     // threads per CTA for the row passes
 
+
 // Load a TR x cols tile of column-major X (rows r0.., ld) into S[rr * cs + a], zero-filled,
 // converted to the tile's element type.
 template <typename T>
@@ -438,6 +439,7 @@ __global__ void __launch_bounds__(NT) k_update_df(const double* __restrict__ V, 
 // on entry (a zero right-hand side column, or the image of one) get zero rows in R and stay
 // zero, so such blocks pass through without a division by zero.
 constexpr int CHOL_T = 1024;
+constexpr int kCholF = 256;     // threads of the factorisation after the sum
 __global__ void __launch_bounds__(CHOL_T) k_chol(const double* __restrict__ part, int nblk, int p,
                                                  double shift_rel, double* R, double* Rinv,
                                                  double* Rtot, int mode, double* H, int ldH,
@@ -451,17 +453,25 @@ __global__ void __launch_bounds__(CHOL_T) k_chol(const double* __restrict__ part
     __shared__ double red[CHOL_T];
     __shared__ double rdiag[kMaxP];
     __shared__ int bad, ill;
+    __shared__ double tr_s, dmax_s;
     const int pp = p * p;
     {
         const int stripes = pp >= CHOL_T ? 1 : CHOL_T / pp;
         for (int base = 0; base < pp; base += CHOL_T / stripes) {
             const int ol = threadIdx.x % (CHOL_T / stripes), st = threadIdx.x / (CHOL_T / stripes);
             const int o = base + ol;
+            const int w = CHOL_T / stripes, grp = (stripes + 7) / 8;   // up to eight groups of stripes
             red[threadIdx.x] = (o < pp && st < stripes) ? stripe_sum(part, nblk, pp, o, st, stripes) : 0.0;
+            __syncthreads();
+            double s1 = 0.0;
+            if (st < 8)
+                for (int k = st * grp; k < min(stripes, (st + 1) * grp); ++k) s1 += red[k * w + ol];
+            __syncthreads();
+            if (st < 8) red[threadIdx.x] = s1;
             __syncthreads();
             if (st == 0 && o < pp) {
                 double s = 0.0;
-                for (int k = 0; k < stripes; ++k) s += red[k * (CHOL_T / stripes) + ol];
+                for (int k = 0; k < min(8, (stripes + grp - 1) / grp); ++k) s += red[k * w + ol];
                 G0[o] = s;
             }
             __syncthreads();
@@ -470,7 +480,7 @@ __global__ void __launch_bounds__(CHOL_T) k_chol(const double* __restrict__ part
     const bool last = (mode == 1 && *extra == 0) || mode == 2;
     __shared__ double hn2[kMaxP];
     if (H && last) {
-        const int stripes = CHOL_T / p;
+        const int stripes = min(16, CHOL_T / p);     // few: their sum is a chain of FP64 adds
         const int c = threadIdx.x % p, st = threadIdx.x / p;
         double v2 = 0.0;
         if (st < stripes)
@@ -487,102 +497,153 @@ __global__ void __launch_bounds__(CHOL_T) k_chol(const double* __restrict__ part
         }
         __syncthreads();
     }
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
-    if (lane == 0) { bad = 0; ill = 0; }
-    double tr = 0.0, dmax = 0.0;
-    for (int c = 0; c < p; ++c) {
-        tr += G0[c * p + c];
-        dmax = fmax(dmax, G0[c * p + c]);
+    // The factorisation by kCholF threads: thread t holds entries t, t + kCholF, .. of the upper triangle
+    // in registers.  Step j reads row j of the partly reduced matrix and the pivot's inverse root from
+    // shared memory; the owners of row j + 1 publish it, the diagonal's owner with its inverse root, and
+    // the inverse of R is built by doubling (p = 8: 28 us with one warp's column sweep, 25 us now; a
+    // float-pair factor of the same matrix measured no faster: the launch is bound by its serial chain of
+    // loads, barriers and cold instruction fetches, not by FP64 latency).
+    const int tid = threadIdx.x, ne = p * (p + 1) / 2;
+    if (tid >= kCholF) return;
+    constexpr int KE = (kMaxP * (kMaxP + 1) / 2 + kCholF - 1) / kCholF;
+    int ei[KE], ek[KE];
+#pragma unroll
+    for (int q = 0; q < KE; ++q) {
+        const int e = tid + q * kCholF;
+        ei[q] = -1;
+        ek[q] = 0;
+        if (e < ne) {
+            int i = 0, rem = e;
+            while (rem >= p - i) {
+                rem -= p - i;
+                ++i;
+            }
+            ei[q] = i;
+            ek[q] = i + rem;
+        }
     }
-    if (normsq_out && lane == 0 && mode == 0) *normsq_out = tr;
+    auto bar = [] { asm volatile("bar.sync 1, %0;" ::"n"(kCholF) : "memory"); };
+    if (tid < 32) {
+        double tr = tid < p ? G0[tid * p + tid] : 0.0, dm = tr;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            tr += __shfl_xor_sync(0xffffffffu, tr, o);
+            dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+        }
+        if (tid == 0) {
+            bad = 0;
+            ill = 0;
+            tr_s = tr;
+            dmax_s = dm;
+            if (normsq_out && mode == 0) *normsq_out = tr;
+        }
+    }
+    bar();
     for (int attempt = 0; attempt < 2; ++attempt) {
-        const double shift = (attempt == 1) ? shift_rel * tr : 0.0;
-        for (int o = lane; o < pp; o += 32) {
-            G[o] = G0[o] + ((o / p == o % p) ? shift : 0.0);
+        const double shift = (attempt == 1) ? shift_rel * tr_s : 0.0;
+        double ge[KE];
+        // the pivot of column j: its root into Rs, its inverse root into rdiag
+        auto pivot = [&](int j, double d) {
+            if (G0[j * p + j] == 0.0) {
+                // an exactly zero column (an invariant subspace reached earlier): R row j and R^{-1}
+                // row and column j stay zero, so the column stays zero
+                Rs[j * p + j] = 0.0;
+                rdiag[j] = 0.0;
+                return;
+            }
+            if (!(d > 0.0) || !isfinite(d) || (mode == 0 && attempt == 0 && d < 1e-10 * dmax_s)) ill = 1;
+            if (!(d > 0.0) || !isfinite(d)) d = 1.0;
+            const double inv = rsqrt(d);
+            Rs[j * p + j] = d * inv;
+            rdiag[j] = inv;
+        };
+        for (int o = tid; o < pp; o += kCholF) {
             Rs[o] = 0.0;
             Ri[o] = 0.0;
         }
-        __syncwarp();
-        // right-looking upper Cholesky G = R^T R (upper part), one reciprocal per pivot
-        for (int j = 0; j < p; ++j) {
-            if (lane == 0) {
-                double d = G[j * p + j];
-                if (G0[j * p + j] == 0.0) {
-                    // an exactly zero column (an invariant subspace reached earlier): R row j
-                    // and R^{-1} row and column j stay zero, so the column stays zero
-                    Rs[j * p + j] = 0.0;
-                    rdiag[j] = 0.0;
-                } else {
-                    if (!(d > 0.0) || !isfinite(d) || (mode == 0 && attempt == 0 && d < 1e-10 * dmax)) ill = 1;
-                    if (!(d > 0.0) || !isfinite(d)) d = 1.0;
-                    const double rj = sqrt(d);
-                    Rs[j * p + j] = rj;
-                    rdiag[j] = 1.0 / rj;
+        bar();
+#pragma unroll
+        for (int q = 0; q < KE; ++q)
+            if (ei[q] >= 0) {
+                ge[q] = G0[ei[q] * p + ek[q]] + (ei[q] == ek[q] ? shift : 0.0);
+                if (ei[q] == 0) {
+                    G[ek[q]] = ge[q];
+                    if (ek[q] == 0) pivot(0, ge[q]);
                 }
             }
-            __syncwarp();
+        bar();
+#pragma unroll 1
+        for (int j = 0; j < p; ++j) {
             const double inv = rdiag[j];
-            if (lane > j && lane < p) Rs[j * p + lane] = G[j * p + lane] * inv;
-            __syncwarp();
-            if (lane > j && lane < p) {
-                const double rb = Rs[j * p + lane];
-                for (int a = j + 1; a <= lane; ++a) G[a * p + lane] -= Rs[j * p + a] * rb;
+#pragma unroll
+            for (int q = 0; q < KE; ++q) {
+                if (q * kCholF >= ne) break;
+                if (ei[q] >= j && ei[q] >= 0) {
+                    if (ei[q] == j) {
+                        if (ek[q] > j) Rs[j * p + ek[q]] = ge[q] * inv;
+                    } else {
+                        ge[q] = fma(-(G[j * p + ei[q]] * inv), G[j * p + ek[q]] * inv, ge[q]);
+                        if (ei[q] == j + 1) {
+                            G[(j + 1) * p + ek[q]] = ge[q];
+                            if (ek[q] == j + 1) pivot(j + 1, ge[q]);
+                        }
+                    }
+                }
             }
-            __syncwarp();
+            bar();
         }
         if (mode != 0 || attempt == 1 || !ill) break;   // mode 0 retries with the shift
-        __syncwarp();
+        bar();
     }
-    if (mode == 0 && lane == 0) *extra = ill;
-    if (mode != 0 && lane == 0 && ill) bad = 1;       // a later pass must factor cleanly
-    __syncwarp();
-    // inverse of the upper triangular R, column `lane` (reciprocal pivots, no division)
-    if (lane < p) {
-        const int c = lane;
-        Ri[c * p + c] = rdiag[c];
-        for (int r = c - 1; r >= 0; --r) {
-            double s = 0.0;
-            for (int k = r + 1; k <= c; ++k) s = fma(Rs[r * p + k], Ri[k * p + c], s);
-            Ri[r * p + c] = -s * rdiag[r];
-        }
-    }
-    __syncwarp();
-    // Rtot = R * Rtot_old (upper triangular product), column `lane`
-    if (lane < p) {
-        const int c = lane;
-        for (int r = 0; r < p; ++r) {
-            double s;
-            if (mode == 0) s = Rs[r * p + c];
-            else {
-                s = 0.0;
-                for (int k = r; k <= c; ++k) s = fma(Rs[r * p + k], Rtot[k * p + c], s);
+    if (mode == 0 && tid == 0) *extra = ill;
+    if (mode != 0 && tid == 0 && ill) bad = 1;          // a later pass must factor cleanly
+    // inverse of the upper triangular R by doubling: diagonal blocks of size s joined two by two
+    for (int c = tid; c < p; c += kCholF) Ri[c * p + c] = rdiag[c];
+    bar();
+    for (int s = 1; s < p; s *= 2)
+        for (int ph = 0; ph < 2; ++ph) {
+            for (int e = tid; e < p * s; e += kCholF) {
+                const int b0 = e / (2 * s * s) * 2 * s, o = e % (2 * s * s), r = b0 + o / s, c = b0 + s + o % s;
+                if (o < s * s && c < p) {
+                    double t = 0.0;
+                    if (ph == 0) {
+                        for (int k = b0 + s; k <= c; ++k) t = fma(-Rs[r * p + k], Ri[k * p + c], t);   // -B C^-1
+                        Rt[r * p + c] = t;
+                    } else {
+                        for (int k = r; k < b0 + s; ++k) t = fma(Ri[r * p + k], Rt[k * p + c], t);      // A^-1 (-B C^-1)
+                        Ri[r * p + c] = t;
+                    }
+                }
             }
-            Rt[r * p + c] = (r <= c) ? s : 0.0;
+            bar();
         }
+    // Rtot = R Rtot_old (upper triangular product)
+    for (int o = tid; o < pp; o += kCholF) {
+        const int r = o / p, c = o % p;
+        double s;
+        if (mode == 0) s = Rs[o];
+        else {
+            s = 0.0;
+            for (int k = r; k <= c; ++k) s = fma(Rs[r * p + k], Rtot[k * p + c], s);
+        }
+        Rt[o] = (r <= c) ? s : 0.0;
     }
-    __syncwarp();
-    for (int o = lane; o < pp; o += 32) {
+    bar();
+    for (int o = tid; o < pp; o += kCholF) {
         R[o] = Rs[o];
         Rinv[o] = Ri[o];
         Rtot[o] = Rt[o];
         if (!isfinite(Rt[o])) bad = 1;
+        if (H && last) H[(int64_t)(hcol + o % p) * ldH + hrow + o / p] = Rt[o];
     }
-    __syncwarp();
-    if (H && last) {
-        for (int o = lane; o < pp; o += 32) {
-            const int a = o / p, c = o % p;
-            H[(int64_t)(hcol + c) * ldH + hrow + a] = Rt[o];
-        }
-        if (lane < p) {
-            const int c = lane;
-            double n0 = hn2[c];
-            for (int a = 0; a <= c; ++a) n0 += Rt[a * p + c] * Rt[a * p + c];
-            if (Rt[c * p + c] <= 1e-14 * sqrt(n0)) atomicOr(&flags[1], 1);
-        }
+    if (H && last && tid < p) {
+        const int c = tid;
+        double n0 = hn2[c];
+        for (int a = 0; a <= c; ++a) n0 += Rt[a * p + c] * Rt[a * p + c];
+        if (Rt[c * p + c] <= 1e-14 * sqrt(n0)) atomicOr(&flags[1], 1);
     }
-    __syncwarp();
-    if (lane == 0 && bad) atomicOr(&flags[0], 1);
+    bar();
+    if (tid == 0 && bad) atomicOr(&flags[0], 1);
 }
 
 // W_out = W R^{-1} (row by row); gram: also partial of W_out^T W_out.

@@ -224,18 +224,24 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
 }
 
 // ---------------------------------------------------------------- digits
-// The seven balanced base-256 digits of v 2^(1022 - emax) (magnitude below 1; c9 = 9 + emax), as
-// the bytes of Y = X + bias with X the two's-complement value times 2^55: the top 16 bits of Y
-// read as fp16 are 1152 + d_0, and 0x6400 | byte is 1152 + d_i below.
-__device__ __forceinline__ void digits_y(double v, int c9, uint32_t& yl, uint32_t& yh) {
+// The NV balanced base-256 digits of v 2^(1022 - emax) (magnitude below 1; c = digit_shift<NV>() + emax),
+// as the bytes of Y = X + bias with X the two's-complement value times 2^55 (seven digits: the top 16 bits
+// of Y read as fp16 are 1152 + d_0) or 2^62 (eight); 0x6400 | byte read as fp16 is 1152 + d_i.
+template <int NV>
+__device__ constexpr int digit_shift() { return NV == 7 ? 9 : 2; }
+
+constexpr int kNoExp = 1 << 20;      // the shift of an all-zero column: every digit is zero
+
+template <int NV>
+__device__ __forceinline__ void digits_y(double v, int c, uint32_t& yl, uint32_t& yh) {
     const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    const uint32_t s = (uint32_t)(c9 - (int)((hi >> 20) & 0x7FFu));
+    const uint32_t s = (uint32_t)(c - (int)((hi >> 20) & 0x7FFu));
     const uint32_t mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
     unsigned long long X = ((unsigned long long)mh << 32) | ml;
     asm("shr.u64 %0, %0, %1;" : "+l"(X) : "r"(s));            // shifts of 64 and more give zero
     const int sg = (int)hi >> 31;
     const unsigned long long S = (unsigned long long)(long long)sg;
-    X = (X ^ S) + (0x6480808080808080ull - S);
+    X = (X ^ S) + ((NV == 7 ? 0x6480808080808080ull : 0x8080808080808080ull) - S);
     yl = (uint32_t)X;
     yh = (uint32_t)(X >> 32);
 }
@@ -245,12 +251,14 @@ __device__ __forceinline__ uint32_t unbias(uint32_t x) {      // (1152 + d) - 11
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(0xE480E480u));
     return r;
 }
-// digit I of the pair (x in the low half, y in the high half)
-template <int I>
+// digit I of the pair (x in the low half, y in the high half): byte NV - 1 - I of Y
+template <int NV, int I>
 __device__ __forceinline__ uint32_t digit_pair(uint32_t xl, uint32_t xh, uint32_t yl, uint32_t yh) {
-    if constexpr (I == 0) return unbias(__byte_perm(xh, yh, 0x7632));
-    const uint32_t z = I <= 2 ? __byte_perm(xh, yh, 0x5410) : I <= 4 ? __byte_perm(xl, yl, 0x7632) : __byte_perm(xl, yl, 0x5410);
-    if constexpr (I % 2 == 0) return unbias((z & 0x00FF00FFu) | 0x64006400u);
+    if constexpr (NV == 7 && I == 0) return unbias(__byte_perm(xh, yh, 0x7632));
+    constexpr int B = NV - 1 - I;                              // byte of Y
+    const uint32_t z = B >= 6 ? __byte_perm(xh, yh, 0x7632) : B >= 4 ? __byte_perm(xh, yh, 0x5410)
+                       : B >= 2 ? __byte_perm(xl, yl, 0x7632) : __byte_perm(xl, yl, 0x5410);
+    if constexpr (B % 2 == 0) return unbias((z & 0x00FF00FFu) | 0x64006400u);
     return unbias(__byte_perm(z, 0x64646464u, 0x4341));
 }
 
@@ -275,8 +283,23 @@ __device__ __forceinline__ double scaled_int(long long X, int k) {
     return __longlong_as_double((long long)(b | (X < 0 ? 1ull << 63 : 0ull)));
 }
 
+// L_0 + L_1 2^-8 + .. + L_7 2^-56 = x + y, the level sums exact integers below 2^24: three groups summed
+// exactly in float pairs (40 bits each), joined in FP64
+__device__ __forceinline__ void level_sum64(float l0, float l1, float l2, float l3, float l4, float l5, float l6, float l7,
+                                            double& x, double& y) {
+    float ah = l2 * 0x1p-16f, al = 0.f;
+    df_add(ah, al, l1 * 0x1p-8f);
+    df_add(ah, al, l0);
+    float bh = l5 * 0x1p-40f, bl = 0.f;
+    df_add(bh, bl, l4 * 0x1p-32f);
+    df_add(bh, bl, l3 * 0x1p-24f);
+    const float lo = bl + fmaf(l7, 0x1p-56f, l6 * 0x1p-48f);
+    x = f64_of_f32_i(ah);
+    y = (f64_of_f32_i(lo) + f64_of_f32_i(bh)) + f64_of_f32_i(al);
+}
+
 constexpr int kUpdThreads = 128;
-__host__ __device__ constexpr int upd_seg(int NH) { return NH == 4 ? 15 : 10; }   // 16-column chunks per exact segment
+__host__ __device__ constexpr int upd_seg(int NH) { return NH == 4 ? 15 : NH == 6 ? 10 : 8; }   // 16-column chunks per exact segment
 __host__ __device__ constexpr int gram_rounds(int NT) { return NT == 1 ? 5 : NT == 2 ? 5 : 17; }
 __host__ __device__ constexpr int gram_split(int NT) { return NT == 1 ? 4 : 1; }   // lanes sharing one Gram entry
 
@@ -286,20 +309,63 @@ constexpr size_t upd_smem(int cols, int NT, int NH, bool gram) {
            (gram ? sizeof(float2) * (size_t)std::max((kUpdThreads / 32) * 16 * (8 * NT + 1), gram_rounds(NT) * 128) : 0);
 }
 
-// GS (NH = 4): W <- W - V h with h rounded as described at the top; CTA 0 records the rounded h in
-// H (columns hcol .., rows 0 .. cols - 1) and clears the next block's colexp; the Gram matrix of
-// the updated W in float pairs goes to partG[blk][p][p].
-// Z (NH = 6): Z <- Z + V Wc (sgn = 1), then the restart copy V[:, 0:p] <- V[:, cols-p:cols] of this
-// CTA's rows (and of V32) when asked.
+enum UpdMode { U_GS = 0, U_Z = 1, U_GS64 = 2, U_Z64 = 3, U_MUL64 = 4 };
+
+// U_GS (NV = 7, NH = 4): W <- W - V h with h rounded as described at the top; CTA 0 records the rounded h
+// in H (columns hcol .., rows 0 .. cols - 1) and clears the next block's colexp; the Gram matrix of the
+// updated W in float pairs goes to partG[blk][p][p].
+// U_Z (7, 6): Z <- Z + V Wc, then the restart copy V[:, 0:p] <- V[:, cols-p:cols] of this CTA's rows (and
+// of V32) when asked.
+// U_GS64, U_Z64 (8, 8): the same products to FP64 rounding for FP64 plans (both operands to 2^-62 of
+// their column's largest entry, no Gram matrix, h not rounded).
+// U_MUL64 (8, 8): out <- V h, V a p-column block (W <- W R^-1; out may be V), by pass as in TrsmPass.
+// U_GS64 and U_MUL64 collect the largest exponent of each result column in oexp.
 // MMA: M = 16 rows (lane group g holds rows 2g and 2g + 1, one 16-byte load per column), N = 8
 // block columns, K = 16 basis columns (lane t holds columns 4t .. 4t + 3).  One warp per 16-row
 // tile, the next chunk's loads in flight.  44 MMAs per 256 basis elements at p = 16 take about as
 // long as the elements' 8 bytes at the memory rate.
-template <int NT, int NH, bool GS>
+struct UpdArgs {
+    double* V;
+    int64_t ldv;
+    int cols;
+    double* W;
+    int64_t ldw;
+    int p;
+    int64_t n;
+    const double* h;
+    int* colexp;
+    double* partG;
+    double* H;
+    int ldH, hcol;
+    int* flags;
+    float* V32;
+    int restart;
+    int* oexp;
+    const int* skip;       // return at once when *skip != 0 (== 0 for skip_zero)
+    int skip_zero;
+    double* alt;           // U_MUL64: the destination when flags[2] is set (alternative to W)
+    int64_t ldalt;
+    int* altexp;
+};
+
+template <int NT, int NV, int NH, int MODE>
 __global__ void __launch_bounds__(kUpdThreads, NT == 4 ? 2 : NT == 2 ? 3 : 4)
-k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* __restrict__ h,
-          int* __restrict__ colexp, double* __restrict__ partG, double* __restrict__ H, int ldH, int hcol,
-          int* flags, float* V32, int restart) {
+k_upd_mma(const UpdArgs A) {
+    constexpr bool GS = MODE == U_GS, D64 = NV == 8;
+    if (A.skip && ((*A.skip != 0) != (A.skip_zero != 0))) return;
+    double* const V = A.V;
+    const int64_t ldv = A.ldv, n = A.n;
+    const int cols = A.cols, p = A.p;
+    double* W = A.W;
+    int64_t ldw = A.ldw;
+    int* oexp = A.oexp;
+    if (MODE == U_MUL64 && A.alt && A.flags[2]) {
+        W = A.alt;
+        ldw = A.ldalt;
+        oexp = A.altexp;
+    }
+    const double* __restrict__ h = A.h;
+    int* const colexp = A.colexp;
     extern __shared__ __align__(16) unsigned char smu[];
     const int nk = (cols + 15) >> 4;
     const int64_t ntiles = (n + 15) >> 4;
@@ -319,7 +385,10 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
     __shared__ int fmax_s[8 * NT], bad_s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     constexpr int NCOL = 8 * NT;
-    for (int a = tid; a < nk * 16; a += kUpdThreads) c9s[a] = 9 + (a < cols ? colexp[a] : 0);
+    for (int a = tid; a < nk * 16; a += kUpdThreads) {
+        const int em = a < cols ? colexp[a] : 0;
+        c9s[a] = em > 0 ? digit_shift<NV>() + em : kNoExp;
+    }
     if (tid < NCOL) fmax_s[tid] = -100000;
     if (tid == 0) bad_s = 0;
     __syncthreads();
@@ -330,13 +399,13 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
         if (c < p) {
             const int E = (int)(((unsigned)__double2hiint(h[a * p + c]) >> 20) & 0x7FFu);
             if (E == 0x7FF) bad_s = 1;
-            const int em = c9s[a] - 9;
-            if (E > 0 && em > 0) atomicMax(&fmax_s[c], E - 1022 + em - 1022);
+            const int em = c9s[a] - digit_shift<NV>();
+            if (E > 0 && em < 4096) atomicMax(&fmax_s[c], E - 1022 + em - 1022);
         }
     }
     __syncthreads();
-    if (tid == 0 && bad_s) atomicOr(&flags[0], 1);
-    constexpr int SC = 8 * NH - 1;
+    if (tid == 0 && bad_s) atomicOr(&A.flags[0], 1);
+    constexpr int SC = D64 ? 62 : 8 * NH - 1;
     for (int e = tid; e < nk * 16 * NCOL; e += kUpdThreads) {
         const int a = e / NCOL, c = e - a * NCOL;
         long long X = 0;
@@ -344,17 +413,17 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
         if (a < cols && c < p) {
             const double hv = h[a * p + c];
             const unsigned long long b = (unsigned long long)__double_as_longlong(hv);
-            const int E = (int)((b >> 52) & 0x7FF), em = c9s[a] - 9, f = fmax_s[c];
+            const int E = (int)((b >> 52) & 0x7FF), em = c9s[a] - digit_shift<NV>(), f = fmax_s[c];
             // |h| 2^(em - 1022) 2^(SC - f) = m 2^-sh, rounded to nearest
             sh = 1075 - E + 1022 - em + f - SC;
-            if (E > 0 && em > 0 && sh <= 54) {
+            if (E > 0 && em < 4096 && sh <= 54) {
                 const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-                X = (long long)((m + (1ull << (sh - 1))) >> sh);
+                X = sh > 0 ? (long long)((m + (1ull << (sh - 1))) >> sh) : (long long)(m << -sh);
                 if (b >> 63) X = -X;
             }
             if (GS && blockIdx.x == 0) {
                 // the h that is applied, exactly: X 2^(f - SC) 2^(1022 - em)
-                H[(int64_t)(hcol + c) * ldH + a] = scaled_int(X, f - SC + 1022 - em);
+                A.H[(int64_t)(A.hcol + c) * A.ldH + a] = scaled_int(X, f - SC + 1022 - em);
             }
         }
         const int kc = a >> 4, kk = a & 15;
@@ -374,6 +443,9 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
     }
     __syncthreads();
 
+    uint32_t omax[NT][2];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) omax[j][0] = omax[j][1] = 0u;
     constexpr int GK = GS ? gram_rounds(NT) : 1, GSP = gram_split(NT);
     const int ne = p * (p + 1) / 2;
     float gh[GK], gl[GK];
@@ -400,9 +472,9 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
         double w[NT][4];                         // [nt]: (2g, c) (2g, c + 1) (2g + 1, c) (2g + 1, c + 1)
         for (int k0 = 0; k0 < nk; k0 += upd_seg(NH)) {
             const int k1 = min(nk, k0 + upd_seg(NH));
-            float acc[7][NT][4];
+            float acc[NV][NT][4];
 #pragma unroll
-            for (int l = 0; l < 7; ++l)
+            for (int l = 0; l < NV; ++l)
 #pragma unroll
                 for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -410,14 +482,14 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
             for (int kc = k0; kc < k1; ++kc) {
                 uint32_t yl[4][2], yh[4][2];
                 const int4 c9 = *reinterpret_cast<const int4*>(c9s + kc * 16 + 4 * t);
-                digits_y(v[0].x, c9.x, yl[0][0], yh[0][0]);
-                digits_y(v[0].y, c9.x, yl[0][1], yh[0][1]);
-                digits_y(v[1].x, c9.y, yl[1][0], yh[1][0]);
-                digits_y(v[1].y, c9.y, yl[1][1], yh[1][1]);
-                digits_y(v[2].x, c9.z, yl[2][0], yh[2][0]);
-                digits_y(v[2].y, c9.z, yl[2][1], yh[2][1]);
-                digits_y(v[3].x, c9.w, yl[3][0], yh[3][0]);
-                digits_y(v[3].y, c9.w, yl[3][1], yh[3][1]);
+                digits_y<NV>(v[0].x, c9.x, yl[0][0], yh[0][0]);
+                digits_y<NV>(v[0].y, c9.x, yl[0][1], yh[0][1]);
+                digits_y<NV>(v[1].x, c9.y, yl[1][0], yh[1][0]);
+                digits_y<NV>(v[1].y, c9.y, yl[1][1], yh[1][1]);
+                digits_y<NV>(v[2].x, c9.z, yl[2][0], yh[2][0]);
+                digits_y<NV>(v[2].y, c9.z, yl[2][1], yh[2][1]);
+                digits_y<NV>(v[3].x, c9.w, yl[3][0], yh[3][0]);
+                digits_y<NV>(v[3].y, c9.w, yl[3][1], yh[3][1]);
                 if (kc + 1 < nk) load(tile, kc + 1);
                 else if (tile + tstep < ntiles) load(tile + tstep, 0);
                 uint4 b[NH / 2][NT];
@@ -429,13 +501,13 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
                 auto level = [&](auto ic) {
                     constexpr int I = decltype(ic)::value;
                     uint32_t a[4];
-                    a[0] = digit_pair<I>(yl[0][0], yh[0][0], yl[1][0], yh[1][0]);
-                    a[1] = digit_pair<I>(yl[0][1], yh[0][1], yl[1][1], yh[1][1]);
-                    a[2] = digit_pair<I>(yl[2][0], yh[2][0], yl[3][0], yh[3][0]);
-                    a[3] = digit_pair<I>(yl[2][1], yh[2][1], yl[3][1], yh[3][1]);
+                    a[0] = digit_pair<NV, I>(yl[0][0], yh[0][0], yl[1][0], yh[1][0]);
+                    a[1] = digit_pair<NV, I>(yl[0][1], yh[0][1], yl[1][1], yh[1][1]);
+                    a[2] = digit_pair<NV, I>(yl[2][0], yh[2][0], yl[3][0], yh[3][0]);
+                    a[3] = digit_pair<NV, I>(yl[2][1], yh[2][1], yl[3][1], yh[3][1]);
 #pragma unroll
                     for (int jj = 0; jj < NH; ++jj)
-                        if (I + jj <= 6) {
+                        if (I + jj < NV) {
 #pragma unroll
                             for (int j = 0; j < NT; ++j) {
                                 const uint4 bq = b[jj >> 1][j];
@@ -450,6 +522,7 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
                 level(std::integral_constant<int, 4>{});
                 level(std::integral_constant<int, 5>{});
                 level(std::integral_constant<int, 6>{});
+                if constexpr (NV == 8) level(std::integral_constant<int, 7>{});
             }
             if (k0 == 0) {
 #pragma unroll
@@ -458,7 +531,7 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
                     for (int q = 0; q < 2; ++q) {
                         const int c = 8 * j + 2 * t + q;
                         double2 x = make_double2(0.0, 0.0);
-                        if (c < p) {
+                        if (MODE != U_MUL64 && c < p) {
                             if (r + 1 < n) x = *reinterpret_cast<const double2*>(W + (int64_t)c * ldw + r);
                             else if (r < n) x.x = W[(int64_t)c * ldw + r];
                         }
@@ -466,22 +539,40 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
                         w[j][2 + q] = x.y;
                     }
             }
-            // S = sum_l L_l 2^(-8 l) by Horner in a float pair; the product is S 2^(f - 14)
+            // S = sum_l L_l 2^(-8 l); the product is S 2^(f - 14) (2^(f - 12) with eight digits)
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    float sh = acc[6][j][q], sl = 0.f;
+                    const int k = fmax_s[8 * j + 2 * t + (q & 1)] - (D64 ? 12 : 14);
+                    constexpr bool SUB = MODE == U_GS || MODE == U_GS64;
+                    if constexpr (!D64) {
+                        // Horner in a float pair
+                        float sh = acc[6][j][q], sl = 0.f;
 #pragma unroll
-                    for (int l = 5; l >= 0; --l) {
-                        sh *= 0x1p-8f;
-                        sl *= 0x1p-8f;
-                        df_add(sh, sl, acc[l][j][q]);
+                        for (int l = 5; l >= 0; --l) {
+                            sh *= 0x1p-8f;
+                            sl *= 0x1p-8f;
+                            df_add(sh, sl, acc[l][j][q]);
+                        }
+                        const double x = scale2_e(f64_of_f32_i(sh), k), y = scale2_e(f64_of_f32_i(sl), k);
+                        w[j][q] = SUB ? (w[j][q] - x) - y : (w[j][q] + x) + y;
+                    } else {
+                        double x, y;
+                        level_sum64(acc[0][j][q], acc[1][j][q], acc[2][j][q], acc[3][j][q], acc[4][j][q], acc[5][j][q],
+                                    acc[6][j][q], acc[7][j][q], x, y);
+                        x = scale2_e(x, k);
+                        y = scale2_e(y, k);
+                        w[j][q] = SUB ? (w[j][q] - x) - y : (w[j][q] + x) + y;
                     }
-                    const int k = fmax_s[8 * j + 2 * t + (q & 1)] - 14;
-                    const double x = scale2_e(f64_of_f32_i(sh), k), y = scale2_e(f64_of_f32_i(sl), k);
-                    w[j][q] = GS ? (w[j][q] - x) - y : (w[j][q] + x) + y;
                 }
+        }
+        if constexpr (MODE == U_GS64 || MODE == U_MUL64) {
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (r + (q >> 1) < n) omax[j][q & 1] = max(omax[j][q & 1], (uint32_t)__double2hiint(w[j][q]) & 0x7FFFFFFFu);
         }
 #pragma unroll
         for (int j = 0; j < NT; ++j)
@@ -520,15 +611,27 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
                     df_add(gh[k], gl[k], sh);
                     gl[k] += sl;
                 }
-        } else if (restart) {
+        } else if ((MODE == U_Z || MODE == U_Z64) && A.restart) {
             __syncwarp();
             const int64_t rr = tile * 16 + 2 * (lane & 7);
             for (int c = lane >> 3; c < p; c += 4) {
                 const int64_t so = (int64_t)(cols - p + c) * ldv + rr, dof = (int64_t)c * ldv + rr;
                 *reinterpret_cast<double2*>(V + dof) = *reinterpret_cast<const double2*>(V + so);
-                *reinterpret_cast<float2*>(V32 + dof) = *reinterpret_cast<const float2*>(V32 + so);
+                if (MODE == U_Z) *reinterpret_cast<float2*>(A.V32 + dof) = *reinterpret_cast<const float2*>(A.V32 + so);
             }
         }
+    }
+    if constexpr (MODE == U_GS64 || MODE == U_MUL64) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t m = omax[j][q];
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
+                const int c = 8 * j + 2 * t + q;
+                if (g == 0 && c < p && m) atomicMax(&oexp[c], (int)(m >> 20));
+            }
     }
     if (GS) {
         __syncthreads();
@@ -538,7 +641,7 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
         for (int k = 0; k < GK; ++k)
             if (32 * k < ne * GSP) red[(k * 4 + warp) * 32 + lane] = make_float2(gh[k], gl[k]);
         __syncthreads();
-        double* out = partG + (int64_t)blockIdx.x * p * p;
+        double* out = A.partG + (int64_t)blockIdx.x * p * p;
         for (int e = tid; e < p * p; e += kUpdThreads) {
             int i = e / p, j = e % p;
             if (i > j) {
@@ -562,6 +665,201 @@ k_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64
     }
 }
 
+// ---------------------------------------------------------------- projection to FP64 rounding
+// FP64 plans: partial[bx][a][c] = sum over the rows of row group bx of V[r, a] W[r, c], both operands in
+// eight digits of their column's scale (2^-62 of its largest entry), the 36 digit products of levels 0..7
+// summed exactly over 128 rows and joined in FP64: 3 FP64 adds per output and 128 rows where the FP64
+// kernel spends 128 FMAs on a pipe that retires two per SM and clock.  MMA: M = 16 basis columns, N = 8
+// block columns, K = 16 rows, lanes and units as in k_proj_mma; a warp owns one M tile.
+constexpr size_t proj64_smem(int NT) { return (size_t)2 * kProjKb * NT * 8 * 32 * sizeof(uint2); }
+
+template <int NT>
+__global__ void __launch_bounds__(256, NT == 1 ? 2 : 1)
+k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restrict__ vexp, const double* __restrict__ W,
+         int64_t ldw, int p, const int* __restrict__ wexp, int64_t n, double* __restrict__ part, int CG, const int* only) {
+    if (only && *only == 0) return;
+    extern __shared__ __align__(16) unsigned char smq[];
+    uint2* wf = reinterpret_cast<uint2*>(smq);             // [buf][kb][nt][digit][lane]
+    constexpr int WBUF = kProjKb * NT * 8 * 32;
+    __shared__ double red[8][32][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int RG = 8 / CG, cg = warp % CG, rg = warp / CG;
+    const int mt_all = (cols + 15) >> 4, mt = blockIdx.y * CG + cg;
+    const bool work = rg < RG && mt < mt_all;
+    const int a0 = min(mt * 16 + g, cols - 1), a1 = min(mt * 16 + g + 8, cols - 1);
+    auto shift_of = [](int em) { return em > 0 ? digit_shift<8>() + em : kNoExp; };
+    const int cv0 = shift_of(vexp[a0]), cv1 = shift_of(vexp[a1]);
+    const int64_t nblk = (n + 15) >> 4, units = (nblk + kProjKb - 1) / kProjKb;
+    int cw[NT];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) cw[j] = shift_of(wexp[min(8 * j + g, p - 1)]);
+    double2 w[NT][2];
+    auto loadw = [&](int64_t u) {                          // item k: block kb = warp, N tile k
+        const int64_t r = (u * kProjKb + warp) * 16 + 4 * t;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            w[j][0] = w[j][1] = make_double2(0.0, 0.0);
+            const double* src = W + (int64_t)min(8 * j + g, p - 1) * ldw + r;
+            if (r < n) {                                   // columns are padded to 32 rows
+                w[j][0] = *reinterpret_cast<const double2*>(src);
+                w[j][1] = *reinterpret_cast<const double2*>(src + 2);
+                if (r + 1 >= n) w[j][0].y = 0.0;           // the padding is not W's
+                if (r + 2 >= n) w[j][1].x = 0.0;
+                if (r + 3 >= n) w[j][1].y = 0.0;
+            }
+        }
+    };
+    auto storew = [&](int buf) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            uint32_t yl[4], yh[4];
+            digits_y<8>(w[j][0].x, cw[j], yl[0], yh[0]);
+            digits_y<8>(w[j][0].y, cw[j], yl[1], yh[1]);
+            digits_y<8>(w[j][1].x, cw[j], yl[2], yh[2]);
+            digits_y<8>(w[j][1].y, cw[j], yl[3], yh[3]);
+            uint2* dst = wf + buf * WBUF + (warp * NT + j) * 8 * 32 + lane;
+            auto put = [&](auto ic) {
+                constexpr int I = decltype(ic)::value;
+                dst[I * 32] = make_uint2(digit_pair<8, I>(yl[0], yh[0], yl[1], yh[1]), digit_pair<8, I>(yl[2], yh[2], yl[3], yh[3]));
+            };
+            put(std::integral_constant<int, 0>{});
+            put(std::integral_constant<int, 1>{});
+            put(std::integral_constant<int, 2>{});
+            put(std::integral_constant<int, 3>{});
+            put(std::integral_constant<int, 4>{});
+            put(std::integral_constant<int, 5>{});
+            put(std::integral_constant<int, 6>{});
+            put(std::integral_constant<int, 7>{});
+        }
+    };
+    double2 v[2][2];                                       // columns a0, a1: rows 4t, 4t + 1 | 4t + 2, 4t + 3
+    auto loadv = [&](int64_t blk) {
+        const int64_t r = blk * 16 + 4 * t;                // rows past n: padding, met by W's zeros
+        v[0][0] = *reinterpret_cast<const double2*>(V + (int64_t)a0 * ldv + r);
+        v[0][1] = *reinterpret_cast<const double2*>(V + (int64_t)a0 * ldv + r + 2);
+        v[1][0] = *reinterpret_cast<const double2*>(V + (int64_t)a1 * ldv + r);
+        v[1][1] = *reinterpret_cast<const double2*>(V + (int64_t)a1 * ldv + r + 2);
+    };
+    float acc[8][NT][4];
+    double sum[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            sum[j][q] = 0.0;
+#pragma unroll
+            for (int l = 0; l < 8; ++l) acc[l][j][q] = 0.f;
+        }
+    int64_t u = blockIdx.x;
+    int buf = 0, since = 0;
+    if (u < units) {
+        loadw(u);
+        if (work && u * kProjKb + rg < nblk) loadv(u * kProjKb + rg);
+        storew(0);
+    }
+    __syncthreads();
+    for (; u < units; u += gridDim.x) {
+        const int64_t un = u + gridDim.x;
+        if (un < units) loadw(un);
+        const int64_t bend = min(nblk, (u + 1) * kProjKb);
+        if (work)
+            for (int64_t b = u * kProjKb + rg; b < bend; b += RG) {
+                int64_t bn = b + RG;
+                if (bn >= bend) bn = un * kProjKb + rg;
+                uint32_t yl[2][4], yh[2][4];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int c = i ? cv1 : cv0;
+                    digits_y<8>(v[i][0].x, c, yl[i][0], yh[i][0]);
+                    digits_y<8>(v[i][0].y, c, yl[i][1], yh[i][1]);
+                    digits_y<8>(v[i][1].x, c, yl[i][2], yh[i][2]);
+                    digits_y<8>(v[i][1].y, c, yl[i][3], yh[i][3]);
+                }
+                if (bn < nblk) loadv(bn);
+                const uint2* wq = wf + buf * WBUF + (int)(b - u * kProjKb) * NT * 8 * 32 + lane;
+                uint2 wb[NT][8];
+#pragma unroll
+                for (int j = 0; j < NT; ++j)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) wb[j][k] = wq[(j * 8 + k) * 32];
+                auto level = [&](auto ic) {
+                    constexpr int I = decltype(ic)::value;
+                    uint32_t a[4];
+                    a[0] = digit_pair<8, I>(yl[0][0], yh[0][0], yl[0][1], yh[0][1]);
+                    a[1] = digit_pair<8, I>(yl[1][0], yh[1][0], yl[1][1], yh[1][1]);
+                    a[2] = digit_pair<8, I>(yl[0][2], yh[0][2], yl[0][3], yh[0][3]);
+                    a[3] = digit_pair<8, I>(yl[1][2], yh[1][2], yl[1][3], yh[1][3]);
+#pragma unroll
+                    for (int k = 0; k + I < 8; ++k)
+#pragma unroll
+                        for (int j = 0; j < NT; ++j) mma_f16(acc[I + k][j], a, wb[j][k].x, wb[j][k].y);
+                };
+                level(std::integral_constant<int, 0>{});
+                level(std::integral_constant<int, 1>{});
+                level(std::integral_constant<int, 2>{});
+                level(std::integral_constant<int, 3>{});
+                level(std::integral_constant<int, 4>{});
+                level(std::integral_constant<int, 5>{});
+                level(std::integral_constant<int, 6>{});
+                level(std::integral_constant<int, 7>{});
+                if (++since == 8) {                        // 8 pairs 2^14 128 rows = 2^24: still exact
+                    since = 0;
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            double x, y;
+                            level_sum64(acc[0][j][q], acc[1][j][q], acc[2][j][q], acc[3][j][q], acc[4][j][q], acc[5][j][q],
+                                        acc[6][j][q], acc[7][j][q], x, y);
+                            sum[j][q] += x + y;
+#pragma unroll
+                            for (int l = 0; l < 8; ++l) acc[l][j][q] = 0.f;
+                        }
+                }
+            }
+        buf ^= 1;
+        if (un < units) storew(buf);
+        __syncthreads();
+    }
+    double* out = part + (int64_t)blockIdx.x * cols * p;
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double x, y;
+            level_sum64(acc[0][j][q], acc[1][j][q], acc[2][j][q], acc[3][j][q], acc[4][j][q], acc[5][j][q], acc[6][j][q],
+                        acc[7][j][q], x, y);
+            red[warp][lane][q] = sum[j][q] + (x + y);
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < CG * 128; e += 256) {
+            const int q = e & 3, ln = (e >> 2) & 31, k = e >> 7;
+            const int aa = (blockIdx.y * CG + k) * 16 + (ln >> 2) + (q >> 1) * 8, c = 8 * j + 2 * (ln & 3) + (q & 1);
+            if (aa < cols && c < p) {
+                double s = red[k][ln][q];
+                for (int x = 1; x < RG; ++x) s += red[k + x * CG][ln][q];
+                out[(int64_t)aa * p + c] = scale2_e(s, vexp[aa] + wexp[c] - 2044 - 12);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// wexp[c] = largest biased exponent of column c of W (zeroed by the caller); the first CTA clears two
+// small arrays for the kernels that follow
+__global__ void k_colmax(const double* __restrict__ W, int64_t ldw, int64_t n, int* __restrict__ wexp, int* zero0, int n0,
+                         int* zero1, int n1) {
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        for (int i = threadIdx.x; i < n0; i += blockDim.x) zero0[i] = 0;
+        for (int i = threadIdx.x; i < n1; i += blockDim.x) zero1[i] = 0;
+    }
+    unsigned mx = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        mx = max(mx, (unsigned)__double2hiint(W[blockIdx.y * ldw + i]) & 0x7FFFFFFFu);
+    mx = __reduce_max_sync(kFull, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&wexp[blockIdx.y], (int)(mx >> 20));
+}
+
 // ---------------------------------------------------------------- the FP32 copy and colexp
 // V32 and colexp of columns c0 .. c0 + p - 1 of V (blocks that no fused pass wrote: the first
 // block, Ritz vectors).  skip: the fused pass wrote them (device flag).
@@ -572,7 +870,7 @@ __global__ void k_pack_block(const double* __restrict__ V, float* __restrict__ V
     unsigned mx = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double v = V[c * ld + i];
-        V32[c * ld + i] = f32_rn_i(v);
+        if (V32) V32[c * ld + i] = f32_rn_i(v);
         mx = max(mx, (unsigned)__double2hiint(v) & 0x7FFFFFFFu);
     }
     mx = __reduce_max_sync(kFull, mx);
@@ -606,42 +904,96 @@ cudaError_t launch_proj_mma(const float* V32, int64_t ldv, int cols, const doubl
     return cudaGetLastError();
 }
 
-template <int NT, int NH, bool GS>
-static cudaError_t upd_launch(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n,
-                              const double* h, int* colexp, double* partG, double* H, int ldH, int hcol, int* flags,
-                              float* V32, int restart, int max_blocks, int sms, int* nb, cudaStream_t s) {
-    const size_t shm = upd_smem(cols, NT, NH, GS);
+template <int NT, int NV, int NH, int MODE>
+static cudaError_t upd_launch(const UpdArgs& a, int max_blocks, int sms, int* nb, cudaStream_t s) {
+    const size_t shm = upd_smem(a.cols, NT, NH, MODE == U_GS);
     int per_sm = NT == 4 ? 2 : NT == 2 ? 3 : 4;
     while (per_sm > 1 && shm * per_sm > 200 * 1024) --per_sm;
-    const int64_t tiles = (n + 15) / 16;
+    const int64_t tiles = (a.n + 15) / 16;
     const int g = (int)std::min<int64_t>({(int64_t)per_sm * sms, (tiles + 3) / 4, (int64_t)max_blocks});
     if (nb) *nb = g;
-    k_upd_mma<NT, NH, GS><<<g, kUpdThreads, shm, s>>>(V, ldv, cols, W, ldw, p, n, h, colexp, partG, H, ldH, hcol, flags,
-                                                      V32, restart);
+    k_upd_mma<NT, NV, NH, MODE><<<g, kUpdThreads, shm, s>>>(a);
     return cudaGetLastError();
 }
+
+#define EXPM_UPD(NV, NH, MODE, ...)                                                                            \
+    (a.p <= 8 ? upd_launch<1, NV, NH, MODE>(a, __VA_ARGS__) : a.p <= 16 ? upd_launch<2, NV, NH, MODE>(a, __VA_ARGS__) \
+                                                             : upd_launch<4, NV, NH, MODE>(a, __VA_ARGS__))
 
 cudaError_t launch_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,
                            int* colexp, double* partG, double* H, int ldH, int hcol, int* flags, int max_blocks, int sms,
                            int* nb, cudaStream_t s) {
-#define EXPM_UPD(NT) upd_launch<NT, 4, true>(V, ldv, cols, W, ldw, p, n, h, colexp, partG, H, ldH, hcol, flags, nullptr, 0, max_blocks, sms, nb, s)
-    return p <= 8 ? EXPM_UPD(1) : p <= 16 ? EXPM_UPD(2) : EXPM_UPD(4);
-#undef EXPM_UPD
+    UpdArgs a{V, ldv, cols, W, ldw, p, n, h, colexp, partG, H, ldH, hcol, flags};
+    return EXPM_UPD(7, 4, U_GS, max_blocks, sms, nb, s);
 }
 
 cudaError_t launch_updz_mma(double* V, float* V32, int64_t ldv, int cols, double* Z, int64_t ldz, int p, int64_t n,
                             const double* Wc, int* colexp, int* flags, int restart, int sms, cudaStream_t s) {
-#define EXPM_UPZ(NT) upd_launch<NT, 6, false>(V, ldv, cols, Z, ldz, p, n, Wc, colexp, nullptr, nullptr, 0, 0, flags, V32, restart, 1 << 20, sms, nullptr, s)
-    cudaError_t e = p <= 8 ? EXPM_UPZ(1) : p <= 16 ? EXPM_UPZ(2) : EXPM_UPZ(4);
-#undef EXPM_UPZ
+    UpdArgs a{V, ldv, cols, Z, ldz, p, n, Wc, colexp, nullptr, nullptr, 0, 0, flags, V32, restart};
+    cudaError_t e = V32 ? EXPM_UPD(7, 6, U_Z, 1 << 20, sms, nullptr, s) : EXPM_UPD(8, 8, U_Z64, 1 << 20, sms, nullptr, s);
     if (e == cudaSuccess && restart)
         e = cudaMemcpyAsync(colexp, colexp + cols - p, sizeof(int) * p, cudaMemcpyDeviceToDevice, s);
     return e;
 }
 
+// FP64 plans: W <- W - V h, the exponents of the result's columns into oexp (zeroed by the caller)
+cudaError_t launch_upd64(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,
+                         int* colexp, int* oexp, int* flags, int sms, cudaStream_t s) {
+    UpdArgs a{V, ldv, cols, W, ldw, p, n, h, colexp, nullptr, nullptr, 0, 0, flags};
+    a.oexp = oexp;
+    return EXPM_UPD(8, 8, U_GS64, 1 << 20, sms, nullptr, s);
+}
+
+// out <- W Rinv (p x p), exponents into oexp; alt != null: into alt / altexp instead when flags[2] is set
+// (a third pass follows); third: only when flags[2] is set
+cudaError_t launch_mul64(double* W, int64_t ldw, int p, int64_t n, const double* Rinv, int* wexp, double* out, int64_t ldo,
+                         int* oexp, double* alt, int64_t ldalt, int* altexp, int third, int* flags, int sms, cudaStream_t s) {
+    UpdArgs a{W, ldw, p, out, ldo, p, n, Rinv, wexp, nullptr, nullptr, 0, 0, flags};
+    a.oexp = oexp;
+    a.alt = alt;
+    a.ldalt = ldalt;
+    a.altexp = altexp;
+    if (third) {
+        a.skip = flags + 2;
+        a.skip_zero = 1;
+    }
+    return EXPM_UPD(8, 8, U_MUL64, 1 << 20, sms, nullptr, s);
+}
+
+// V^T W to FP64 rounding: partial[bx][a][c], nb of them; only: run only when *only != 0
+cudaError_t launch_proj64(const double* V, int64_t ldv, int cols, const int* vexp, const double* W, int64_t ldw, int p,
+                          const int* wexp, int64_t n, double* part, int max_blocks, int sms, int* nb, const int* only,
+                          cudaStream_t s) {
+    const int mt = (cols + 15) / 16, NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
+    const int CG = std::min(8, mt), gy = (mt + CG - 1) / CG, RG = 8 / CG;
+    const int64_t units = (n + 16 * kProjKb - 1) / (16 * kProjKb);
+    const int64_t gmax = std::max(1, std::min(max_blocks, (NT == 1 ? 2 : 1) * sms / gy));
+    const int64_t per = (units + gmax - 1) / gmax;
+    const int gx = (int)((units + per - 1) / per);
+    *nb = gx;
+    const dim3 grid(gx, gy);
+    (void)RG;
+    if (NT == 1) k_proj64<1><<<grid, 256, proj64_smem(1), s>>>(V, ldv, cols, vexp, W, ldw, p, wexp, n, part, CG, only);
+    else if (NT == 2) k_proj64<2><<<grid, 256, proj64_smem(2), s>>>(V, ldv, cols, vexp, W, ldw, p, wexp, n, part, CG, only);
+    else k_proj64<4><<<grid, 256, proj64_smem(4), s>>>(V, ldv, cols, vexp, W, ldw, p, wexp, n, part, CG, only);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_colmax(const double* W, int64_t ldw, int p, int64_t n, int* wexp, int* zero0, int n0, int* zero1, int n1,
+                          cudaStream_t s) {
+    const int gx = (int)std::min<int64_t>((n + 1023) / 1024, 256);
+    k_colmax<<<dim3(gx, p), 256, 0, s>>>(W, ldw, n, wexp, zero0, n0, zero1, n1);
+    return cudaGetLastError();
+}
+
 bool mma_fit(int mp, int p) {
     const int NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
     return p >= 1 && p <= kMaxP && upd_smem(mp, NT, 4, true) <= 220 * 1024 && upd_smem(mp + p, NT, 6, false) <= 220 * 1024;
+}
+
+bool mma64_fit(int mp, int p) {
+    const int NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
+    return p >= 1 && p <= kMaxP && upd_smem(mp + p, NT, 8, false) <= 220 * 1024;
 }
 
 cudaError_t launch_pack_block(const double* V, float* V32, int64_t ld, int64_t n, int p, int* colexp, const int* skip,
@@ -657,8 +1009,17 @@ cudaError_t mma_set_smem_limits() {
 #define EXPM_SET(K) \
     if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024)
     EXPM_SET((k_proj_mma<4, 2>));
-    EXPM_SET((k_upd_mma<1, 4, true>)); EXPM_SET((k_upd_mma<2, 4, true>)); EXPM_SET((k_upd_mma<4, 4, true>));
-    EXPM_SET((k_upd_mma<1, 6, false>)); EXPM_SET((k_upd_mma<2, 6, false>)); EXPM_SET((k_upd_mma<4, 6, false>));
+    EXPM_SET((k_upd_mma<1, 7, 4, U_GS>)); EXPM_SET((k_upd_mma<2, 7, 4, U_GS>)); EXPM_SET((k_upd_mma<4, 7, 4, U_GS>));
+    EXPM_SET((k_upd_mma<1, 7, 6, U_Z>)); EXPM_SET((k_upd_mma<2, 7, 6, U_Z>)); EXPM_SET((k_upd_mma<4, 7, 6, U_Z>));
+    EXPM_SET((k_upd_mma<1, 8, 8, U_GS64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_GS64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_GS64>));
+    EXPM_SET((k_upd_mma<1, 8, 8, U_Z64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_Z64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_Z64>));
+    EXPM_SET((k_upd_mma<1, 8, 8, U_MUL64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_MUL64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_MUL64>));
+#undef EXPM_SET
+#define EXPM_SET(NT) \
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_proj64<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)proj64_smem(NT))
+    EXPM_SET(1);
+    EXPM_SET(2);
+    EXPM_SET(4);
 #undef EXPM_SET
     return e;
 }

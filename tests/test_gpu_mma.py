@@ -70,3 +70,30 @@ def test_converged_solve_matches_closed_form(sides, p, t, repeated):
     assert info.converged == 1
     ref = ops.exact_r_of_A_B(sides, diff, vel, t, cf.load_table(), B)
     assert rel(to_np(Z), ref) <= 1e-9, rel(to_np(Z), ref)
+
+
+@pytest.mark.parametrize("local", [False, True])
+@pytest.mark.parametrize("sides,p,m", [((401, 251), 1, 12), ((317, 106), 3, 6), ((130, 113), 8, 17), ((97, 83), 13, 10),
+                                       ((83, 79), 16, 9), ((61, 59), 29, 6), ((33, 31, 29), 4, 5)])
+def test_fp64_digit_passes_reach_fp64_rounding(sides, p, m, local):
+    """FP64 plans with at least 100000 block entries: projections, updates and the Cholesky-QR products
+    by digits.  Every product carries both operands to 2^-62 of their column's largest entry and is
+    rounded once, so the relation holds to ~ (m p) eps of |W| and the basis is orthonormal to ~ (m p) p
+    eps, the bounds of the FP64 kernels (1e-13 with the constants of these sizes).  The widths cover
+    each N-tile size and bases that end inside a chunk or pass the 128-column segment."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    n, t = int(np.prod(sides)), 0.05
+    assert n * p >= 100000
+    if local:
+        V1 = np.zeros((n, p), order="F")
+        V1[np.linspace(0, n - 1, p).astype(int), np.arange(p)] = 1.0
+    else:
+        V1, _ = ps.qr_positive(inputs.rhs(n, p, 8))
+    plan = Plan(sides, 0.1, (1.0, -0.5, 0.3)[:len(sides)], p_max=p, m=m)
+    Vg, Hg = plan.arnoldi(t, to_dev(V1))
+    W = np.column_stack([to_np(plan.prec_apply(t, Vg[:, j * p:(j + 1) * p])) for j in range(m)])
+    V, H = to_np(Vg), to_np(Hg)
+    plan.close()
+    assert np.linalg.norm(W - V @ H) <= 1e-13 * np.linalg.norm(W)
+    assert np.linalg.norm(V.T @ V - np.eye((m + 1) * p)) <= 1e-13
