@@ -273,6 +273,20 @@ __device__ __forceinline__ double scale2_e(double x, int k) {
     return __longlong_as_double(r);
 }
 
+// x 2^k as a double from the bit pattern; x finite, subnormal x and results below 2^-1022 give zero, results
+// past the range inf
+__device__ __forceinline__ double scaled_f32(float x, int k) {
+    const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+    const int e = (int)(m >> 23) + 896 + k;
+    uint32_t hi = (m >> 3) + ((uint32_t)(896 + k) << 20), lo = m << 29;
+    if (m < 0x00800000u || e <= 0) hi = lo = 0u;
+    if (e >= 2047 && m >= 0x00800000u) {
+        hi = 0x7FF00000u;
+        lo = 0u;
+    }
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
+}
+
 // X 2^k as a double, |X| <= 2^52, built from its bit pattern (results below 2^-1022 flush to zero)
 __device__ __forceinline__ double scaled_int(long long X, int k) {
     if (X == 0) return 0.0;
@@ -547,15 +561,15 @@ k_upd_mma(const UpdArgs A) {
                     const int k = fmax_s[8 * j + 2 * t + (q & 1)] - (D64 ? 12 : 14);
                     constexpr bool SUB = MODE == U_GS || MODE == U_GS64;
                     if constexpr (!D64) {
-                        // Horner in a float pair
-                        float sh = acc[6][j][q], sl = 0.f;
-#pragma unroll
-                        for (int l = 5; l >= 0; --l) {
-                            sh *= 0x1p-8f;
-                            sl *= 0x1p-8f;
-                            df_add(sh, sl, acc[l][j][q]);
-                        }
-                        const double x = scale2_e(f64_of_f32_i(sh), k), y = scale2_e(f64_of_f32_i(sl), k);
+                        // levels 0..2 exactly in a float pair (40 bits), the others, 2^-24 below, in FP32
+                        float sh = acc[2][j][q] * 0x1p-16f, sl = 0.f;
+                        df_add(sh, sl, acc[1][j][q] * 0x1p-8f);
+                        df_add(sh, sl, acc[0][j][q]);
+                        float lo = fmaf(acc[6][j][q], 0x1p-48f, acc[5][j][q] * 0x1p-40f);
+                        lo = fmaf(acc[4][j][q], 0x1p-32f, lo);
+                        lo = fmaf(acc[3][j][q], 0x1p-24f, lo);
+                        sl += lo;
+                        const double x = scaled_f32(sh, k), y = scaled_f32(sl, k);
                         w[j][q] = SUB ? (w[j][q] - x) - y : (w[j][q] + x) + y;
                     } else {
                         double x, y;
