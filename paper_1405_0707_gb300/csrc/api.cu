@@ -885,31 +885,7 @@ expm_status run_block(expm_plan* P, double t, const double* dB, int64_t ldb, int
 
 void free_plan(expm_plan* P) {
     if (!P) return;
-    for (int d = 0; d < 3; ++d) {
-        cudaFree(P->Qf[d]);
-        cudaFree(P->Qi[d]);
-        cudaFree(P->lam[d]);
-    }
-    cudaFree(P->th_m);
-    cudaFree(P->th_c);
-    for (int d = 0; d < 3; ++d) {
-        cudaFree(P->QfF[d]);
-        cudaFree(P->QiF[d]);
-    }
-    cudaFree(P->th_m32);
-    cudaFree(P->th_c32);
-    cudaFree(P->T1f);
-    cudaFree(P->T2f);
-    cudaFree(P->R64);
-    cudaFree(P->V);
-    cudaFree(P->W);
-    cudaFree(P->T1);
-    cudaFree(P->T2);
-    cudaFree(P->Zacc);
-    cudaFree(P->Bst);
-    cudaFree(P->Zst);
-    cudaFree(P->Xcert);
-    cudaFree(P->Acert);
+    cudaFree(P->slab);
     cudaFree(P->cs.rowptr);
     cudaFree(P->cs.colind);
     cudaFree(P->cs.val);
@@ -933,26 +909,8 @@ void free_plan(expm_plan* P) {
     cudaFree(P->tz.Ub);
     cudaFree(P->tz.mu1);
     cudaFree(P->tz.mu2);
-    cudaFree(P->Zcert);
-    cudaFree(P->Ccert);
-    cudaFree(P->rcert);
     delete[] P->hcert;
-    cudaFree(P->H);
-    cudaFree(P->part);
     cudaFree(P->V32);
-    cudaFree(P->colexp);
-    cudaFree(P->wexp);
-    cudaFree(P->partG);
-    cudaFree(P->fac);
-    cudaFree(P->small);
-    cudaFree(P->poles);
-    cudaFree(P->S);
-    cudaFree(P->Wc_slots);
-    cudaFree(P->stat);
-    cudaFree(P->ctr);
-    cudaFree(P->dotpart);
-    cudaFree(P->Vk);
-    cudaFree(P->Pkd);
     if (P->hH) cudaFreeHost(P->hH);
     if (P->hPk) cudaFreeHost(P->hPk);
     if (P->hHnew) cudaFreeHost(P->hHnew);
@@ -1532,39 +1490,45 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
     P->ldH = (m + 1) * p_max;
     const int mpm = m * p_max;
     bool ok = true;
-    ok = ok && dalloc(&P->V, (size_t)ld * (m + 1) * p_max);
-    ok = ok && dalloc(&P->W, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->T1, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->T2, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->Zacc, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->Bst, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->Zst, (size_t)ld * p_max);
-    ok = ok && dalloc(&P->H, (size_t)P->ldH * mpm);
-    ok = ok && dalloc(&P->part, (size_t)std::max(P->nblk, P->nblk_cgs) * (mpm + p_max) * p_max);
-    ok = ok && dalloc(&P->small, kSmallDoubles);
-    ok = ok && dalloc(&P->S, (size_t)P->npoles * p_max * p_max * 2);
-    ok = ok && dalloc(&P->Wc_slots, (size_t)P->npoles * (mpm + p_max) * p_max);
-    ok = ok && dalloc(&P->stat, kStatDoubles);
-    ok = ok && dalloc(&P->ctr, 4) && cudaMemset(P->ctr, 0, sizeof(unsigned) * 4) == cudaSuccess;
+    // one allocation for the plan's buffers (their pointers are set once all are listed)
+    std::vector<std::pair<void**, size_t>> reqs;
+    auto want = [&](auto** ptr, size_t count) {
+        reqs.emplace_back(reinterpret_cast<void**>(ptr), (std::max<size_t>(count, 1) * sizeof(**ptr) + 255) / 256 * 256);
+        return true;
+    };
+    ok = ok && want(&P->V, (size_t)ld * (m + 1) * p_max);
+    ok = ok && want(&P->W, (size_t)ld * p_max);
+    ok = ok && want(&P->T1, (size_t)ld * p_max);
+    ok = ok && want(&P->T2, (size_t)ld * p_max);
+    ok = ok && want(&P->Zacc, (size_t)ld * p_max);
+    ok = ok && want(&P->Bst, (size_t)ld * p_max);
+    ok = ok && want(&P->Zst, (size_t)ld * p_max);
+    ok = ok && want(&P->H, (size_t)P->ldH * mpm);
+    ok = ok && want(&P->part, (size_t)std::max(P->nblk, P->nblk_cgs) * (mpm + p_max) * p_max);
+    ok = ok && want(&P->small, kSmallDoubles);
+    ok = ok && want(&P->S, (size_t)P->npoles * p_max * p_max * 2);
+    ok = ok && want(&P->Wc_slots, (size_t)P->npoles * (mpm + p_max) * p_max);
+    ok = ok && want(&P->stat, kStatDoubles);
+    ok = ok && want(&P->ctr, 4);
     if (opts->certify) {
         const size_t w = 2 * (size_t)P->npoles * p_max, rows = (size_t)mpm + p_max;
         if (8 * (rows * w + 16 * (rows | 1)) > 225 * 1024) { free_plan(P); return EXPM_INVALID_ARG; }
-        ok = ok && dalloc(&P->Xcert, (size_t)ld * w) && dalloc(&P->Zcert, (size_t)P->npoles * mpm * p_max * 2) &&
-             dalloc(&P->Ccert, rows * w) && dalloc(&P->rcert, (size_t)P->npoles * true_resid_blocks(n));
-        if (toeplitz) ok = ok && dalloc(&P->Acert, (size_t)ld * w);
+        ok = ok && want(&P->Xcert, (size_t)ld * w) && want(&P->Zcert, (size_t)P->npoles * mpm * p_max * 2) &&
+             want(&P->Ccert, rows * w) && want(&P->rcert, (size_t)P->npoles * true_resid_blocks(n));
+        if (toeplitz) ok = ok && want(&P->Acert, (size_t)ld * w);
         P->hcert = new (std::nothrow) double[(size_t)P->npoles * true_resid_blocks(n)];
         ok = ok && P->hcert != nullptr;
     }
-    ok = ok && dalloc(&P->poles, (size_t)P->npoles * poles_work_doubles(mpm, p_max));
+    ok = ok && want(&P->poles, (size_t)P->npoles * poles_work_doubles(mpm, p_max));
     ok = ok && cudaMallocHost(reinterpret_cast<void**>(&P->hpin), sizeof(double) * kStatDoubles) == cudaSuccess;
-    ok = ok && dalloc(&P->dotpart, (size_t)dot_blocks() * p_max) &&
+    ok = ok && want(&P->dotpart, (size_t)dot_blocks() * p_max) &&
          cudaMallocHost(reinterpret_cast<void**>(&P->hdot), sizeof(double) * dot_blocks() * p_max) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&P->cycle_ev, cudaEventDisableTiming) == cudaSuccess;
     if (opts->k_defl > 0) {
         // the kept count never exceeds k_defl rounded up to a multiple of p, nor (m - 1) p
         P->kdefl_max = std::min(opts->k_defl + p_max - 1, (m - 1) * p_max);
         const size_t kd = (size_t)P->kdefl_max;
-        ok = ok && dalloc(&P->Vk, (size_t)ld * kd) && dalloc(&P->Pkd, (size_t)mpm * kd);
+        ok = ok && want(&P->Vk, (size_t)ld * kd) && want(&P->Pkd, (size_t)mpm * kd);
         ok = ok && cudaMallocHost(reinterpret_cast<void**>(&P->hH), sizeof(double) * (size_t)P->ldH * mpm) == cudaSuccess;
         ok = ok && cudaMallocHost(reinterpret_cast<void**>(&P->hPk), sizeof(double) * (size_t)mpm * kd) == cudaSuccess;
         ok = ok && cudaMallocHost(reinterpret_cast<void**>(&P->hHnew), sizeof(double) * (size_t)P->ldH * kd) == cudaSuccess;
@@ -1587,32 +1551,39 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         int64_t nmodes = 1;
         for (int d = 1; d < P->ndim; ++d) {
             const int N = P->ax[d].N;
-            ok = ok && dalloc(&P->Qf[d], (size_t)N * N) && dalloc(&P->Qi[d], (size_t)N * N) &&
-                 dalloc(&P->lam[d], (size_t)N);
+            ok = ok && want(&P->Qf[d], (size_t)N * N) && want(&P->Qi[d], (size_t)N * N) &&
+                 want(&P->lam[d], (size_t)N);
             nmodes *= N;
         }
         P->nmodes = nmodes;
-        ok = ok && dalloc(&P->th_m, (size_t)P->ax[0].N * nmodes) && dalloc(&P->th_c, (size_t)P->ax[0].N * nmodes);
+        ok = ok && want(&P->th_m, (size_t)P->ax[0].N * nmodes) && want(&P->th_c, (size_t)P->ax[0].N * nmodes);
         if (mixed) {
             for (int d = 1; d < P->ndim; ++d) {
                 const int N = P->ax[d].N;
-                ok = ok && dalloc(&P->QfF[d], table_frag_count(N)) && dalloc(&P->QiF[d], table_frag_count(N));
+                ok = ok && want(&P->QfF[d], table_frag_count(N)) && want(&P->QiF[d], table_frag_count(N));
             }
-            ok = ok && dalloc(&P->th_m32, (size_t)P->ax[0].N * nmodes) &&
-                 dalloc(&P->th_c32, (size_t)P->ax[0].N * nmodes);
-            ok = ok && dalloc(&P->T1f, (size_t)ld * p_max) && dalloc(&P->T2f, (size_t)ld * p_max);
-            ok = ok && dalloc(&P->R64, (size_t)ld * p_max);
+            ok = ok && want(&P->th_m32, (size_t)P->ax[0].N * nmodes) &&
+                 want(&P->th_c32, (size_t)P->ax[0].N * nmodes);
+            ok = ok && want(&P->T1f, (size_t)ld * p_max) && want(&P->T2f, (size_t)ld * p_max);
+            ok = ok && want(&P->R64, (size_t)ld * p_max);
         }
     }
     if (P->mma64)
-        ok = ok && dalloc(&P->colexp, (size_t)(m + 2) * p_max) && dalloc(&P->wexp, 10 * (size_t)p_max);
-    if (P->mma) {
-        const size_t v32 = (size_t)ld * (m + 1) * p_max;
-        ok = ok && dalloc(&P->V32, v32) && dalloc(&P->colexp, (size_t)(m + 2) * p_max) &&
-             dalloc(&P->partG, (size_t)P->nblkG * p_max * p_max) && dalloc(&P->fac, 2 * kMaxP * kMaxP + 2 * kMaxP) &&
-             cudaMemsetAsync(P->V32, 0, sizeof(float) * v32, P->stream) == cudaSuccess &&
-             cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, P->stream) == cudaSuccess;
+        ok = ok && want(&P->colexp, (size_t)(m + 2) * p_max) && want(&P->wexp, 10 * (size_t)p_max);
+    if (P->mma)
+        ok = ok && want(&P->colexp, (size_t)(m + 2) * p_max) && want(&P->partG, (size_t)P->nblkG * p_max * p_max) &&
+             want(&P->fac, 2 * kMaxP * kMaxP + 2 * kMaxP);
+    if (ok) {
+        size_t total = 0;
+        for (const auto& r : reqs) total += r.second;
+        ok = dalloc(&P->slab, total);
+        unsigned char* at = P->slab;
+        for (const auto& r : reqs) {
+            *r.first = ok ? at : nullptr;
+            at += r.second;
+        }
     }
+    ok = ok && cudaMemsetAsync(P->ctr, 0, sizeof(unsigned) * 4, P->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_plan(P);
@@ -1670,6 +1641,21 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
             cudaGetLastError();
             free_plan(P);
             return ts;
+        }
+    }
+    if (P->mma) {
+        // last, the FP32 copy of the basis (half the basis again): a plan that has no room for it runs on
+        // the kernels that read the FP64 basis alone
+        const size_t v32 = (size_t)ld * (m + 1) * p_max;
+        if (!dalloc(&P->V32, v32)) {
+            cudaGetLastError();
+            P->V32 = nullptr;
+            P->mma = false;
+        } else if (cudaMemsetAsync(P->V32, 0, sizeof(float) * v32, s) != cudaSuccess ||
+                   cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, s) != cudaSuccess) {
+            cudaGetLastError();
+            free_plan(P);
+            return EXPM_CUDA_ERROR;
         }
     }
     *out = P;

@@ -187,6 +187,8 @@ struct expm_plan_s {
     float* T2f = nullptr;      // ld x p_max
     double* R64 = nullptr;     // ld x p_max   residual of the refined inverse
     int refine = 2;            // FP64 refinement steps of the FP32 inverse
+    unsigned char* slab = nullptr;   // the one allocation behind the buffers of this struct (V32 and the
+                                     // Toeplitz and sparse operators own theirs)
     // workspace (device)
     double* V = nullptr;       // ld x (m+1) p_max       Krylov basis
     double* W = nullptr;       // ld x p_max
