@@ -135,10 +135,11 @@ expm_status qr_block(expm_plan* P, int p, double* out, int64_t ldo, bool withH, 
     return EXPM_OK;
 }
 
-// One FP32 application of (tA)^{-1} to R (FP32), written (acc = 0) or added (acc = 1) to X (FP64).
+// One FP32 application of (tA)^{-1} to R (FP32), written (acc = 0) or added (acc = 1) to X (FP64).  On 3-D grids
+// also to D (FP32, leading dimension P->ld) in place of X, or X <- X + (product + add) with add laid out as D.
 // Same transforms and layouts as the FP64 path.
 expm_status inv32_apply(expm_plan* P, double t, const float* R, int64_t ldr, int p, double* X,
-                        int64_t ldx, int acc) {
+                        int64_t ldx, int acc, float* D = nullptr, const float* add = nullptr) {
     cudaStream_t s = P->stream;
     const int nx = P->ax[0].N, ny = P->ax[1].N, nz = P->ax[2].N;
     const int64_t ld = P->ld;
@@ -160,35 +161,47 @@ expm_status inv32_apply(expm_plan* P, double t, const float* R, int64_t ldr, int
     LAUNCH(EXPM_STAGE_TRIDIAG, launch_tridiag_lines32(P->T1f, ld, p, nx, nyz, lsub, P->th_m32, P->th_c32, inv_t, s));
     const TransformArgs g3{P->T1f, P->QiF[1], P->T2f, nx * nz, ny, ny, nyz, 1, ld, 1, nx, ld, 0, 0, nx, ny, nxy};
     LAUNCH(EXPM_STAGE_GEMM, launch_transform(g3, p, P->sms, s));
-    const TransformArgs g4{P->T2f, P->QiF[2], X, (int)nxy, nz, nz, 1, nxy, ld, 1, nxy, ldx, 1, acc};
-    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g4, p, P->sms, s));
+    const TransformArgs g4{P->T2f, P->QiF[2], D ? (void*)D : (void*)X, (int)nxy, nz, nz, 1, nxy, ld, 1, nxy, D ? ld : ldx,
+                           D ? 0 : 1, acc};
+    LAUNCH(EXPM_STAGE_GEMM, launch_transform(g4, p, P->sms, s, add, ld));
     return EXPM_OK;
 }
 
-// Mixed precision: W = (tA)^{-1} V to FP64 accuracy by iterative refinement of the FP32
-// inverse: x_0 = inv32(V), x_{k+1} = x_k + inv32(V - tA x_k) with the residual in FP64
+// Mixed precision: W = (tA)^{-1} V to FP64 accuracy by two steps of iterative refinement of the
+// FP32 inverse: x_0 = inv32(V), x_{k+1} = x_k + d_k, d_k = inv32(r_k), r_k = V - tA x_k
 // (Theorem 4.3: the inverse's accuracy is what the shifted solutions inherit).  Each step
 // multiplies the backward error by about eps_32 * rho^-N (diagonal similarity).
+// r_0 is formed in FP64.  On 3-D grids r_1 = r_0 - tA d_0 in float pairs, and W is read and written
+// once for both corrections, W = x_0 + (d_0 + d_1): 96^3, p = 16, 167.1 -> 161.9 ms per solve.  On 2-D
+// grids r_1 is formed from x_1 in FP64 like r_0: the five-point stencil is 3 us shorter in float pairs there
+// and the last transform 5 us longer with the extra addend (256 x 256, p = 8: 15.5 ms against 15.8 ms).
 // V32, when given, is V's FP32 copy (leading dimension P->ld), which the first transform reads.
 expm_status prec_apply_mixed(expm_plan* P, double t, const double* V, int64_t ldv, int p,
                              double* W, int64_t ldw, const float* V32) {
     cudaStream_t s = P->stream;
-    float* R32 = reinterpret_cast<float*>(P->R64);
+    const int64_t ld = P->ld;
+    const int nx = P->ax[0].N, ny = P->ax[1].N, nz = P->ax[2].N, nd = P->ndim;
+    // T1 and T2 are the FP64 inverse's transform buffers, which a mixed plan's inverse does not use
+    float* R32 = reinterpret_cast<float*>(P->T1);
+    float* D = reinterpret_cast<float*>(P->T2);
+    double* R1 = nd == 3 ? P->R64 : nullptr;
     if (!V32) {
-        LAUNCH(EXPM_STAGE_GEMM, launch_d2f(V, R32, P->n, s, ldv, P->ld, p));
+        LAUNCH(EXPM_STAGE_GEMM, launch_d2f(V, R32, P->n, s, ldv, ld, p));
         V32 = R32;
     }
-    expm_status st = inv32_apply(P, t, V32, P->ld, p, W, ldw, 0);
+    expm_status st = inv32_apply(P, t, V32, ld, p, W, ldw, 0);
     if (st != EXPM_OK) return st;
-    for (int k = 0; k < P->refine; ++k) {
-        // the residual V - tA x in FP64, stored in FP32 (the R64 buffer): the transforms read
-        // it as FP32 either way
-        LAUNCH(EXPM_STAGE_STENCIL, launch_cd_apply(W, ldw, nullptr, P->ld, p, P->ndim, P->ax[0].N, P->ax[1].N,
-                                                   P->ax[2].N, P->ax, -t, s, V, ldv, 1.0, R32, P->stencil_df & 2));
-        st = inv32_apply(P, t, R32, P->ld, p, W, ldw, 1);
-        if (st != EXPM_OK) return st;
+    LAUNCH(EXPM_STAGE_STENCIL, launch_cd_apply(W, ldw, R1, ld, p, nd, nx, ny, nz, P->ax, -t, s, V, ldv, 1.0, R32,
+                                               P->stencil_df & 2));
+    if (nd == 3) {
+        if ((st = inv32_apply(P, t, R32, ld, p, nullptr, 0, 0, D)) != EXPM_OK) return st;
+        LAUNCH(EXPM_STAGE_STENCIL, launch_cd_next_residual(R1, ld, D, ld, R32, ld, p, nx, ny, nz, P->ax, t, s));
+        return inv32_apply(P, t, R32, ld, p, W, ldw, 1, nullptr, D);
     }
-    return EXPM_OK;
+    if ((st = inv32_apply(P, t, R32, ld, p, W, ldw, 1)) != EXPM_OK) return st;
+    LAUNCH(EXPM_STAGE_STENCIL, launch_cd_apply(W, ldw, nullptr, ld, p, nd, nx, ny, nz, P->ax, -t, s, V, ldv, 1.0, R32,
+                                               P->stencil_df & 2));
+    return inv32_apply(P, t, R32, ld, p, W, ldw, 1);
 }
 
 // ---- symmetric Toeplitz operator (k_fft.cu): products and the Gohberg-Semencul inverse
@@ -1565,7 +1578,7 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
             ok = ok && want(&P->th_m32, (size_t)P->ax[0].N * nmodes) &&
                  want(&P->th_c32, (size_t)P->ax[0].N * nmodes);
             ok = ok && want(&P->T1f, (size_t)ld * p_max) && want(&P->T2f, (size_t)ld * p_max);
-            ok = ok && want(&P->R64, (size_t)ld * p_max);
+            if (P->ndim == 3) ok = ok && want(&P->R64, (size_t)ld * p_max);
         }
     }
     if (P->mma64)

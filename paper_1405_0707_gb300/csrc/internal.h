@@ -185,8 +185,7 @@ struct expm_plan_s {
     float* th_c32 = nullptr;
     float* T1f = nullptr;      // ld x p_max
     float* T2f = nullptr;      // ld x p_max
-    double* R64 = nullptr;     // ld x p_max   residual of the refined inverse
-    int refine = 2;            // FP64 refinement steps of the FP32 inverse
+    double* R64 = nullptr;     // ld x p_max   first residual of the refined inverse (3-D grids)
     unsigned char* slab = nullptr;   // the one allocation behind the buffers of this struct (V32 and the
                                      // Toeplitz and sparse operators own theirs)
     // workspace (device)
@@ -277,9 +276,14 @@ cudaError_t launch_cd_apply(const double* V, int64_t ldv, double* W, int64_t ldw
                             int ndim, int nx, int ny, int nz, const Axis* ax, double t,
                             cudaStream_t s, const double* Y = nullptr, int64_t ldy = 0,
                             double beta = 0.0, float* W32 = nullptr, int df = 0);
+cudaError_t launch_cd_next_residual(const double* R1, int64_t ldr, const float* D, int64_t ldd, float* R2, int64_t ld2,
+                                    int p, int nx, int ny, int nz, const Axis* ax, double t, cudaStream_t s);
 size_t table_frag_count(int N);
 cudaError_t launch_table_frags(const double* Q, int N, uint4* F, cudaStream_t s);
-cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s);
+// add: an FP32 array added with the product when it accumulates into an FP64 C, C <- C + (product + add), one
+// rounding at C's size; laid out as C (M x N, m contiguous) with its own column stride add_b
+cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s,
+                             const float* add = nullptr, int64_t add_b = 0);
 cudaError_t transform_set_smem();
 cudaError_t launch_tridiag_lines32(float* y, int64_t ld, int p, int L, int64_t nmodes, float l_sub,
                                    const float* th_m, const float* th_c, float inv_t,

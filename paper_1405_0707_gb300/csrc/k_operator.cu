@@ -20,7 +20,7 @@ constexpr int BK = 16;
 // layout so that the fastest-varying thread index walks C's contiguous dimension.  The FP64 pipe (2 FMAs
 // per SM and clock) is the bound, whatever the tile: a 64 x 64 tile keeps one SM busy for 100 us at
 // K = 99, so small problems take smaller tiles and spread over the SMs (launch_gemm picks the tile with
-// the least work on the fullest SM; 99 x 99, 3 columns: 127 us with 12 CTAs, 10 us with 147).
+// the least work on the fullest SM; 99 x 99, 3 columns: 127 us with 12 CTAs, 14 us with 147).
 template <bool CM, int TM>
 __global__ void __launch_bounds__(256) k_gemm(GemmArgs g) {
     constexpr int BM = 16 * TM, BN = 16 * TM;
@@ -208,7 +208,7 @@ __global__ void k_tridiag_lines(const double* in, int64_t ld_in, double* out, in
 // CTA scans the threads' maps, and each point is corrected with the value that enters its segment
 // (y = y_local + P y_in), so every point is read once per sweep and costs nine FP64 operations.  With the
 // warp-per-four-lines kernel above, 2000 points were 250 dependent FP64 steps per lane: 178 us a solve,
-// now 11 us, most of it the one SM's FP64 pipe.
+// now 13 us, most of it the one SM's FP64 pipe.
 constexpr int kLineT = 256, kLineE = 8;
 
 struct Affine {
@@ -362,9 +362,9 @@ struct StencilT {
 };
 
 // W = tA V (+ beta Y): one thread per grid point and column; grid index arithmetic in 32 bits
-// (n < 2^31 is checked by the launcher).  With W32 set, the FP64 result is stored rounded to
-// FP32 there (same leading dimension) instead of in W: the refinement residual, which only
-// the FP32 transforms read.
+// (n < 2^31 is checked by the launcher).  With W32 set, the result is stored rounded to FP32 there (same
+// leading dimension), and in W as well when that is given: the refinement residual, whose FP32 copy the
+// transforms read and whose FP64 value the next residual starts from.
 __global__ void k_cd_apply(const double* __restrict__ V, int64_t ldv, double* __restrict__ W,
                            int64_t ldw, int ndim, int nx, int ny, int nz, StencilT k,
                            const double* __restrict__ Y, int64_t ldy, double beta, float* __restrict__ W32) {
@@ -390,7 +390,46 @@ __global__ void k_cd_apply(const double* __restrict__ V, int64_t ldv, double* __
     }
     const double r = Y ? fma(beta, Y[c * ldy + i], acc) : acc;
     if (W32) W32[c * ldw + i] = f32_rn_i(r);   // integer rounding: no FP64-pipe conversion
-    else W[c * ldw + i] = r;
+    if (W) W[c * ldw + i] = r;
+}
+
+// The next residual of a 3-D grid's refined inverse from the last one: R1 - tA D for the FP32 correction D that was
+// added to x, in float pairs (coefficients as pairs, D exact floats), rounded to FP32.  D is ~1e-7 of x, so
+// the pairs' 2^-48 of |tA||D| lies far below what FP64 resolves of the residual formed from x itself
+// (2^-53 |tA||x|); the FP64 pipe, which bounds that form (8 operations a point, 201 us at 96^3, p = 16, now 104 us),
+// is not used.
+struct StencilDF {
+    float ch, cl, lh[3], ll[3], uh[3], ul[3];
+};
+
+__device__ __forceinline__ void df_term32(float& sh, float& sl, float v, float ch, float cl) {
+    const float pr = v * ch;
+    const float e = fmaf(v, cl, fmaf(v, ch, -pr));
+    df_add(sh, sl, pr);
+    sl += e;
+}
+
+__global__ void k_cd_next_residual(const double* __restrict__ R1, int64_t ldr, const float* __restrict__ D, int64_t ldd,
+                                   float* __restrict__ R2, int64_t ld2, int nx, int ny, int nz, StencilDF k) {
+    const unsigned n = (unsigned)nx * (unsigned)ny * (unsigned)nz;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = blockIdx.y;
+    if (i >= n) return;
+    const float* v = D + c * ldd;
+    const unsigned q = i / (unsigned)nx;
+    const unsigned ix = i - q * (unsigned)nx;
+    float sh, sl;
+    split_df_i(R1[c * ldr + i], sh, sl);
+    const unsigned iz = q / (unsigned)ny, iy = q - iz * (unsigned)ny;
+    const unsigned st = (unsigned)nx * (unsigned)ny;
+    df_term32(sh, sl, v[i], k.ch, k.cl);
+    if (ix > 0) df_term32(sh, sl, v[i - 1], k.lh[0], k.ll[0]);
+    if (ix < (unsigned)nx - 1) df_term32(sh, sl, v[i + 1], k.uh[0], k.ul[0]);
+    if (iy > 0) df_term32(sh, sl, v[i - nx], k.lh[1], k.ll[1]);
+    if (iy < (unsigned)ny - 1) df_term32(sh, sl, v[i + nx], k.uh[1], k.ul[1]);
+    if (iz > 0) df_term32(sh, sl, v[i - st], k.lh[2], k.ll[2]);
+    if (iz < (unsigned)nz - 1) df_term32(sh, sl, v[i + st], k.uh[2], k.ul[2]);
+    R2[c * ld2 + i] = sh + sl;
 }
 
 // The same stencil in double-float arithmetic on the FP32 pipe, for mixed-precision plans:
@@ -399,9 +438,6 @@ __global__ void k_cd_apply(const double* __restrict__ V, int64_t ldv, double* __
 // FP64 FMAs per SM per clock, so the FP64 stencil (5 or 7 per point) is bound by the FP64
 // pipe, not by memory; the pair arithmetic is ~2^-48 accurate, the level of the mixed path's
 // other double-float kernels.  Y (the refinement's right-hand side) enters with beta = 1.
-struct StencilDF {
-    float ch, cl, lh[3], ll[3], uh[3], ul[3];
-};
 
 __device__ __forceinline__ void df_term(float& sh, float& sl, double v, float ch, float cl) {
     float vh, vl;
@@ -788,6 +824,22 @@ cudaError_t launch_cd_apply(const double* V, int64_t ldv, double* W, int64_t ldw
     }
     dim3 grid((unsigned)((n + 255) / 256), p);
     k_cd_apply<<<grid, 256, 0, s>>>(V, ldv, W, ldw, ndim, nx, ny, nz, k, Y, ldy, beta, W32);
+    return cudaGetLastError();
+}
+
+// R2 = R1 - tA D (see k_cd_next_residual)
+cudaError_t launch_cd_next_residual(const double* R1, int64_t ldr, const float* D, int64_t ldd, float* R2, int64_t ld2,
+                                    int p, int nx, int ny, int nz, const Axis* ax, double t, cudaStream_t s) {
+    const int64_t n = (int64_t)nx * ny * nz;
+    if (n >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+    StencilDF k;
+    split_host(-t * (ax[0].c + ax[1].c + ax[2].c), k.ch, k.cl);
+    for (int d = 0; d < 3; ++d) {
+        split_host(-t * ax[d].l, k.lh[d], k.ll[d]);
+        split_host(-t * ax[d].u, k.uh[d], k.ul[d]);
+    }
+    const dim3 grid((unsigned)((n + 255) / 256), p);
+    k_cd_next_residual<<<grid, 256, 0, s>>>(R1, ldr, D, ldd, R2, ld2, nx, ny, nz, k);
     return cudaGetLastError();
 }
 

@@ -14,12 +14,15 @@
 // lane (cp.async, 16 bytes at a time, four chunks ahead across tiles; no barrier): the K index inside a
 // 16-deep chunk and the row index inside a 32-row tile are permuted (lane t holds k = 4t .. 4t + 3,
 // lane group g holds rows 4g .. 4g + 3), which any MMA allows as long as both operands agree.  Q is
-// split once when the plan is made and stored in fragment order; a CTA keeps the slab of its 32
-// columns in shared memory and its warps walk over 32-row tiles.
+// split once when the plan is made and stored in fragment order; a CTA keeps the slab of its 32 or 48
+// columns in shared memory and its warps walk over 32-row tiles.  96^3, p = 16, all 12 transforms of a
+// block step: 1.50 -> 0.95 ms (61 to 72 us each, 100 us into FP64; 8 bytes a value at 3.7 TB/s), bound now by
+// dependent issue at 8 to 12 warps per SM and 48 % of the mma.sync rate.
 //
 //   IN_M  (rows contiguous in A)        OUT_M (rows contiguous in C): Q is the left operand (M = n)
 //   IN_K  (k contiguous in A)           OUT_N (n contiguous in C):    A is the left operand (M = m)
 #include <algorithm>
+#include <type_traits>
 
 #include "df.cuh"
 #include "internal.h"
@@ -51,7 +54,8 @@ constexpr size_t slab_bytes(int K, int NTS) { return (size_t)((K + 15) / 16) * N
 // NTS: 16-column tiles of C per warp (a 16 x 32 chunk of A is split once for NTS tiles; the splitting
 // and addressing take more issue slots than the MMAs).
 template <int VAR, typename TC, int NTS, bool VA, bool FL>
-__global__ void __launch_bounds__(kTrThreads, VA ? 3 : 2) k_transform(TransformArgs g, int batch, int qsm, int vc) {
+__global__ void __launch_bounds__(kTrThreads, VA ? 3 : 2) k_transform(TransformArgs g, int batch, int qsm, int vc,
+                                                                        const float* add_to, int64_t add_b) {
     extern __shared__ __align__(16) unsigned char smt[];
     const int tid = threadIdx.x, lane = tid & 31, gq = lane >> 2, t = lane & 3;
     const int nt16 = (g.N + 15) >> 4, nt0 = blockIdx.y * NTS, nts = min(NTS, nt16 - nt0);
@@ -126,6 +130,10 @@ __global__ void __launch_bounds__(kTrThreads, VA ? 3 : 2) k_transform(TransformA
     for (int job = blockIdx.x * (kTrThreads / 32) + (tid >> 5); job < jobs; job += jstep) {
     const int bb = job / mtiles, m0 = (job - bb * mtiles) * 32;
     TC* C = reinterpret_cast<TC*>(g.C) + (int64_t)bb * g.c_b;
+    // the extra addend, in the one variant that takes it (a kernel argument of its own: inside TransformArgs it
+    // changed the code of every variant, 5 % slower at 256 x 256)
+    constexpr bool kAdd = VAR == T_IN_M_OUT_M && std::is_same<TC, double>::value;
+    const float* add = kAdd && add_to ? add_to + (int64_t)bb * add_b : nullptr;
     float cm[NTS][4][4], cc[NTS][4][4], cs[FL ? NTS : 1][4][4];
 #pragma unroll
     for (int i = 0; i < NTS; ++i)
@@ -246,6 +254,7 @@ __global__ void __launch_bounds__(kTrThreads, VA ? 3 : 2) k_transform(TransformA
                 };
                 if constexpr (sizeof(TC) == 8) {
                     double2 o[4];
+                    float2 o32[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         o[k] = make_double2(0.0, 0.0);
@@ -257,10 +266,24 @@ __global__ void __launch_bounds__(kTrThreads, VA ? 3 : 2) k_transform(TransformA
                                 if (ro[2 * k + 1] >= 0) o[k].y = Cn[ro[2 * k + 1]];
                             }
                         }
+                        if constexpr (kAdd) o32[k] = make_float2(0.f, 0.f);
+                        if (kAdd && add) {
+                            const float* an = add + (int64_t)n * g.c_cs;
+                            if (vc) {
+                                if (ro[2 * k] >= 0) o32[k] = *reinterpret_cast<const float2*>(an + ro[2 * k]);
+                            } else {
+                                if (ro[2 * k] >= 0) o32[k].x = an[ro[2 * k]];
+                                if (ro[2 * k + 1] >= 0) o32[k].y = an[ro[2 * k + 1]];
+                            }
+                        }
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         double2 v = make_double2(f64_of_f32_i(val(2 * k)), f64_of_f32_i(val(2 * k + 1)));
+                        if (kAdd && add) {
+                            v.x += f64_of_f32_i(o32[k].x);
+                            v.y += f64_of_f32_i(o32[k].y);
+                        }
                         if (g.accumulate) {
                             v.x += o[k].x;
                             v.y += o[k].y;
@@ -311,7 +334,8 @@ __global__ void k_table_frags(const double* __restrict__ Q, int N, uint4* __rest
 }
 
 template <int VAR, typename TC>
-cudaError_t launch_var(const TransformArgs& g, int batch, int sms, cudaStream_t s) {
+cudaError_t launch_var(const TransformArgs& g, int batch, int sms, cudaStream_t s, const float* add = nullptr,
+                       int64_t add_b = 0) {
     // aligned groups of four of A and aligned pairs of C: strides between them multiples of 4 (2) and
     // no group crossing a run of the split row index
     auto mult = [](int64_t x, int k) { return x % k == 0; };
@@ -320,7 +344,8 @@ cudaError_t launch_var(const TransformArgs& g, int batch, int sms, cudaStream_t 
     const bool va = am && mult(g.a_b, 4) && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
     const bool cmv = VAR == T_IN_M_OUT_N ? mult(g.c_rs, 2) && mult(g.c_ms2, 2) && mult(g.N, 2)
                                          : mult(g.c_cs, 2) && mult(g.ms, 2) && mult(g.c_ms2, 2) && mult(g.M, 2);
-    const bool vc = cmv && mult(g.c_b, 2) && (reinterpret_cast<uintptr_t>(g.C) & (2 * sizeof(TC) - 1)) == 0;
+    const bool vc = cmv && mult(g.c_b, 2) && (reinterpret_cast<uintptr_t>(g.C) & (2 * sizeof(TC) - 1)) == 0 &&
+                    (!add || (mult(add_b, 2) && (reinterpret_cast<uintptr_t>(add) & 7) == 0));
     // column tiles per warp: three on short axes (no flush); two on long ones, where the flush costs an
     // accumulator and the smaller 2-D problems need the warps (256 x 256, p = 8: 14 us against 29 us
     // with four tiles, 512 x 352, p = 32: 104 us against 152 us with three)
@@ -336,9 +361,9 @@ cudaError_t launch_var(const TransformArgs& g, int batch, int sms, cudaStream_t 
     const int64_t gmax = std::max<int64_t>(1, std::min((jobs + 3) / 4, std::max<int64_t>(1, resident / ngroups)));
     const int64_t per = (jobs + 4 * gmax - 1) / (4 * gmax);
     const dim3 grid((unsigned)((jobs + 4 * per - 1) / (4 * per)), (unsigned)ngroups);
-    if (!va) k_transform<VAR, TC, 2, false, true><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc);
-    else if (fl) k_transform<VAR, TC, 2, true, true><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc);
-    else k_transform<VAR, TC, 3, true, false><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc);
+    if (!va) k_transform<VAR, TC, 2, false, true><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc, add, add_b);
+    else if (fl) k_transform<VAR, TC, 2, true, true><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc, add, add_b);
+    else k_transform<VAR, TC, 3, true, false><<<grid, kTrThreads, shm, s>>>(g, batch, qsm, vc, add, add_b);
     return cudaGetLastError();
 }
 
@@ -368,11 +393,12 @@ cudaError_t launch_table_frags(const double* Q, int N, uint4* F, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s) {
+cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s, const float* add, int64_t add_b) {
+    if (add && !(g.c_rs == 1 && g.a_cs != 1 && g.c_f64)) return cudaErrorInvalidValue;
     if (g.c_rs == 1) {
         if (g.a_cs == 1)
             return g.c_f64 ? launch_var<T_IN_K_OUT_M, double>(g, batch, sms, s) : launch_var<T_IN_K_OUT_M, float>(g, batch, sms, s);
-        return g.c_f64 ? launch_var<T_IN_M_OUT_M, double>(g, batch, sms, s) : launch_var<T_IN_M_OUT_M, float>(g, batch, sms, s);
+        return g.c_f64 ? launch_var<T_IN_M_OUT_M, double>(g, batch, sms, s, add, add_b) : launch_var<T_IN_M_OUT_M, float>(g, batch, sms, s);
     }
     if (g.c_cs != 1 || g.a_rs != 1 || g.c_f64) return cudaErrorInvalidValue;
     return launch_var<T_IN_M_OUT_N, float>(g, batch, sms, s);

@@ -14,6 +14,7 @@ bounds of those passes' own tests).
 """
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 from oracle import cf, operators as ops, psbfom as ps
 from paper_1405_0707_gb300 import inputs
@@ -97,3 +98,39 @@ def test_fp64_digit_passes_reach_fp64_rounding(sides, p, m, local):
     plan.close()
     assert np.linalg.norm(W - V @ H) <= 1e-13 * np.linalg.norm(W)
     assert np.linalg.norm(V.T @ V - np.eye((m + 1) * p)) <= 1e-13
+
+
+def _times_longdouble(A, X):
+    A, Y = A.tocsr(), np.zeros(X.shape, dtype=np.longdouble)
+    X = X.astype(np.longdouble)
+    for k in range(int(np.diff(A.indptr).max())):
+        rows = np.nonzero(np.diff(A.indptr) > k)[0]
+        idx = A.indptr[rows] + k
+        Y[rows] += A.data[idx].astype(np.longdouble)[:, None] * X[A.indices[idx]]
+    return Y
+
+
+@pytest.mark.parametrize("local", [False, True])
+@pytest.mark.parametrize("sides,diff,vel,t,p", [((256, 256), 0.1, (1.0, -0.5), 1e-2, 8), ((61, 59), 0.1, (2.0, 1.0), 0.05, 3),
+                                                ((130, 65), 1.0, (0.0, 0.0), 1e-5, 32), ((2, 7), 1.0, (1.0, -0.5), 0.1, 2),
+                                                ((33, 31, 29), 0.1, (1.0, -0.5, 0.3), 1e-3, 9),
+                                                ((40, 37, 35), 0.1, (1.0, -1.0, 1.0), 0.1, 16)])
+def test_refined_inverse_backward_error(sides, diff, vel, t, p, local):
+    """The second correction starts from the first residual (r - tA d in float pairs) and both are added to
+    x at once.  With u = 2^-53: the first residual carries at most 8 roundings of |tA||x|, the addition to
+    x one, the pairs below 2^-40 of them and the third power of the FP32 inverse's error
+    below all of it, so the residual in 64-bit-mantissa arithmetic stays under 16 u |tA||x| normwise."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    n = int(np.prod(sides))
+    V = inputs.rhs(n, p, 79)
+    if local:
+        V = np.zeros((n, p), order="F")
+        V[np.linspace(0, n - 1, p).astype(int), np.arange(p)] = 1.0
+    plan = Plan(sides, diff, vel, p_max=p, m=2, precision="mixed")
+    W = to_np(plan.prec_apply(t, to_dev(V)))
+    plan.close()
+    A = sp.csr_matrix(ops.cd_matrix(sides, diff, vel, t))
+    R = V.astype(np.longdouble) - _times_longdouble(A, W)
+    scale = abs(A).sum(axis=1).max() * np.abs(W).max(axis=0)
+    assert np.all(np.abs(R).max(axis=0) <= 16 * 2.0 ** -53 * scale)
