@@ -50,15 +50,14 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070  # SMs x FP32 lanes x flop/FMA x GHz = 
 # both reproducible on the device with `python bench.py --component fmapeak` (expm_peak_fma)
 L2_FLUSH_BYTES = 512 << 20
 KERNEL_OF = {"gemm": "k_gemm (DST-I transforms of the exact inverse, FP64)",
-             "cgs": "k_proj/k_update (block CGS2 row passes, FP64)",
-             "cgs_mixed": "k_cgs_rows / k_proj_tc / k_cgs_tc (first block CGS2 pass: projection in FP32, or TF32 "
-                          "hi/lo products on the tensor cores; update in double-float fused with the FP32 second "
-                          "projection and the double-float Gram matrix, or exact bf16 slices on the tensor cores)",
-             "qr_mixed": "k_qr_mixed_rows (second CGS pass's FP32 correction fused with one accurate Cholesky-QR "
+             "cgs": "k_proj64/k_upd_mma (block CGS2 passes, exact digit products; k_proj/k_update in FP64 for small blocks)",
+             "cgs_mixed": "k_proj_mma / k_upd_mma (block CGS2: projections from an FP32 copy of the basis in six "
+                          "bf16 products, update in exact fp16 digit products with the Gram matrix in float pairs)",
+             "qr_mixed": "k_qr_apply (second CGS pass's FP32 correction fused with one accurate Cholesky-QR "
                          "pass: double-float factor applied exactly in double-float; FP32 deviation passes only "
                          "for ill-conditioned blocks)",
              "tridiag_mixed": "k_tridiag_tile32 (FP32 Thomas line solves, segmented affine scans)",
-             "gemm_mixed": "k_gemm32 (FP32 DST-I transforms of the exact inverse)",
+             "gemm_mixed": "k_transform (DST-I transforms of the exact inverse, FP32 operands in six bf16 products)",
              "fft_mixed": "k_fft_cols/k_fft_rows (four-step FFT Toeplitz product, double-float)",
              "gsf_mixed": "k_fft_cols/k_fft_rows (Gohberg-Semencul inverse, double-float)",
              "stencil": "k_cd_apply (stencil W = tA V, FP64)",

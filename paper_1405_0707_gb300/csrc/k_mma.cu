@@ -27,6 +27,10 @@
 //    (2^-32 of the largest scaled entry of its column, finer than the FP32 projection it came
 //    from), subtracts V times exactly that h and records exactly that h in H: the relation does
 //    not see the rounding, and 22 digit products replace 27.  The Z update keeps six digits.
+//
+// Measured, 96^3, p = 16, per block step averaged over a 10-step cycle: Gram-Schmidt 1.09 -> 0.66 ms
+// (projection 62 us at 16 and 243 us at 160 columns, 2.8 TB/s, bound by the loads in flight; update 218 and
+// 516 us, 2.6 TB/s, bound by issue slots at 12 to 16 warps per SM), 512 x 352, p = 32: 3.3 -> 0.6 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>

@@ -1,4 +1,4 @@
-// k_poles.cu -- the projected shifted systems, one CTA per pole.
+// k_poles.cu -- the projected shifted systems, one CTA or one cluster of CTAs per pole.
 //
 // For each pole tau_i (Im > 0) in one launch, Algorithm 2:
 //   (I - tau_i H_m) Z_i = E_1 S_i                              eq. (3236)
