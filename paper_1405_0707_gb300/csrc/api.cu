@@ -941,7 +941,10 @@ void free_plan(expm_plan* P) {
 template <class T>
 bool dalloc(T** p, size_t count) {
     if (count == 0) count = 1;
-    return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * count) == cudaSuccess;
+    if (cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * count) != cudaSuccess) return false;
+    // test switch: every byte of a new buffer holds this value (0..255) in place of what the allocator left there
+    const char* fill = std::getenv("EXPM_FILL_BYTE");
+    return !fill || (cudaMemset(*p, std::atoi(fill), sizeof(T) * count) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess);
 }
 
 // ---- Toeplitz plan setup

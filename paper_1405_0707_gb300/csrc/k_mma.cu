@@ -604,14 +604,16 @@ k_upd_mma(const UpdArgs A) {
                 }
             }
         if (GS) {
-            // Gram entries of the tile's 16 rows (zero past n and p) from float pairs
+            // Gram entries of the tile's 16 rows from float pairs.  Rows past n are set to zero here: V's
+            // padding rows hold whatever the allocation did, and -V h of them is no part of W
+            const bool in0 = r < n, in1 = r + 1 < n;
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     float wh, wl;
-                    split_df_i(w[j][q], wh, wl);
+                    split_df_i((q < 2 ? in0 : in1) ? w[j][q] : 0.0, wh, wl);
                     gw[(2 * g + (q >> 1)) * (NCOL + 1) + 8 * j + 2 * t + (q & 1)] = make_float2(wh, wl);
                 }
             __syncwarp();

@@ -1,0 +1,69 @@
+"""A plan's results do not depend on what its workspace held when it was allocated.
+
+EXPM_FILL_BYTE makes plan creation fill every buffer with one byte: 0, 0x3F (FP64 4.8e-4, the size of a
+basis entry), 0x41 (2.3e6, far above one) and 0xFF (NaN).  Every solve is deterministic, so the results
+have to be the same bit for bit.  The row counts leave 1, 8 and 15 rows in the last 16-row tile and 1 to
+31 in the columns' padding.
+"""
+import numpy as np
+import pytest
+
+from paper_1405_0707_gb300 import inputs
+from tests.gpu_util import need_gpu, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+FILLS = (0, 0x3F, 0x41, 0xFF)
+
+
+def _plan(kind, **kw):
+    from paper_1405_0707_gb300 import Plan
+    if kind == "toeplitz":
+        return Plan.toeplitz(inputs.toeplitz_column(20), 703, **kw), 0.9
+    if kind == "csr":
+        indptr, indices, data = inputs.sparse_stencil_matrix((11, 9, 7), seed=3)
+        return Plan.csr((data, indices, indptr), **kw), 0.3
+    return Plan(kind, 0.1, (1.0, -0.5, 0.3)[:len(kind)], **kw), 0.05
+
+
+def _same(run, monkeypatch):
+    out = []
+    for fill in FILLS:
+        monkeypatch.setenv("EXPM_FILL_BYTE", str(fill))
+        out.append(run())
+    assert all(np.all(np.isfinite(x)) for x in out[0])
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("kind,p,opts", [((41, 25), 3, {}), ((23, 24), 8, {}), ((53, 35), 16, {}), ((27, 13), 24, {}),
+                                         ((13, 11, 9), 4, {}), ((7,), 1, {}), ((401, 251), 1, {}), ((97, 83), 13, {}),
+                                         ((33, 29), 3, dict(k_defl=6)), ((33, 29), 6, dict(certify=True)),
+                                         ("toeplitz", 3, {}), ("csr", 3, {})])
+def test_solve_is_independent_of_the_workspace(kind, p, opts, precision, monkeypatch):
+    need_gpu()
+
+    def run():
+        plan, t = _plan(kind, p_max=p, m=5, tol=1e-10, max_cycles=60, precision=precision, **opts)
+        Z, info = plan.expm_block(t, to_dev(inputs.rhs(plan.n, p, 5)))
+        plan.close()
+        return to_np(Z), np.array(list(info.resid))
+
+    _same(run, monkeypatch)
+
+
+@pytest.mark.parametrize("sides,p,m", [((97, 83), 16, 6), ((41, 25), 3, 8), ((61, 59), 8, 10), ((130, 65), 32, 3)])
+def test_arnoldi_is_independent_of_the_workspace(sides, p, m, monkeypatch):
+    need_gpu()
+    n = int(np.prod(sides))
+    V1 = np.linalg.qr(inputs.rhs(n, p, 8))[0]
+
+    def run():
+        plan, t = _plan(sides, p_max=p, m=m, precision="mixed")
+        V, H = plan.arnoldi(t, to_dev(V1))
+        plan.close()
+        return to_np(V), to_np(H)
+
+    _same(run, monkeypatch)
