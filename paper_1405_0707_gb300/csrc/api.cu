@@ -1660,15 +1660,17 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         }
     }
     if (P->mma) {
-        // last, the FP32 copy of the basis (half the basis again): a plan that has no room for it runs on
-        // the kernels that read the FP64 basis alone
-        const size_t v32 = (size_t)ld * (m + 1) * p_max;
-        if (!dalloc(&P->V32, v32)) {
+        // last, the FP32 copy of the basis (half the basis again), its padding rows zero: a plan that has no
+        // room for it runs on the kernels that read the FP64 basis alone
+        const size_t cols = (size_t)(m + 1) * p_max;
+        if (!dalloc(&P->V32, (size_t)ld * cols)) {
             cudaGetLastError();
             P->V32 = nullptr;
             P->mma = false;
-        } else if (cudaMemsetAsync(P->V32, 0, sizeof(float) * v32, s) != cudaSuccess ||
-                   cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, s) != cudaSuccess) {
+        } else if ((ld > n && cudaMemset2DAsync(P->V32 + n, sizeof(float) * ld, 0, sizeof(float) * (ld - n), cols, s) != cudaSuccess) ||
+                   cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, s) != cudaSuccess ||
+                   // a batch graph runs on a stream of its own, which nothing orders after this one
+                   cudaStreamSynchronize(s) != cudaSuccess) {
             cudaGetLastError();
             free_plan(P);
             return EXPM_CUDA_ERROR;

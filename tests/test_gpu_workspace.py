@@ -67,3 +67,25 @@ def test_arnoldi_is_independent_of_the_workspace(sides, p, m, monkeypatch):
         return to_np(V), to_np(H)
 
     _same(run, monkeypatch)
+
+
+def test_batch_runs_right_after_its_plans_are_made():
+    """Plan creation returns with nothing of its own pending on the plan's stream: a batch graph, which runs
+    on another stream, may follow at once."""
+    torch = need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    from paper_1405_0707_gb300.api import Batch
+    probs = [((61, 59, 47), 8), ((45, 41, 39), 3), ((300, 301), 16)]
+    Bs = [to_dev(inputs.rhs(int(np.prod(s)), p, 3)) for s, p in probs]
+    streams = [torch.cuda.Stream() for _ in range(len(probs) + 1)]
+    torch.cuda.synchronize()
+    for _ in range(4):
+        plans = [Plan(s, 1.0, (1.0, -1.0, 0.5)[:len(s)], p_max=p, m=5, fixed_cycles=2, precision="mixed", stream=q)
+                 for (s, p), q in zip(probs, streams)]
+        batch = Batch(plans, [1e-3] * len(probs), Bs, stream=streams[-1])
+        first = [to_np(Z) for Z in batch.run()[0]]
+        for a, Z in zip(first, batch.run()[0]):
+            assert np.array_equal(a, to_np(Z))
+        batch.close()
+        for plan in plans:
+            plan.close()
