@@ -565,13 +565,17 @@ k_upd_mma(const UpdArgs A) {
                     const int k = fmax_s[8 * j + 2 * t + (q & 1)] - (D64 ? 12 : 14);
                     constexpr bool SUB = MODE == U_GS || MODE == U_GS64;
                     if constexpr (!D64) {
-                        // levels 0..2 exactly in a float pair (40 bits), the others, 2^-24 below, in FP32
-                        float sh = acc[2][j][q] * 0x1p-16f, sl = 0.f;
+                        // levels 0..3 in a float pair (exact but for the last bit of 49), 4..6, 2^-32 below, in
+                        // FP32.  An error at 2^-48 of the largest V h counts on every row, and rows far below
+                        // it (a localised block) have many: with level 3 in FP32 as well, the relation's
+                        // error was 1.3e-13 in place of 4e-15 (33 x 31 x 29, unit vectors; pairs throughout, before the
+                        // digits, 1e-14)
+                        float sh = acc[3][j][q] * 0x1p-24f, sl = 0.f;
+                        df_add(sh, sl, acc[2][j][q] * 0x1p-16f);
                         df_add(sh, sl, acc[1][j][q] * 0x1p-8f);
                         df_add(sh, sl, acc[0][j][q]);
                         float lo = fmaf(acc[6][j][q], 0x1p-48f, acc[5][j][q] * 0x1p-40f);
                         lo = fmaf(acc[4][j][q], 0x1p-32f, lo);
-                        lo = fmaf(acc[3][j][q], 0x1p-24f, lo);
                         sl += lo;
                         const double x = scaled_f32(sh, k), y = scaled_f32(sl, k);
                         w[j][q] = SUB ? (w[j][q] - x) - y : (w[j][q] + x) + y;

@@ -1,0 +1,41 @@
+"""Accuracy of the mixed path's block step on blocks whose columns are localised (unit vectors), spread out, or
+both: the cases where one row or one column dominates a product and the rest has to keep its own digits."""
+import numpy as np
+import pytest
+
+from paper_1405_0707_gb300 import inputs
+from tests.gpu_util import need_gpu, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [((33, 31, 29), 9, 5), ((300, 300), 4, 10), ((97, 83), 16, 6), ((130, 65), 32, 4), ((64, 40), 17, 6),
+          ((129, 127), 1, 12)]
+
+
+def _start(kind, n, p):
+    V1 = inputs.rhs(n, p, 8)
+    if kind != "spread":
+        first = 0 if kind == "local" else p // 2
+        V1[:, first:] = 0.0
+        V1[np.linspace(1, n - 2, p - first).astype(int), np.arange(first, p)] = 1.0
+    return np.linalg.qr(V1)[0]
+
+
+def _arnoldi(sides, p, m, V1):
+    from paper_1405_0707_gb300 import Plan
+    plan = Plan(sides, 0.1, (1.0, -0.5, 0.3)[:len(sides)], p_max=p, m=m, precision="mixed")
+    V, H = plan.arnoldi(0.05, to_dev(V1))
+    W = np.column_stack([to_np(plan.prec_apply(0.05, V[:, j * p:(j + 1) * p])) for j in range(m)])
+    plan.close()
+    return to_np(V), to_np(H), W
+
+
+@pytest.mark.parametrize("kind", ["local", "half", "spread"])
+@pytest.mark.parametrize("sides,p,m", SHAPES)
+def test_relation(sides, p, m, kind):
+    """(tA)^{-1} V_m = V_{m+1} H~_m.  V's digits resolve 2^-55 of a column's largest entry on each of the n <= 2^17
+    rows (2^-46.5 of a unit column), the update's and the substitution's float pairs 2^-48 of the sums they
+    hold, the FP32 correction V h2 2^-24 of an h2 near 2^-23 |W|: together below 2^-45 |W|."""
+    need_gpu()
+    V, H, W = _arnoldi(sides, p, m, _start(kind, int(np.prod(sides)), p))
+    assert np.linalg.norm(W - V @ H) <= 2.0 ** -45 * np.linalg.norm(W)
