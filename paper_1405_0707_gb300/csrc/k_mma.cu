@@ -15,8 +15,8 @@
 //    FP32 rounding is the one the CUDA-core projection applied on each read), half the bytes.
 //    Each FP32 value is split exactly enough into three bf16 parts, and the six products
 //    v0w0 | v0w1 v1w0 v1w1 v0w2 v2w0 go to two accumulators (the second 2^-8 smaller), so the
-//    product error is ~2^-25, below the FP32 rounding of the operands.  Every few hundred rows
-//    the main accumulator is added to a float pair, so summation error does not grow with n.
+//    product error is ~2^-25, below the FP32 rounding of the operands.  Every 16 rows the
+//    main accumulator is added to a float pair, so summation error does not grow with n.
 //  * The update must hold to FP64 rounding (the Arnoldi relation of eq. (4.5)).  Both operands
 //    are cut into balanced base-256 digits held exactly in fp16, products of digits are summed
 //    by level (digit positions i + j) in FP32 accumulators that stay below 2^24, hence exact,
@@ -118,7 +118,6 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
         }
     };
     int64_t u = blockIdx.x;
-    int since = 0;
     float4 v[MTW][2];
 #pragma unroll
     for (int i = 0; i < MTW; ++i) v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);   // tiles past nmt
@@ -176,22 +175,19 @@ k_proj_mma(const float* __restrict__ V, int64_t ldv, int cols, const double* __r
                             for (int j = 0; j < NT; ++j)
                                 mma_bf16(pr == 0 ? cm[i0 + i][j] : cc[i0 + i][j], a[i][kProdA[pr]], wb[j][kProdB[pr]].x,
                                          wb[j][kProdB[pr]].y);
-                }
-        }
-        // every eight blocks of this warp (CG of them per unit), and at the end
-        since += CG;
-        if (since >= kProjKb || un >= units) {
-            since = 0;
+                    // the main sums go to the float pairs after every block: the MMA truncates towards zero,
+                    // so a sum that one row dominates and the rest cancels drifts by 2^-24 of it per block
+                    // (300 x 300, unit vectors, orthogonality: 1.0e-7 with eight blocks, 9e-9 with one, no
+                    // difference in time)
 #pragma unroll
-            for (int i = 0; i < MTW; ++i)
-                if (i < nmt) {
+                    for (int i = 0; i < 2; ++i)
 #pragma unroll
-                    for (int j = 0; j < NT; ++j)
+                        for (int j = 0; j < NT; ++j)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            df_add(ch[i][j][q], cc[i][j][q], cm[i][j][q]);
-                            cm[i][j][q] = 0.f;
-                        }
+                            for (int q = 0; q < 4; ++q) {
+                                df_add(ch[i0 + i][j][q], cc[i0 + i][j][q], cm[i0 + i][j][q]);
+                                cm[i0 + i][j][q] = 0.f;
+                            }
                 }
         }
         buf ^= 1;

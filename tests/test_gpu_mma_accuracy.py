@@ -39,3 +39,13 @@ def test_relation(sides, p, m, kind):
     need_gpu()
     V, H, W = _arnoldi(sides, p, m, _start(kind, int(np.prod(sides)), p))
     assert np.linalg.norm(W - V @ H) <= 2.0 ** -45 * np.linalg.norm(W)
+
+
+@pytest.mark.parametrize("kind", ["local", "half", "spread"])
+@pytest.mark.parametrize("sides,p,m", SHAPES)
+def test_orthogonality(sides, p, m, kind):
+    """The projections read V and W rounded to FP32 and add 16-row sums in float pairs: their error is that of
+    the operands' rounding, 2^-24 of |V||W| entry by entry, whichever rows dominate."""
+    need_gpu()
+    V, _, _ = _arnoldi(sides, p, m, _start(kind, int(np.prod(sides)), p))
+    assert np.abs(V.T @ V - np.eye((m + 1) * p)).max() <= 2.0 ** -24
