@@ -127,7 +127,7 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
     }
     // G - h2^T h2.  The correction is ~2^-40 of G unless the first pass cancelled almost all of W,
     // so its products are formed in FP32 first; only when a diagonal entry's correction passes
-    // 2^-20 of it are they formed again in float pairs (G needs ~2^-48).
+    // 2^-24 of it are they formed again in float pairs (G needs ~2^-48).
     for (int full = 0; full < 2; ++full) {
 #pragma unroll
         for (int k = 0; k < KI; ++k) ah[k] = al[k] = 0.f;
@@ -168,7 +168,7 @@ k_reduce_factor(const double* __restrict__ part, int nblk, const double* __restr
             const int o = i * p + i + rem;
             float gh, gl;
             split_df_i(scale_pow2(__ldcg(h + nh + o), -kexp), gh, gl);
-            if (rem == 0 && !full && ch > 0x1p-20f * gh) big = 1;
+            if (rem == 0 && !full && ch > 0x1p-24f * gh) big = 1;
             df_add(gh, gl, -ch);
             gl -= cl;
             Gs[o] = make_float2(gh, gl);
