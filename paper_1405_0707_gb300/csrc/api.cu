@@ -603,14 +603,18 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
         LAUNCH(EXPM_STAGE_OTHER, launch_update_z(P->V, ld, mp + p, 2 * P->npoles * p, n, P->Ccert, P->Xcert, ld, 0,
                                                  s, P->nblk));
     }
-    // mixed path: the product V Wc in double-float on the FP32 pipe (FP64 accumulation into Z)
+    // Z += V Wc and the restart copy, by digit products; without them in double-float (mixed) or FP64
     // (with deflation the restart happens in the next cycle's prologue, after V_m P_k)
     const bool defl = P->opts.k_defl > 0;
-    if (P->mma || use64(P, p))
+    if ((P->mma || use64(P, p)) && updz_mma_fit(mp + p, p)) {
         LAUNCH(EXPM_STAGE_UPDATE, launch_updz_mma(P->V, P->V32, ld, mp + p, P->Zacc, ld, p, n, sm(P, kOffWc), P->colexp,
                                                   flags_of(P->stat), defl ? 0 : 1, P->sms_rows, s));
-    else LAUNCH(EXPM_STAGE_UPDATE, launch_update_z(P->V, ld, mp + p, p, n, sm(P, kOffWc), P->Zacc, ld, defl ? 0 : 1, s,
-                                              P->nblk, P->opts.precision == EXPM_PREC_MIXED ? 1 : 0));
+    } else {
+        LAUNCH(EXPM_STAGE_UPDATE, launch_update_z(P->V, ld, mp + p, p, n, sm(P, kOffWc), P->Zacc, ld, defl ? 0 : 1, s,
+                                                  P->nblk, P->opts.precision == EXPM_PREC_MIXED ? 1 : 0));
+        // mixed plans with (m + 1) p > 432 and p > 16 (FP64 plans of that size do not take the digit passes)
+        if (P->mma && !defl) LAUNCH(EXPM_STAGE_UPDATE, launch_pack_block(P->V, P->V32, ld, n, p, P->colexp, nullptr, s));
+    }
     if (!d2h) return EXPM_OK;   // the batch graph's stop test reads the status on the device
     CK(cudaMemcpyAsync(P->hpin, P->stat, sizeof(double) * kStatDoubles, cudaMemcpyDeviceToHost, s));
     if (defl) CK(cudaMemcpyAsync(P->hH, P->H, sizeof(double) * (size_t)P->ldH * mp, cudaMemcpyDeviceToHost, s));

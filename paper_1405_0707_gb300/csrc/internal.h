@@ -335,6 +335,7 @@ cudaError_t cgs_tc_set_smem_limits();
 // the FP32 basis copy (nb partials of cols x p), update with the Gram partials (nb of p x p) and
 // the rounded h recorded in H, Z update with the restart copy; V32 and colexp of other blocks.
 bool mma_fit(int mp, int p);
+bool updz_mma_fit(int cols, int p);   // of launch_updz_mma: its coefficients' digits fit in shared memory
 cudaError_t launch_proj_mma(const float* V32, int64_t ldv, int cols, const double* W, int64_t ldw, int p, int64_t n,
                             double* part, int max_blocks, int sms, int* nb, cudaStream_t s);
 cudaError_t launch_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t ldw, int p, int64_t n, const double* h,

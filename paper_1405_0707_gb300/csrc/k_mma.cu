@@ -25,8 +25,12 @@
 //    2^-55 of that entry.
 //  * h of the first pass only seeds the second pass, so the update rounds it to four digits
 //    (2^-32 of the largest scaled entry of its column, finer than the FP32 projection it came
-//    from), subtracts V times exactly that h and records exactly that h in H: the relation does
-//    not see the rounding, and 22 digit products replace 27.  The Z update keeps six digits.
+//    from unless the columns' largest entries differ by more than 2^8, where the second pass has
+//    that much more to correct), subtracts V times exactly that h and records exactly that h in H:
+//    the relation does not see the rounding, and 22 digit products replace 28.  The Z update keeps
+//    all seven digits of its coefficients (2^-55): beside a localised column, whose largest entry
+//    is one, six left the spread ones 2^-48 / their largest entry (90 x 77, p = 32, unit vectors:
+//    solution error 2.3e-14, now 1.5e-14).
 //
 // Measured, 96^3, p = 16, per block step averaged over a 10-step cycle: Gram-Schmidt 1.09 -> 0.66 ms
 // (projection 62 us at 16 and 243 us at 160 columns, 2.8 TB/s, bound by the loads in flight; update 218 and
@@ -328,7 +332,7 @@ enum UpdMode { U_GS = 0, U_Z = 1, U_GS64 = 2, U_Z64 = 3, U_MUL64 = 4 };
 // U_GS (NV = 7, NH = 4): W <- W - V h with h rounded as described at the top; CTA 0 records the rounded h
 // in H (columns hcol .., rows 0 .. cols - 1) and clears the next block's colexp; the Gram matrix of the
 // updated W in float pairs goes to partG[blk][p][p].
-// U_Z (7, 6): Z <- Z + V Wc, then the restart copy V[:, 0:p] <- V[:, cols-p:cols] of this CTA's rows (and
+// U_Z (7, 8, seven digits used): Z <- Z + V Wc, then the restart copy V[:, 0:p] <- V[:, cols-p:cols] of this CTA's rows (and
 // of V32) when asked.
 // U_GS64, U_Z64 (8, 8): the same products to FP64 rounding for FP64 plans (both operands to 2^-62 of
 // their column's largest entry, no Gram matrix, h not rounded).
@@ -419,7 +423,8 @@ k_upd_mma(const UpdArgs A) {
     }
     __syncthreads();
     if (tid == 0 && bad_s) atomicOr(&A.flags[0], 1);
-    constexpr int SC = D64 ? 62 : 8 * NH - 1;
+    constexpr int ND = D64 ? 8 : NH < NV ? NH : NV;       // digits of h (no product reaches past level NV - 1)
+    constexpr int SC = D64 ? 62 : 8 * ND - 1;
     for (int e = tid; e < nk * 16 * NCOL; e += kUpdThreads) {
         const int a = e / NCOL, c = e - a * NCOL;
         long long X = 0;
@@ -445,7 +450,9 @@ k_upd_mma(const UpdArgs A) {
 #pragma unroll
         for (int j = NH - 1; j >= 0; --j) {
             int d;
-            if (j > 0) {
+            if (j >= ND) {
+                d = 0;
+            } else if (j > 0) {
                 d = (int)((X + 128) & 255) - 128;
                 X = (X - d) >> 8;
             } else {
@@ -950,7 +957,7 @@ cudaError_t launch_upd_mma(double* V, int64_t ldv, int cols, double* W, int64_t 
 cudaError_t launch_updz_mma(double* V, float* V32, int64_t ldv, int cols, double* Z, int64_t ldz, int p, int64_t n,
                             const double* Wc, int* colexp, int* flags, int restart, int sms, cudaStream_t s) {
     UpdArgs a{V, ldv, cols, Z, ldz, p, n, Wc, colexp, nullptr, nullptr, 0, 0, flags, V32, restart};
-    cudaError_t e = V32 ? EXPM_UPD(7, 6, U_Z, 1 << 20, sms, nullptr, s) : EXPM_UPD(8, 8, U_Z64, 1 << 20, sms, nullptr, s);
+    cudaError_t e = V32 ? EXPM_UPD(7, 8, U_Z, 1 << 20, sms, nullptr, s) : EXPM_UPD(8, 8, U_Z64, 1 << 20, sms, nullptr, s);
     if (e == cudaSuccess && restart)
         e = cudaMemcpyAsync(colexp, colexp + cols - p, sizeof(int) * p, cudaMemcpyDeviceToDevice, s);
     return e;
@@ -1008,13 +1015,15 @@ cudaError_t launch_colmax(const double* W, int64_t ldw, int p, int64_t n, int* w
 
 bool mma_fit(int mp, int p) {
     const int NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
-    return p >= 1 && p <= kMaxP && upd_smem(mp, NT, 4, true) <= 220 * 1024 && upd_smem(mp + p, NT, 6, false) <= 220 * 1024;
+    return p >= 1 && p <= kMaxP && upd_smem(mp, NT, 4, true) <= 220 * 1024;
 }
 
-bool mma64_fit(int mp, int p) {
+bool updz_mma_fit(int cols, int p) {
     const int NT = p <= 8 ? 1 : p <= 16 ? 2 : 4;
-    return p >= 1 && p <= kMaxP && upd_smem(mp + p, NT, 8, false) <= 220 * 1024;
+    return p >= 1 && p <= kMaxP && upd_smem(cols, NT, 8, false) <= 220 * 1024;
 }
+
+bool mma64_fit(int mp, int p) { return updz_mma_fit(mp + p, p); }
 
 cudaError_t launch_pack_block(const double* V, float* V32, int64_t ld, int64_t n, int p, int* colexp, const int* skip,
                               cudaStream_t s) {
@@ -1030,7 +1039,7 @@ cudaError_t mma_set_smem_limits() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024)
     EXPM_SET((k_proj_mma<4, 2>));
     EXPM_SET((k_upd_mma<1, 7, 4, U_GS>)); EXPM_SET((k_upd_mma<2, 7, 4, U_GS>)); EXPM_SET((k_upd_mma<4, 7, 4, U_GS>));
-    EXPM_SET((k_upd_mma<1, 7, 6, U_Z>)); EXPM_SET((k_upd_mma<2, 7, 6, U_Z>)); EXPM_SET((k_upd_mma<4, 7, 6, U_Z>));
+    EXPM_SET((k_upd_mma<1, 7, 8, U_Z>)); EXPM_SET((k_upd_mma<2, 7, 8, U_Z>)); EXPM_SET((k_upd_mma<4, 7, 8, U_Z>));
     EXPM_SET((k_upd_mma<1, 8, 8, U_GS64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_GS64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_GS64>));
     EXPM_SET((k_upd_mma<1, 8, 8, U_Z64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_Z64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_Z64>));
     EXPM_SET((k_upd_mma<1, 8, 8, U_MUL64>)); EXPM_SET((k_upd_mma<2, 8, 8, U_MUL64>)); EXPM_SET((k_upd_mma<4, 8, 8, U_MUL64>));

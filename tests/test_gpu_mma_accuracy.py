@@ -49,3 +49,27 @@ def test_orthogonality(sides, p, m, kind):
     need_gpu()
     V, _, _ = _arnoldi(sides, p, m, _start(kind, int(np.prod(sides)), p))
     assert np.abs(V.T @ V - np.eye((m + 1) * p)).max() <= 2.0 ** -24
+
+
+@pytest.mark.parametrize("sides,p,m", [((90, 80, 70), 2, 10), ((90, 80, 70), 8, 10), ((600, 500), 17, 6), ((40, 41), 32, 16),
+                                       ((33, 31), 17, 30)])
+def test_solution_columns_beside_localised_ones(sides, p, m):
+    """Half of B's columns are unit vectors, half spread out, each of norm one; four cycles of Algorithm 1 converge
+    far past FP64.  Against the FP64 plan, column by column: the coefficients of the solution update keep 2^-55
+    of their largest scaled entry on n <= 2^19 rows and (m + 1) p columns (2^-43), and the partial fractions
+    amplify the relation's 2^-48 by less than 2^6.  The last two shapes pass the width up to which the update's digits
+    fit in shared memory."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    n, d = int(np.prod(sides)), len(sides)
+    B = inputs.rhs(n, p, 4)
+    B[:, p // 2:] = 0.0
+    B[np.linspace(n // 3, n // 2, p - p // 2).astype(int), np.arange(p // 2, p)] = 1.0
+    B /= np.linalg.norm(B, axis=0)
+    t = 20.0 / sum((N + 1) ** 2 for N in sides)
+    Z = []
+    for precision in ("mixed", "fp64"):
+        plan = Plan(sides, 0.1, (1.0, 1.0, 0.5)[:d], p_max=p, m=m, fixed_cycles=4, algorithm=1, precision=precision)
+        Z.append(to_np(plan.expm_block(t, to_dev(B))[0]))
+        plan.close()
+    assert np.all(np.linalg.norm(Z[0] - Z[1], axis=0) <= 2.0 ** -41 * np.linalg.norm(Z[1], axis=0))
