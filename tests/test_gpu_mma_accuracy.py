@@ -51,13 +51,13 @@ def test_orthogonality(sides, p, m, kind):
     assert np.abs(V.T @ V - np.eye((m + 1) * p)).max() <= 2.0 ** -24
 
 
-@pytest.mark.parametrize("sides,p,m", [((90, 80, 70), 2, 10), ((90, 80, 70), 8, 10), ((600, 500), 17, 6), ((40, 41), 32, 16),
-                                       ((33, 31), 17, 30)])
+@pytest.mark.parametrize("sides,p,m", [((90, 80, 70), 2, 10), ((90, 80, 70), 8, 10), ((600, 500), 17, 6), ((40, 41), 32, 12),
+                                       ((33, 31), 17, 30), ((40, 41), 24, 19)])
 def test_solution_columns_beside_localised_ones(sides, p, m):
     """Half of B's columns are unit vectors, half spread out, each of norm one; four cycles of Algorithm 1 converge
     far past FP64.  Against the FP64 plan, column by column: the coefficients of the solution update keep 2^-55
     of their largest scaled entry on n <= 2^19 rows and (m + 1) p columns (2^-43), and the partial fractions
-    amplify the relation's 2^-48 by less than 2^6.  The last two shapes pass the width up to which the update's digits
+    amplify the relation's 2^-48 by less than 2^6.  The last three shapes lie at and beyond the width up to which the digits
     fit in shared memory."""
     need_gpu()
     from paper_1405_0707_gb300 import Plan
