@@ -1,0 +1,29 @@
+"""The FP64 Cholesky-QR's factor against the inverse that is applied (k_chol)."""
+import numpy as np
+import pytest
+
+from paper_1405_0707_gb300 import inputs
+from tests.gpu_util import need_gpu, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("sides,count", [((31, 29), 300), ((401, 251), 40)])
+def test_one_column_factor(sides, count):
+    """p = 1, where R is a number: W = V_0 h + V_1 R up to a scale error of V_1 of at most one rounding for each of
+    the two passes' reciprocals and one for the product of their roots (3 u, u = 2^-53); the roundings of the
+    n entries average out against V_1 (a quarter of u)."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    L = np.longdouble
+    plan = Plan(sides, 0.1, (1.0, -0.5), p_max=1, m=2)
+    worst = 0.0
+    for seed in range(count):
+        v = inputs.rhs(plan.n, 1, seed)
+        V, H = plan.arnoldi(0.05, to_dev(v / np.linalg.norm(v)))
+        W = to_np(plan.prec_apply(0.05, V[:, :1])).astype(L)[:, 0]
+        V, H = to_np(V).astype(L), to_np(H).astype(L)
+        r = W - V[:, 0] * H[0, 0] - V[:, 1] * H[1, 0]
+        worst = max(worst, abs(float(V[:, 1] @ r / H[1, 0])))
+    plan.close()
+    assert worst <= 3.25 * 2.0 ** -53
