@@ -476,7 +476,7 @@ __global__ void k_cd_apply_df(const double* __restrict__ V, int64_t ldv, double*
         sl += yl;
     }
     if (W32) W32[c * ldw + i] = sh + sl;
-    else W[c * ldw + i] = f64_of_f32_i(sh) + f64_of_f32_i(sl);
+    if (W) W[c * ldw + i] = f64_of_f32_i(sh) + f64_of_f32_i(sl);
 }
 
 // ---------------------------------------------------------------- mixed precision

@@ -7,9 +7,12 @@ have to be the same bit for bit.  The row counts leave 1, 8 and 15 rows in the l
 """
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
+from oracle import operators as ops
 from paper_1405_0707_gb300 import inputs
 from tests.gpu_util import need_gpu, to_dev, to_np
+from tests.test_gpu_mma import _times_longdouble
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +92,26 @@ def test_batch_runs_right_after_its_plans_are_made():
         batch.close()
         for plan in plans:
             plan.close()
+
+
+@pytest.mark.parametrize("value,bits", [(None, 49), ("1", 49), ("3", 44)])
+@pytest.mark.parametrize("sides,p", [((61, 59), 3), ((33, 31, 29), 9), ((16, 12, 20), 4)])
+def test_refined_inverse_under_each_stencil_switch(sides, p, value, bits, monkeypatch):
+    """(tA)^{-1} V of mixed plans with the residual's stencil in FP64 (unset, "1") and in float pairs ("3"): backward
+    error within 16 roundings of |tA||x|, or 16 times 2^-48 of it, with a workspace that starts as NaN."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    monkeypatch.setenv("EXPM_FILL_BYTE", "255")
+    if value is None:
+        monkeypatch.delenv("EXPM_STENCIL_FP64", raising=False)
+    else:
+        monkeypatch.setenv("EXPM_STENCIL_FP64", value)
+    n, vel, t = int(np.prod(sides)), (1.0, -0.5, 0.3)[:len(sides)], 0.05
+    V = inputs.rhs(n, p, 79)
+    plan = Plan(sides, 0.1, vel, p_max=p, m=2, precision="mixed")
+    X = to_np(plan.prec_apply(t, to_dev(V)))
+    plan.close()
+    A = sp.csr_matrix(ops.cd_matrix(sides, 0.1, vel, t))
+    R = V.astype(np.longdouble) - _times_longdouble(A, X)
+    scale = abs(A).sum(axis=1).max() * np.abs(X).max(axis=0)
+    assert np.all(np.abs(R).max(axis=0) <= 2.0 ** -bits * scale)
