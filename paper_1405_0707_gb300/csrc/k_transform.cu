@@ -394,9 +394,11 @@ cudaError_t launch_table_frags(const double* Q, int N, uint4* F, cudaStream_t s)
 }
 
 cudaError_t launch_transform(const TransformArgs& g, int batch, int sms, cudaStream_t s, const float* add, int64_t add_b) {
-    if (add && !(g.c_rs == 1 && g.a_cs != 1 && g.c_f64)) return cudaErrorInvalidValue;
+    // strides of one on both sides of A (an axis of one point): either reading is right, rows contiguous is taken
+    const bool in_k = g.a_cs == 1 && g.a_rs != 1;
+    if (add && !(g.c_rs == 1 && !in_k && g.c_f64)) return cudaErrorInvalidValue;
     if (g.c_rs == 1) {
-        if (g.a_cs == 1)
+        if (in_k)
             return g.c_f64 ? launch_var<T_IN_K_OUT_M, double>(g, batch, sms, s) : launch_var<T_IN_K_OUT_M, float>(g, batch, sms, s);
         return g.c_f64 ? launch_var<T_IN_M_OUT_M, double>(g, batch, sms, s, add, add_b) : launch_var<T_IN_M_OUT_M, float>(g, batch, sms, s);
     }
