@@ -434,6 +434,8 @@ typedef enum {
 expm_status expm_plan_profile(expm_plan* plan, int enable);
 expm_status expm_plan_get_profile(expm_plan* plan, double* stage_ms, int64_t* stage_launches,
                                   int nstages, int64_t* total_launches);
+/* Cycle graphs: how many the plan holds (at most 16) and how many it has captured so far. */
+expm_status expm_plan_graph_stats(expm_plan* plan, int32_t* held, int64_t* captures);
 
 /* expm_peak_fma -- measurement support for the roofline denominators (not part of the
  * paper's method): the device's FMA throughput, kind 0 = FP64, 1 = FP32, from one launch of

@@ -36,7 +36,7 @@ EXPORTS = ("expm_cf_coeffs", "expm_plan_create", "expm_plan_destroy", "expm_bloc
            "expm_plan_profile", "expm_plan_get_profile", "expm_status_str",
            "expm_prec_apply_noalloc", "expm_block_batched", "expm_block_adjoint", "expm_ritz_basis",
            "expm_block_batched_host", "expm_peak_fma", "expm_batch_create", "expm_batch_run",
-           "expm_batch_destroy")
+           "expm_batch_destroy", "expm_plan_graph_stats")
 STAGES = ("gemm", "tridiag", "cgs", "reduce", "qr", "poles", "update", "other", "stencil")
 
 
@@ -132,6 +132,8 @@ def load(build_if_missing: bool = False):
     lib.expm_plan_get_profile.restype = C.c_int
     lib.expm_plan_get_profile.argtypes = [p, C.POINTER(d), C.POINTER(C.c_int64), C.c_int,
                                           C.POINTER(C.c_int64)]
+    lib.expm_plan_graph_stats.restype = C.c_int
+    lib.expm_plan_graph_stats.argtypes = [p, C.POINTER(C.c_int32), C.POINTER(C.c_int64)]
     _lib = lib
     return lib
 
@@ -243,6 +245,13 @@ def expm_plan_get_profile(plan):
     tot = C.c_int64()
     check(load().expm_plan_get_profile(plan, ms, nl, k, C.byref(tot)), "expm_plan_get_profile")
     return {STAGES[i]: (ms[i], nl[i]) for i in range(k)}, tot.value
+
+
+def expm_plan_graph_stats(plan):
+    """(cycle graphs held, captures so far)."""
+    held, captures = C.c_int32(), C.c_int64()
+    check(load().expm_plan_graph_stats(plan, C.byref(held), C.byref(captures)), "expm_plan_graph_stats")
+    return held.value, captures.value
 
 
 def expm_prec_apply_noalloc(op, t, dV, ldv, p, dW, ldw, stream=0):

@@ -621,36 +621,45 @@ expm_status issue_cycle(expm_plan* P, double t, int p, int alg, int kk = 0, int 
     return EXPM_OK;
 }
 
-// Capture (once) and return the graph of one cycle for (alg, p, t); nullptr if capture is
-// not possible, in which case the caller launches directly.
+// The graph of one cycle for (alg, p, t, restart kind), captured when there is none yet; nullptr when the
+// caller launches directly: capture is not possible, or the key's first use on the legacy default stream (that
+// stream cannot capture: the cycle is captured on a stream of the plan's own and the graph launched into the
+// default stream; a solve of one cycle, as on small or stiff problems, does not pay for a capture it uses
+// once), or its first use when the table is full.  A key whose capture failed is tried again every
+// kMaxGraphs uses.
+constexpr int kMaxGraphs = 16;
+
 GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int prologue = 0) {
-    // the legacy default stream cannot capture: the cycle is captured on a stream of the plan's own and
-    // the graph launched into the default stream.  A cycle is launched directly the first time there
-    // (a solve of one cycle, as on small or stiff problems, does not pay for a capture it uses once)
-    const bool legacy = P->stream == nullptr;
-    GraphEntry* seen = nullptr;
+    GraphEntry e;
+    e.alg = alg;
+    e.p = p;
+    e.t = t;
+    e.kk = kk;
+    e.prologue = prologue;
+    auto same = [&](const GraphEntry& g) {
+        return g.alg == alg && g.p == p && g.t == t && g.kk == kk && g.prologue == prologue;
+    };
     for (auto& g : P->graphs)
-        if (g.alg == alg && g.p == p && g.t == t && g.kk == kk && g.prologue == prologue) {
-            if (g.exec) return &g;
-            seen = &g;
+        if (same(g)) {
+            g.used = ++P->graph_clock;
+            return &g;
         }
-    if (!seen) {
-        if (P->graphs.size() >= 16) return nullptr;
-        if (legacy) {
-            GraphEntry e;
-            e.alg = alg;
-            e.p = p;
-            e.t = t;
-            e.kk = kk;
-            e.prologue = prologue;
-            P->graphs.push_back(e);
-            return nullptr;
+    const bool legacy = P->stream == nullptr;
+    auto seen = std::find_if(P->seen.begin(), P->seen.end(), same);
+    auto note = [&](int wait) {
+        if (seen == P->seen.end()) {
+            if (P->seen.size() >= kMaxGraphs) P->seen.erase(P->seen.begin());
+            seen = P->seen.insert(P->seen.end(), e);
         }
-    }
+        seen->wait = wait;
+        return static_cast<GraphEntry*>(nullptr);
+    };
+    if (seen == P->seen.end() && (legacy || P->graphs.size() >= kMaxGraphs)) return note(0);
+    if (seen != P->seen.end() && seen->wait > 0) return note(seen->wait - 1);
     if (legacy && !P->cap && cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         P->cap = nullptr;
-        return nullptr;
+        return note(kMaxGraphs);
     }
     cudaStream_t s = legacy ? P->cap : P->stream;
     const int64_t l0 = P->launches;
@@ -658,7 +667,7 @@ GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int pr
     for (int k = 0; k < EXPM_NSTAGES; ++k) sl0[k] = P->stage_launches[k];
     if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return note(kMaxGraphs);
     }
     const cudaStream_t own = P->stream;
     P->stream = s;
@@ -666,12 +675,6 @@ GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int pr
     P->stream = own;
     cudaGraph_t graph = nullptr;
     cudaError_t ec = cudaStreamEndCapture(s, &graph);
-    GraphEntry e;
-    e.alg = alg;
-    e.p = p;
-    e.t = t;
-    e.kk = kk;
-    e.prologue = prologue;
     e.launches = P->launches - l0;
     for (int k = 0; k < EXPM_NSTAGES; ++k) {
         e.stage_launches[k] = P->stage_launches[k] - sl0[k];
@@ -681,17 +684,35 @@ GraphEntry* graph_for(expm_plan* P, double t, int p, int alg, int kk = 0, int pr
     if (st != EXPM_OK || ec != cudaSuccess || !graph) {
         if (graph) cudaGraphDestroy(graph);
         cudaGetLastError();
-        return nullptr;
+        return note(kMaxGraphs);
     }
-    cudaError_t ei = cudaGraphInstantiate(&e.exec, graph, 0);
+    // a full table gives up the graph used longest ago (none is in flight here: a cycle is issued after the
+    // last one's stop test).  A cycle that differs in t alone takes over its executable form, updated: taking
+    // one down and instantiating another cost about 1 ms more
+    GraphEntry* old = nullptr;
+    if (P->graphs.size() >= kMaxGraphs)
+        old = &*std::min_element(P->graphs.begin(), P->graphs.end(),
+                                 [](const GraphEntry& a, const GraphEntry& b) { return a.used < b.used; });
+    if (old && old->alg == alg && old->p == p && old->kk == kk && old->prologue == prologue) {
+        cudaGraphExecUpdateResultInfo info;
+        if (cudaGraphExecUpdate(old->exec, graph, &info) == cudaSuccess) e.exec = old->exec;
+        else cudaGetLastError();
+    }
+    if (!e.exec) {
+        if (cudaGraphInstantiate(&e.exec, graph, 0) != cudaSuccess) {
+            cudaGetLastError();
+            cudaGraphDestroy(graph);
+            return note(kMaxGraphs);
+        }
+        if (old) cudaGraphExecDestroy(old->exec);
+    }
     cudaGraphDestroy(graph);
-    if (ei != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (seen) {
-        *seen = e;
-        return seen;
+    ++P->captures;
+    e.used = ++P->graph_clock;
+    if (seen != P->seen.end()) P->seen.erase(seen);
+    if (old) {
+        *old = e;
+        return old;
     }
     P->graphs.push_back(e);
     return &P->graphs.back();
@@ -936,8 +957,7 @@ void free_plan(expm_plan* P) {
     if (P->cycle_ev) cudaEventDestroy(P->cycle_ev);
     if (P->adj) free_plan(P->adj);
     for (auto& e : P->ev) cudaEventDestroy(e);
-    for (auto& g : P->graphs)
-        if (g.exec) cudaGraphExecDestroy(g.exec);
+    for (auto& g : P->graphs) cudaGraphExecDestroy(g.exec);
     if (P->cap) cudaStreamDestroy(P->cap);
     delete P;
 }
@@ -2100,6 +2120,13 @@ expm_status expm_plan_profile(expm_plan* plan, int enable) {
         }
     }
     plan->prof = enable != 0;
+    return EXPM_OK;
+}
+
+expm_status expm_plan_graph_stats(expm_plan* plan, int32_t* held, int64_t* captures) {
+    if (!plan) return EXPM_INVALID_ARG;
+    if (held) *held = (int32_t)plan->graphs.size();
+    if (captures) *captures = plan->captures;
     return EXPM_OK;
 }
 

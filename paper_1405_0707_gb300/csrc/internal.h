@@ -148,7 +148,9 @@ struct GraphEntry {
     int alg = 0, p = 0;
     double t = 0.0;
     int kk = 0, prologue = 0;   // deflated restart: kept Ritz vectors, kind of restart prologue
-    cudaGraphExec_t exec = nullptr;   // null: seen once, not captured yet
+    cudaGraphExec_t exec = nullptr;   // null in expm_plan_s::seen: launched directly so far
+    int wait = 0;               // seen: uses left before the next try, after a capture that failed
+    int64_t used = 0;           // graphs: time of the last use
     int64_t launches = 0;
     int64_t stage_launches[EXPM_NSTAGES] = {};
 };
@@ -250,7 +252,9 @@ struct expm_plan_s {
     double* hH = nullptr;      // pinned: H~ after each cycle (ldH x m p_max)
     double* hPk = nullptr;     // pinned: staging of Pkd
     double* hHnew = nullptr;   // pinned: the leading (kk + p) x kk block of H~ after the restart
-    std::vector<GraphEntry> graphs;
+    std::vector<GraphEntry> graphs;   // captured cycles, at most kMaxGraphs: the least recently used one goes
+    std::vector<GraphEntry> seen;     // keys launched directly so far, at most kMaxGraphs: the oldest goes
+    int64_t graph_clock = 0, captures = 0;
     cudaStream_t cap = nullptr;   // capture stream of plans on the legacy default stream (which cannot capture)
 };
 

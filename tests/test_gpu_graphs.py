@@ -44,3 +44,33 @@ def test_default_stream_graphs_repeat_the_direct_launches(kind, precision, algor
         assert np.array_equal(Z, out[0])
     assert np.array_equal(other[0], other[1])
     assert np.all(np.isfinite(out[0]))
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_more_times_than_graphs_are_kept(own_stream):
+    """A plan keeps the 16 graphs used last.  20 times, one solve of several cycles each: 16 graphs at the end, and a
+    time that repeats has or gets one, whatever came before; results repeat bit for bit."""
+    torch = need_gpu()
+    from paper_1405_0707_gb300 import Plan, _native as N
+    B = to_dev(inputs.rhs(33 * 21, 3, 17))
+    stream = torch.cuda.Stream() if own_stream else None
+    torch.cuda.synchronize()
+    plan = Plan((33, 21), 0.1, (1.0, -0.5), p_max=3, m=4, tol=1e-9, max_cycles=60, precision="mixed", stream=stream)
+    times = [0.05 * 1.01 ** k for k in range(20)]
+
+    def solve(t):
+        Z, info = plan.expm_block(t, B)
+        assert info.cycles >= 3
+        return to_np(Z)
+
+    first = [solve(t) for t in times]
+    held, captures = N.expm_plan_graph_stats(plan._h)
+    assert (held, captures) == (16, 20)
+    assert np.array_equal(solve(times[-1]), first[-1])
+    assert N.expm_plan_graph_stats(plan._h) == (16, 20)          # kept
+    assert np.array_equal(solve(times[0]), first[0])
+    assert N.expm_plan_graph_stats(plan._h) == (16, 21)          # had gone, captured again
+    assert np.array_equal(solve(times[0]), first[0])
+    assert np.array_equal(solve(times[-1]), first[-1])
+    assert N.expm_plan_graph_stats(plan._h) == (16, 21)
+    plan.close()
