@@ -43,3 +43,26 @@ def test_solve(sides):
     ref = ops.exact_r_of_A_B(sides, 1.0, vel, t, cf.load_table(), B)
     assert rel(to_np(Z), ref) <= 1e-9 * np.linalg.norm(B) / np.linalg.norm(ref)
     plan.close()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("sides,p", [((61, 59), 3), ((32, 24), 8), ((13, 12, 11), 5), ((16, 12, 20), 4)])
+def test_unaligned_columns(sides, p, precision):
+    """Columns that start 8 bytes past a 16-byte boundary, an odd number of rows apart: the same values, bit for
+    bit, as with packed columns."""
+    torch = need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    n, vel, t = int(np.prod(sides)), (0.5, -0.3, 0.2)[:len(sides)], 0.01
+
+    def odd():
+        return torch.zeros((p, n + 3 + n % 2), dtype=torch.float64, device="cuda")[:, 1:n + 1].T
+
+    B, X, Z, Xo, Zo = to_dev(inputs.rhs(n, p, 3)), None, None, odd(), odd()
+    Bo = odd()
+    Bo.copy_(B)
+    plan = Plan(sides, 1.0, vel, p_max=p, m=6, fixed_cycles=2, precision=precision, algorithm=2)
+    X, (Z, _) = plan.prec_apply(t, B), plan.expm_block(t, B)
+    plan.prec_apply(t, Bo, Xo)
+    plan.expm_block(t, Bo, Zo)
+    assert np.array_equal(to_np(Xo), to_np(X)) and np.array_equal(to_np(Zo), to_np(Z))
+    plan.close()
