@@ -301,17 +301,17 @@ __device__ __forceinline__ double scaled_int(long long X, int k) {
     return __longlong_as_double((long long)(b | (X < 0 ? 1ull << 63 : 0ull)));
 }
 
-// L_0 + L_1 2^-8 + .. + L_7 2^-56 = x + y, the level sums exact integers below 2^24: three groups summed
+// L_0 + L_1 2^-8 + .. + L_8 2^-64 = x + y, the level sums exact integers below 2^24: three groups summed
 // exactly in float pairs (40 bits each), joined in FP64
 __device__ __forceinline__ void level_sum64(float l0, float l1, float l2, float l3, float l4, float l5, float l6, float l7,
-                                            double& x, double& y) {
+                                            double& x, double& y, float l8 = 0.f) {
     float ah = l2 * 0x1p-16f, al = 0.f;
     df_add(ah, al, l1 * 0x1p-8f);
     df_add(ah, al, l0);
     float bh = l5 * 0x1p-40f, bl = 0.f;
     df_add(bh, bl, l4 * 0x1p-32f);
     df_add(bh, bl, l3 * 0x1p-24f);
-    const float lo = bl + fmaf(l7, 0x1p-56f, l6 * 0x1p-48f);
+    const float lo = bl + fmaf(l8, 0x1p-64f, fmaf(l7, 0x1p-56f, l6 * 0x1p-48f));
     x = f64_of_f32_i(ah);
     y = (f64_of_f32_i(lo) + f64_of_f32_i(bh)) + f64_of_f32_i(al);
 }
@@ -695,8 +695,11 @@ k_upd_mma(const UpdArgs A) {
 // ---------------------------------------------------------------- projection to FP64 rounding
 // FP64 plans: partial[bx][a][c] = sum over the rows of row group bx of V[r, a] W[r, c], both operands in
 // eight digits of their column's scale (2^-62 of its largest entry), the 36 digit products of levels 0..7
-// summed exactly over 128 rows and joined in FP64: 3 FP64 adds per output and 128 rows where the FP64
-// kernel spends 128 FMAs on a pipe that retires two per SM and clock.  MMA: M = 16 basis columns, N = 8
+// summed exactly over 128 rows and joined in FP64: 4 FP64 adds per output and 128 rows where the FP64
+// kernel spends 128 FMAs on a pipe that retires two per SM and clock.  The products left out have random
+// signs but for the squares on a Gram matrix's diagonal, of which the largest, digit 4 by digit 4, is a
+// 37th product: without it a localised column's norm came out short by n 2^-64 of its largest entry
+// squared (300 x 300, unit vectors: |v|^2 - 1 = 6.8e-15, with it 4e-16).  MMA: M = 16 basis columns, N = 8
 // block columns, K = 16 rows, lanes and units as in k_proj_mma; a warp owns one M tile.
 constexpr size_t proj64_smem(int NT) { return (size_t)2 * kProjKb * NT * 8 * 32 * sizeof(uint2); }
 
@@ -767,7 +770,7 @@ k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restr
         v[1][0] = *reinterpret_cast<const double2*>(V + (int64_t)a1 * ldv + r);
         v[1][1] = *reinterpret_cast<const double2*>(V + (int64_t)a1 * ldv + r + 2);
     };
-    float acc[8][NT][4];
+    float acc[9][NT][4];
     double sum[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j)
@@ -775,7 +778,7 @@ k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restr
         for (int q = 0; q < 4; ++q) {
             sum[j][q] = 0.0;
 #pragma unroll
-            for (int l = 0; l < 8; ++l) acc[l][j][q] = 0.f;
+            for (int l = 0; l < 9; ++l) acc[l][j][q] = 0.f;
         }
     int64_t u = blockIdx.x;
     int buf = 0, since = 0;
@@ -817,7 +820,7 @@ k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restr
                     a[2] = digit_pair<8, I>(yl[0][2], yh[0][2], yl[0][3], yh[0][3]);
                     a[3] = digit_pair<8, I>(yl[1][2], yh[1][2], yl[1][3], yh[1][3]);
 #pragma unroll
-                    for (int k = 0; k + I < 8; ++k)
+                    for (int k = 0; k + I < 8 + (I == 4); ++k)
 #pragma unroll
                         for (int j = 0; j < NT; ++j) mma_f16(acc[I + k][j], a, wb[j][k].x, wb[j][k].y);
                 };
@@ -837,10 +840,10 @@ k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restr
                         for (int q = 0; q < 4; ++q) {
                             double x, y;
                             level_sum64(acc[0][j][q], acc[1][j][q], acc[2][j][q], acc[3][j][q], acc[4][j][q], acc[5][j][q],
-                                        acc[6][j][q], acc[7][j][q], x, y);
+                                        acc[6][j][q], acc[7][j][q], x, y, acc[8][j][q]);
                             sum[j][q] += x + y;
 #pragma unroll
-                            for (int l = 0; l < 8; ++l) acc[l][j][q] = 0.f;
+                            for (int l = 0; l < 9; ++l) acc[l][j][q] = 0.f;
                         }
                 }
             }
@@ -855,7 +858,7 @@ k_proj64(const double* __restrict__ V, int64_t ldv, int cols, const int* __restr
         for (int q = 0; q < 4; ++q) {
             double x, y;
             level_sum64(acc[0][j][q], acc[1][j][q], acc[2][j][q], acc[3][j][q], acc[4][j][q], acc[5][j][q], acc[6][j][q],
-                        acc[7][j][q], x, y);
+                        acc[7][j][q], x, y, acc[8][j][q]);
             red[warp][lane][q] = sum[j][q] + (x + y);
         }
         __syncthreads();

@@ -27,3 +27,18 @@ def test_one_column_factor(sides, count):
         worst = max(worst, abs(float(V[:, 1] @ r / H[1, 0])))
     plan.close()
     assert worst <= 3.25 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("sides,p", [((300, 300), 4), ((300, 300), 8), ((401, 251), 1), ((1000, 900), 1), ((150, 150), 24)])
+def test_norms_of_localised_columns(sides, p):
+    """Columns of (tA)^{-1} applied to unit vectors: one large entry, all others small.  Their norms come from the
+    digit products' Gram matrix (n p >= 100000), whose partial sums and factor take about ten roundings."""
+    need_gpu()
+    from paper_1405_0707_gb300 import Plan
+    plan = Plan(sides, 0.1, (1.0, -0.5), p_max=p, m=2)
+    assert plan.n * p >= 100000
+    V1 = np.zeros((plan.n, p), order="F")
+    V1[np.linspace(0, plan.n - 1, p).astype(int), np.arange(p)] = 1.0
+    V = to_np(plan.arnoldi(0.05, to_dev(V1))[0]).astype(np.longdouble)
+    plan.close()
+    assert np.max(np.abs((V * V).sum(axis=0) - 1.0)) <= 16 * 2.0 ** -53
