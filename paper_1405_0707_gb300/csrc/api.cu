@@ -80,7 +80,7 @@ void prof_flush(expm_plan* P) {
         prof_end(P, (stage), e_, 1);                 \
     } while (0)
 
-// The mixed path with p <= 8 runs the Cholesky QR with FP32 factorisations fused into the
+// The mixed path with p <= 16 runs the Cholesky QR with FP32 factorisations fused into the
 // triangular solves (k_qr_mixed_rows); everything else uses k_chol + k_trsm.
 inline bool fused_qr(const expm_plan* P, int p) {
     return p <= kRowsMaxP && P->opts.precision == EXPM_PREC_MIXED;
@@ -408,8 +408,9 @@ inline bool use64(const expm_plan* P, int p) { return P->mma64 && P->n * p >= kU
 
 // The FP64 path's Gram-Schmidt and Cholesky-QR of block step j by exact digit products (k_mma.cu): the
 // column scales of W, projection and update twice, then two Cholesky-QR passes (a third one when the first
-// asks for it), every tall product on the tensor cores and every result rounded once to FP64.  wexp holds
-// two sets of five p-column exponent arrays; a step uses one and clears the other.
+// asks for it), every tall product on the tensor cores.  A product enters its FP64 result as a sum of two
+// doubles, so an entry of an update takes three roundings for each 128 columns.  wexp holds two sets of
+// five p-column exponent arrays; a step uses one and clears the other.
 expm_status ortho64(expm_plan* P, int j, int p) {
     cudaStream_t s = P->stream;
     const int64_t n = P->n, ld = P->ld;
@@ -1430,19 +1431,20 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         // block (the fallback of the single accurate pass)
         const char* sq = std::getenv("EXPM_QR_SINGLE_PASS");
         P->qr_single = !(sq && sq[0] == '0');
-        // the first CGS pass's update on the tensor cores (k_cgs_tc, then the projection kernel
-        // for the second pass and the Gram matrix) for mixed plans: by default for block
+        // Mixed plans run the register-streamed passes (k_mma.cu).  What follows steers those that do not:
+        // plans without room for the basis's FP32 copy, and plans that a test switch keeps on these kernels.
+        // The first CGS pass's update on the tensor cores (k_cgs_tc, then the projection kernel
+        // for the second pass and the Gram matrix): by default for block
         // steps with p >= 12 and at least 64 basis columns, where it measured faster than the
         // double-float pass (whose cost grows with p, the tensor-core pass's with the basis
         // alone).  Test switch: "1" for every block step it fits, "0" never
         const char* tc = std::getenv("EXPM_CGS_TC");
         P->cgs_tc = opts->precision != EXPM_PREC_MIXED ? 0 : !tc ? 2 : tc[0] == '1' ? 1 : 0;
-        // the first CGS pass's projection on the tensor cores (k_proj_tc) for mixed plans, by
-        // shape (see block_step).  Test switch: "1" for every block step it fits, "0" never
+        // the first CGS pass's projection on the tensor cores (k_proj_tc), by shape (see
+        // block_step).  Test switch: "1" for every block step it fits, "0" never
         const char* ptc = std::getenv("EXPM_PROJ_TC");
         P->proj_tc = opts->precision != EXPM_PREC_MIXED ? 0 : !ptc ? 2 : ptc[0] == '1' ? 1 : 0;
-        // mixed plans run the register-streamed passes (k_mma.cu); either switch above keeps a plan
-        // on the kernels it names
+        // either switch above keeps a plan on the kernels it names
         P->mma64 = opts->precision == EXPM_PREC_FP64 && mma64_fit(opts->m * p_max, p_max);
         P->mma = opts->precision == EXPM_PREC_MIXED && !tc && !ptc && mma_fit(opts->m * p_max, p_max);
         // test switch: the bound of the tensor-core kernel's waits (0 makes every wait run out)
@@ -1670,35 +1672,33 @@ expm_status expm_plan_create(const expm_op_desc* op, int p_max, const expm_opts*
         }
         cuda_ok = cudaMemcpyAsync(P->small + kOffTau, taus, sizeof(taus), cudaMemcpyHostToDevice, s) == cudaSuccess;
     }
-    if (cuda_ok) cuda_ok = cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess;
-    if (!cuda_ok) {
-        free_plan(P);
-        return EXPM_CUDA_ERROR;
-    }
-    if (toeplitz) {
-        const expm_status ts = toeplitz_setup(P, op, opts->algorithm != EXPM_ALG_SBFOM);
+    if (toeplitz && cuda_ok) {
+        cuda_ok = cudaStreamSynchronize(s) == cudaSuccess;
+        const expm_status ts = cuda_ok ? toeplitz_setup(P, op, opts->algorithm != EXPM_ALG_SBFOM) : EXPM_CUDA_ERROR;
         if (ts != EXPM_OK) {
             cudaGetLastError();
             free_plan(P);
             return ts;
         }
     }
-    if (P->mma) {
-        // last, the FP32 copy of the basis (half the basis again), its padding rows zero: a plan that has no
-        // room for it runs on the kernels that read the FP64 basis alone
+    if (P->mma && cuda_ok) {
+        // the last buffer, the FP32 copy of the basis (half the basis again), its padding rows zero: a plan that
+        // has no room for it runs on the kernels that read the FP64 basis alone
         const size_t cols = (size_t)(m + 1) * p_max;
         if (!dalloc(&P->V32, (size_t)ld * cols)) {
             cudaGetLastError();
             P->V32 = nullptr;
             P->mma = false;
-        } else if ((ld > n && cudaMemset2DAsync(P->V32 + n, sizeof(float) * ld, 0, sizeof(float) * (ld - n), cols, s) != cudaSuccess) ||
-                   cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, s) != cudaSuccess ||
-                   // a batch graph runs on a stream of its own, which nothing orders after this one
-                   cudaStreamSynchronize(s) != cudaSuccess) {
-            cudaGetLastError();
-            free_plan(P);
-            return EXPM_CUDA_ERROR;
+        } else {
+            cuda_ok = (ld == n || cudaMemset2DAsync(P->V32 + n, sizeof(float) * ld, 0, sizeof(float) * (ld - n), cols, s) == cudaSuccess) &&
+                      cudaMemsetAsync(P->colexp, 0, sizeof(int) * (size_t)(m + 2) * p_max, s) == cudaSuccess;
         }
+    }
+    // nothing is left pending: a batch graph runs on a stream of its own, which nothing orders after this one
+    if (cuda_ok) cuda_ok = cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+    if (!cuda_ok) {
+        free_plan(P);
+        return EXPM_CUDA_ERROR;
     }
     *out = P;
     return EXPM_OK;
