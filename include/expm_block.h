@@ -155,8 +155,13 @@ typedef struct {
                               block width p and conjugate pairs are kept together (see
                               expm_ritz_basis); 0 = plain restart.  Requires
                               k_defl <= (m - 1) p_max.                                 */
-    int32_t row_ctas_per_sm;  /* launch shape of the row-parallel passes (Cholesky-QR, Z
-                                 update, reductions): CTAs per SM, 1..8; 0 = 2          */
+    int32_t row_ctas_per_sm;  /* launch shape of the CUDA-core row passes (Gram-Schmidt,
+                                 Cholesky-QR, Z update): CTAs per SM, 1..8; 0 = 2.  The
+                                 tensor-core passes, which serve all mixed plans with room
+                                 for an FP32 copy of the basis and FP64 blocks of at least
+                                 100000 entries, choose their own grids; there these two
+                                 options only cap the number of partial sums of the
+                                 projections.                                          */
     int32_t cgs_ctas_per_sm;  /* ... of the first Gram-Schmidt pass: 1..8; 0 = twice
                                  row_ctas_per_sm.  Both are what the autotuner of the
                                  Python package chooses per problem class.             */
@@ -164,15 +169,13 @@ typedef struct {
                               solve of A y = v, per column; 0 = 1e-12                  */
     int32_t inner_maxit;   /* ... and its iteration cap per application; 0 = 2000      */
     int32_t grid_sms;      /* SMs that the grids of the row-parallel passes after the
-                              first Gram-Schmidt pass (Cholesky-QR, Z update, reductions)
-                              are sized for: CTAs = row_ctas_per_sm x grid_sms; 0 = all of
-                              the device's.  The first Gram-Schmidt pass always spans the
-                              device.  Plans whose solves run at the same time
-                              (expm_block_batched, expm_batch_*) can each take a share:
-                              those passes are latency-bound (a serial p x p
-                              factorisation in every CTA), and fewer CTAs with more rows
-                              each leave SMs to the other instances' kernels.  Results do
-                              not depend on it beyond the order of the row partial sums. */
+                              Gram-Schmidt projections and updates (Cholesky-QR, Z update)
+                              are sized for; 0 = all of the device's.  The Gram-Schmidt
+                              passes always span the device.  Plans whose solves run at
+                              the same time (expm_block_batched, expm_batch_*) can each
+                              take a share: fewer CTAs with more rows each leave SMs to
+                              the other instances' kernels.  Results do not depend on it
+                              beyond the order of the row partial sums.                 */
 } expm_opts;
 
 #define EXPM_MAX_POLES 16

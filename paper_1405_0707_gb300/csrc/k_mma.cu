@@ -33,8 +33,8 @@
 //    solution error 2.3e-14, now 1.5e-14).
 //
 // Measured, 96^3, p = 16, per block step averaged over a 10-step cycle: Gram-Schmidt 1.09 -> 0.66 ms
-// (projection 62 us at 16 and 243 us at 160 columns, 2.8 TB/s, bound by the loads in flight; update 218 and
-// 516 us, 2.6 TB/s, bound by issue slots at 12 to 16 warps per SM), 512 x 352, p = 32: 3.3 -> 0.6 ms.
+// (projection 66 us at 16 and 237 us at 160 columns, 2.9 TB/s, bound by the loads in flight; update 197 and
+// 491 us, 2.8 TB/s, bound by issue slots at 12 to 16 warps per SM), 512 x 352, p = 32: 3.3 -> 0.6 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>

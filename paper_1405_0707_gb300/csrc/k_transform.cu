@@ -16,7 +16,7 @@
 // lane group g holds rows 4g .. 4g + 3), which any MMA allows as long as both operands agree.  Q is
 // split once when the plan is made and stored in fragment order; a CTA keeps the slab of its 32 or 48
 // columns in shared memory and its warps walk over 32-row tiles.  96^3, p = 16, all 12 transforms of a
-// block step: 1.50 -> 0.95 ms (61 to 72 us each, 100 us into FP64; 8 bytes a value at 3.7 TB/s), bound now by
+// block step: 1.50 -> 0.92 ms (61 to 72 us each, 110 to 157 us into FP64; 8 bytes a value at 3.7 TB/s), bound now by
 // dependent issue at 8 to 12 warps per SM and 48 % of the mma.sync rate.
 //
 //   IN_M  (rows contiguous in A)        OUT_M (rows contiguous in C): Q is the left operand (M = n)
