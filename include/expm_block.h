@@ -158,9 +158,10 @@ typedef struct {
     int32_t row_ctas_per_sm;  /* launch shape of the CUDA-core row passes (Gram-Schmidt,
                                  Cholesky-QR, Z update): CTAs per SM, 1..8; 0 = 2.  The
                                  tensor-core passes, which serve all mixed plans with room
-                                 for an FP32 copy of the basis and FP64 blocks of at least
-                                 100000 entries, choose their own grids; there these two
-                                 options only cap the number of partial sums of the
+                                 for an FP32 copy of the basis and large FP64 blocks (at
+                                 least 100000 entries and five columns, or more entries
+                                 and three or four), choose their own grids; there these
+                                 two options only cap the number of partial sums of the
                                  projections.                                          */
     int32_t cgs_ctas_per_sm;  /* ... of the first Gram-Schmidt pass: 1..8; 0 = twice
                                  row_ctas_per_sm.  Both are what the autotuner of the

@@ -4,7 +4,7 @@ library's kernels).
 The CUDA-core row passes of a restart cycle (Gram-Schmidt, Cholesky-QR, Z update) are launched
 with a number of CTAs per SM that trades latency hiding against the size of the partial-sum
 reductions; the best value depends on the problem's order n and block width p.  Plans that run the
-tensor-core passes (mixed precision, FP64 blocks of at least 100000 entries) choose their own
+tensor-core passes (mixed precision, large FP64 blocks of three or more columns) choose their own
 grids, and the shapes only cap the projections' partial sums there.  For each problem class the tuner times one restart cycle
 (opts.fixed_cycles = 1, CUDA events on the plan's stream, the median of a few repetitions) for
 every candidate (row_ctas_per_sm, cgs_ctas_per_sm) and keeps the fastest.  The table is a JSON

@@ -400,11 +400,14 @@ expm_status ortho_mma(expm_plan* P, int j, int p) {
     return EXPM_OK;
 }
 
-// FP64 plans take the digit passes on blocks of at least kUse64 entries: they need more launches, and on
-// small blocks the FP64 pipe is not the bound (99 x 99, p = 3, 29403 entries: 4.2 ms with the FP64 kernels,
-// 4.4 with the digit passes; n = 50021, p = 5: 7.0 against 6.4; 256 x 256, p = 8: 54.4 against 34.7).
-constexpr int64_t kUse64 = 100000;
-inline bool use64(const expm_plan* P, int p) { return P->mma64 && P->n * p >= kUse64; }
+// FP64 plans take the digit passes where they are the faster form.  Their cost does not depend on the width up to
+// eight columns, that of the FP64 kernels grows with it, and they need more launches: one or two columns never
+// gain (Algorithm 1, two cycles, FP64 kernels against digits: 320 x 320 p = 1 2.41 / 4.24 ms, 1000 x 900 p = 2 13.97 /
+// 14.74, 128^3 p = 2 31.9 / 31.7), three from 1.5 million entries on (n = 359400 7.44 / 7.57, n = 809100 15.4 /
+// 14.5), four from half a million (n = 78120 3.39 / 3.50, n = 159600 4.95 / 4.87), five and more from about
+// 100000 (n = 22350 p = 5 2.76 / 2.82, n = 39800 3.57 / 3.32; 256 x 256, p = 8: 8.1 / 4.7).
+constexpr int64_t use64_from(int p) { return p <= 2 ? INT64_MAX : p == 3 ? 1500000 : p == 4 ? 500000 : 100000; }
+inline bool use64(const expm_plan* P, int p) { return P->mma64 && P->n * p >= use64_from(p); }
 
 // The FP64 path's Gram-Schmidt and Cholesky-QR of block step j by exact digit products (k_mma.cu): the
 // column scales of W, projection and update twice, then two Cholesky-QR passes (a third one when the first
